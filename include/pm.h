@@ -120,16 +120,18 @@ typedef struct pm_solve_opts {
   int32_t x0_is_guess;   /* 1: x holds the initial guess; 0: start from x = 0               */
   int32_t max_restarts;  /* true-residual restarts after the recursive test passes (FP64)   */
   double inner_rtol;     /* mixed precision: relative reduction asked of each inner solve  */
-  int32_t kernel;        /* FP64 solves: PM_KERNEL_AUTO (resident for n <= 16384 rows),
-                            PM_KERNEL_STREAM (one launch per PCG phase, every SM), or
-                            PM_KERNEL_RESIDENT (one block runs the whole solve, n <= 2^20)   */
+  int32_t kernel;        /* FP64 solves: PM_KERNEL_AUTO (resident up to about 3M rows),
+                            PM_KERNEL_STREAM (one launch per PCG phase), or
+                            PM_KERNEL_RESIDENT (one launch runs the whole solve, n <= 2^20).
+                            Mixed-precision solves run as AUTO                              */
   int32_t pad;
 } pm_solve_opts;
 
-/* How an FP64 solve runs on the GPU (no paper counterpart; the iterates are those of the Section 5
- * PCG either way). STREAM issues one kernel per phase of every PCG iteration over the whole GPU;
- * RESIDENT runs the whole solve in one block of one SM, with block barriers between phases and one
- * read-back at the end: for small systems, whose stream iterations are bound by launch latency. */
+/* How a solve runs on the GPU (no paper counterpart; the iterates are those of the Section 5 PCG
+ * either way). STREAM issues one kernel per phase of every PCG iteration over the whole GPU;
+ * RESIDENT runs the whole solve in one cooperative launch of one block per SM (one cluster of 16 blocks for the
+ * smallest systems), with a bounded grid barrier between phases (an expired wait returns PM_TIMEOUT) and one
+ * wait on the host: for systems whose stream iterations are bound by launches. */
 enum { PM_KERNEL_AUTO = 0, PM_KERNEL_STREAM = 1, PM_KERNEL_RESIDENT = 2 };
 
 typedef struct pm_solve_stats {

@@ -14,7 +14,8 @@ LIB = os.path.join(OUT_DIR, "libpm_gb300.so")
 # The checked build (device index checks, PM_CHECKED): a separate library for debugging and tests.
 OUT_DIR_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(OUT_DIR_CHECKED, "libpm_gb300_checked.so")
-SOURCES = ["pm_api.cu", "pm_mesh.cu", "pm_assemble.cu", "pm_solve.cu", "pm_step.cu", "pm_noalloc.cu",
+SOURCES = ["pm_api.cu", "pm_mesh.cu", "pm_assemble.cu", "pm_solve.cu", "pm_resident.cu", "pm_resident_fp32.cu",
+           "pm_resident_bf16.cu", "pm_step.cu", "pm_noalloc.cu",
            "pm_batch.cu", "pm_checkpoint.cu", "pm_trace.cu"]
 # The persistent batched kernel reads data other blocks write during the launch: plain global
 # loads in that file are cached in L2 only (ld.global.cg), never in the non-coherent L1.

@@ -140,6 +140,27 @@ __host__ __device__ inline bool is_dirichlet(uint8_t flag, int k, int nz, int c)
   return k == nz - 1;
 }
 
+// Division of a non-negative 32-bit integer by a divisor known on the host (a basin's levels per
+// column): q = (umulhi(t, mul) + t) >> shift, exact for 0 <= t < 2^31 and 1 <= d < 2^31. Four integer instructions where
+// a division by a run-time value takes about twenty (32 bits) or a hundred (64 bits).
+struct FastDiv {
+  uint32_t mul, shift;
+  int32_t d;
+};
+inline FastDiv fast_div(int32_t d) {
+  FastDiv f{0, 0, d < 1 ? 1 : d};
+  while ((1ull << f.shift) < (uint64_t)f.d) ++f.shift;
+  f.mul = (uint32_t)((((1ull << f.shift) - (uint64_t)f.d) << 32) / (uint64_t)f.d + 1);
+  return f;
+}
+__host__ __device__ __forceinline__ int fdiv(const FastDiv& f, int t) {
+#ifdef __CUDA_ARCH__
+  return (int)((__umulhi((uint32_t)t, f.mul) + (uint32_t)t) >> f.shift);
+#else
+  return (int)(((uint32_t)(((uint64_t)(uint32_t)t * f.mul) >> 32) + (uint32_t)t) >> f.shift);
+#endif
+}
+
 // ---- compensated residual (Ogita, Rump & Oishi, "Accurate sum and dot product", 2005) --------
 // Error-free transformations in FP64. The _rn intrinsics are never contracted into an FMA, which
 // would change what the transformations compute.
@@ -197,6 +218,7 @@ template <typename T> using AccFor = typename AccSel<T>::type;
 struct Geom {
   int32_t ncols, nz;
   int64_t n, npad;
+  FastDiv nzd;              // division by nz
   double dx, dy;
   const int32_t* nbr;       // [ncols * 7], -1 absent (entry q = 0 is the column itself)
   const double* depth;      // [ncols]
@@ -320,7 +342,10 @@ struct pm_operator {
   uint8_t* d_cellmask = nullptr;
   uint8_t* d_colflag = nullptr;
   double* d_coriolis = nullptr;
-  int32_t* d_cls_cols = nullptr;    // columns grouped by parity class, [ncols]
+  int32_t* d_cls_cols = nullptr;    // columns grouped by parity class, [ncols], then index within the
+                                    // class, i and j of each column, [ncols] each
+  int32_t* d_cnbr = nullptr;        // [7][ncols]: neighbour columns of the i-th column in class order
+                                    // (entry 0: that column itself); part of d_cls_cols' allocation
   uint16_t* d_struct = nullptr;     // structural slot bits per row
   uint16_t* d_keep[3] = {};         // per velocity component: bit s = slot s kept (neighbour present and
                                     // not in the component's Dirichlet set), bit 15 = Dirichlet row

@@ -1,0 +1,971 @@
+// Resident PCG: one launch runs a whole solve (Section 5 remark), its blocks in step.
+//
+// A PCG iteration is a chain of short dependent phases: with IC0, 18 of them. As separate kernels
+// each costs a launch on the host and a drain and ramp on the GPU, 8 to 12 us measured per phase
+// whatever its size, far more than the work of a phase below a few hundred thousand rows. Here a
+// team of blocks keeps the GPU (one block per SM) from the first residual to the last and separates
+// the phases by its own barrier; convergence is tested by every block from the same sums, so no
+// iteration is issued in vain and the host waits once.
+//
+// Two teams run the same code:
+//   - grid: one block per SM (cooperative launch), a counter in L2 as the barrier (bounded wait): 2400
+//     cycles, 3000 with stores to publish;
+//   - cluster: 16 blocks of one thread-block cluster, the hardware cluster barrier (550 to 980 cycles, 2000
+//     with global stores to publish), block sums exchanged through distributed shared memory: for systems so
+//     small that the grid barrier would cost more than the work the other SMs take over.
+//
+// Rows: SpMV, update and preconditioners by column work on whole columns, dealt evenly and
+// contiguously to the blocks; an IC0 colour phase deals the colour's rows (in class order, as the
+// factor is stored) evenly to the blocks. Vectors that other blocks read (p, x, the IC0 work vector)
+// go through L2: a barrier's release / acquire pair orders them, and the acquire drops stale L1 lines,
+// so plain loads may use L1 within a phase.
+//
+// One iteration, phases | team barriers:
+//   w = A p, (p, w)                                                              | sum
+//   r -= alpha w, (r, r); Jacobi / line: z and its dots; IC0: y of colour 0        | sum
+//   IC0: y of colours 1..7 (forward), z of colour 7 with its y, (y, y) = (r, z)        | 6, then sum
+//   x += alpha p, p = z - c + beta p; IC0: with z of colours 6..0 (backward)            | 1 (IC0: 7)
+// (r, z) = (y, y) because z = L^-T y and y = L^-1 r; it is known before the backward sweep, so that
+// sweep can form p at once. The pressure's projection needs m'z first: its IC0 sums and p follow the
+// sweeps as passes of their own.
+//
+// What bounds it: barriers and load latency below about 0.3M rows (IC0 52 us per iteration at 0.12M rows, where the
+// stream of kernels takes 218), the FP64 pipe (64 cycles per warp instruction and sub-core) above.
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "pm_internal.cuh"
+
+namespace pm {
+namespace resident {
+
+// Threads per block, one block per SM: 128 registers a thread hold the 15 values and 15 gathered
+// entries of a row, or the factor row fetched ahead of a barrier, without spills.
+constexpr int NT = 512;
+constexpr int CLUSTER = 16;
+
+struct Ctl {
+  uint32_t arrive;   // barrier arrivals of this launch (zeroed before it)
+  int32_t err;       // set by a wait that ran out
+};
+
+struct Out {
+  int32_t iters, restarts, first_pass, status, zero_rhs, pad;
+  double rel_true, rel_rec, floor;
+};
+
+struct Args {
+  Geom g;
+  const void* val;        // operator values: FP64, or the FP32 / BF16 difference form
+  const double* val64;
+  const uint16_t* mask;   // bit s: slot s counts; bit 15: identity row
+  const double* b;
+  double* x;
+  double* bw;             // projected right-hand side (pressure)
+  void *r, *p, *w, *z;    // Krylov vectors (T)
+  float* d;               // FP32 correction since the last residual (mixed precision)
+  const void* dinv;       // T inverse diagonal; null: plain CG
+  const double* m;        // M 1
+  const float2* m2;       // M 1 as two floats (mixed precision)
+  const void* ic0;        // IC0 factor, colour-ordered rows, 1 / L_ii in the diagonal slot
+  const void* line;       // line factors, level-major
+  const int32_t* cnbr;    // neighbour columns in class order
+  const int32_t* clsidx;  // index of a column within its class
+  const int32_t* coli;
+  const int32_t* colj;
+  int32_t cls_off[4], cls_cnt[4];
+  int32_t cbase[8];
+  FastDiv nlev[2];        // levels of even / odd parity
+  double rtol, inner_rtol, one_m;
+  int32_t max_iter, max_restarts, x0_is_guess, proj, z_in_smem;
+  Ctl* ctl;
+  double* part;           // 2 x 4 x blocks block sums (grid team)
+  Out* out;               // pinned host memory
+};
+
+__device__ __forceinline__ void red_release(uint32_t* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Polls of a grid barrier before it gives up: each takes about a microsecond.
+constexpr uint32_t WAIT_LIMIT = 1u << 22;
+
+// Block-level part of a team sum: FP64 adds run at 1/64 of the FP32 rate on this GPU, so the values
+// go through shared memory and full warps add them (NT / 32 + 12 warp-wide adds per value), where
+// shuffles in every warp would take 5 NT / 32.
+struct Scratch {
+  double v[4][NT];
+  double q[4][128];
+  double res[4];
+  double xch[2][4][CLUSTER];   // cluster team: the blocks' sums
+  int ok;
+};
+
+template <bool CL>
+struct Team {
+  Ctl* ctl;
+  double* part;
+  Scratch* s;
+  int G, rank;
+  uint32_t target;
+  int buf;
+
+  __device__ Team(const Args& a, Scratch* s_)
+      : ctl(a.ctl), part(a.part), s(s_), G(gridDim.x), rank(blockIdx.x), target(0), buf(0) {}
+
+  // This block's stores so far are published; wait() returns when every block has arrived.
+  __device__ __forceinline__ void arrive() {
+    if (CL) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    } else {
+      __syncthreads();
+      if (threadIdx.x == 0) red_release(&ctl->arrive);
+      target += (uint32_t)G;
+    }
+  }
+  __device__ __forceinline__ bool wait() {
+    if (CL) {
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      return true;
+    }
+    if (threadIdx.x == 0) {
+      int ok = 1;
+      uint32_t polls = 0;
+      while ((int32_t)(ld_acquire(&ctl->arrive) - target) < 0) {
+        ++polls;
+        if (polls > WAIT_LIMIT || ((polls & 1023u) == 0 && *(volatile int32_t*)&ctl->err)) {
+          atomicExch(&ctl->err, 1);
+          ok = 0;
+          break;
+        }
+      }
+      s->ok = ok;
+    }
+    __syncthreads();
+    return s->ok != 0;
+  }
+  __device__ __forceinline__ bool barrier() {
+    arrive();
+    return wait();
+  }
+
+  // Team totals of NV values in every thread, added in a fixed order. A barrier as well.
+  template <int NV>
+  __device__ __forceinline__ bool sum(double (&v)[NV]) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    static_assert(NT == 512 && NV <= 4, "four warps per value");
+#pragma unroll
+    for (int i = 0; i < NV; ++i) s->v[i][tid] = v[i];
+    __syncthreads();
+    if (wid < 4 * NV) {
+      const double* c = s->v[wid >> 2] + (wid & 3) * 128 + lane;
+      s->q[wid >> 2][(wid & 3) * 32 + lane] = (c[0] + c[32]) + (c[64] + c[96]);
+    }
+    __syncthreads();
+    if (wid < NV) {
+      const double* c = s->q[wid] + lane;
+      double t = warp_sum((c[0] + c[32]) + (c[64] + c[96]));
+      if (CL) {
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (lane < G) {
+          const uint32_t local = (uint32_t)__cvta_generic_to_shared(&s->xch[buf][wid][rank]);
+          uint32_t remote;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(lane));
+          asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(t) : "memory");
+        }
+        __syncwarp();
+      } else if (lane == 0) {
+        part[(buf * 4 + wid) * G + rank] = t;
+      }
+    }
+    arrive();
+    if (!wait()) return false;
+    if (wid < NV) {
+      double t = 0.0;
+      if (CL) {
+        t = lane < G ? s->xch[buf][wid][lane] : 0.0;
+      } else {
+        for (int j = lane; j < G; j += 32) t += __ldcg(part + (buf * 4 + wid) * G + j);
+      }
+      t = warp_sum(t);
+      if (lane == 0) s->res[wid] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = s->res[i];
+    buf ^= 1;
+    return true;
+  }
+};
+
+__device__ __forceinline__ int cnbr_of(const Args& a, int i, int q) {
+  const int nb = __ldg(a.cnbr + q * a.g.ncols + i);
+#ifdef PM_CHECKED
+  if (nb < -1 || nb >= a.g.ncols) {
+    record_bad_index(SITE_NBR, nb, a.g.ncols);
+    return -1;
+  }
+#endif
+  return nb;
+}
+
+__device__ __forceinline__ double ldval(const double* p) { return __ldg(p); }
+__device__ __forceinline__ float ldval(const float* p) { return __ldg(p); }
+__device__ __forceinline__ float ldval(const __nv_bfloat16* p) {
+  return __bfloat162float(__ushort_as_bfloat16(__ldg(reinterpret_cast<const unsigned short*>(p))));
+}
+
+// Row of A times x. The mask's clear bits are slots that do not count: absent neighbours (their
+// values are 0) and, for a velocity, Dirichlet ones. FP32: the difference form (row sum in the
+// diagonal slot, eliminated slots' values taken off it).
+template <typename T, typename TV>
+__device__ __forceinline__ T row_apply(const Geom& g, const TV* __restrict__ val, const T* x,
+                                       const uint16_t* __restrict__ mask, int row, int col, int k) {
+  const int nz = g.nz, npad = (int)g.npad;
+  const uint32_t km = __ldg(mask + row);
+  if (km & 0x8000u) return x[row];
+  int nb[NNBR];
+  nb[0] = col;
+#pragma unroll
+  for (int q = 1; q < NNBR; ++q) nb[q] = nbr_of(g, col, q);
+  T a[NSLOT], xv[NSLOT];
+#pragma unroll
+  for (int s = 0; s < NSLOT; ++s) a[s] = ldval(val + s * npad + row);
+#pragma unroll
+  for (int s = 0; s < NSLOT; ++s) xv[s] = x[((km >> s) & 1u) ? nb[slot_q(s)] * nz + k + slot_dk(s) : row];
+  T sum = 0;
+  if constexpr (std::is_same<T, double>::value) {
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) sum = fma(((km >> s) & 1u) ? a[s] : 0.0, xv[s], sum);
+    return sum;
+  } else {
+    const float xi = xv[DIAG_SLOT];
+    float drop = 0.f;
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      if (s == DIAG_SLOT) continue;
+      const bool keep = (km >> s) & 1u;
+      drop += keep ? 0.f : a[s];
+      sum = fmaf(keep ? a[s] : 0.f, xv[s] - xi, sum);
+    }
+    return fmaf(a[DIAG_SLOT] - drop, xi, sum);
+  }
+}
+
+// b_i - (A x)_i by Dot2 (row_residual_dot2), slots by the mask.
+__device__ __forceinline__ double row_residual(const Geom& g, const double* __restrict__ val, const double* x,
+                                               const uint16_t* __restrict__ mask, double bi, int row, int col, int k,
+                                               double& abs_sum) {
+  const int nz = g.nz, npad = (int)g.npad;
+  const uint32_t km = __ldg(mask + row);
+  if (km & 0x8000u) {
+    const double xi = x[row];
+    abs_sum = fabs(xi);
+    return __dsub_rn(bi, xi);
+  }
+  int nb[NNBR];
+  nb[0] = col;
+#pragma unroll
+  for (int q = 1; q < NNBR; ++q) nb[q] = nbr_of(g, col, q);
+  double s = bi, c = 0.0, asum = 0.0;
+#pragma unroll
+  for (int sl = 0; sl < NSLOT; ++sl) {
+    const bool ok = (km >> sl) & 1u;
+    const double av = ok ? __ldg(val + sl * npad + row) : 0.0;
+    const double xv = x[ok ? nb[slot_q(sl)] * nz + k + slot_dk(sl) : row];
+    double pe, se;
+    const double pr = two_product(av, xv, pe);
+    s = two_sum(s, -pr, se);
+    c = __dadd_rn(c, __dsub_rn(se, pe));
+    asum += fabs(pr);
+  }
+  abs_sum = asum;
+  return __dadd_rn(s, c);
+}
+
+// ---- IC0 ---------------------------------------------------------------------------------------
+
+// Sums of one sweep pass: (r, r), (y, y) = (r, z), m'z, 1'r.
+template <typename T>
+struct Dots {
+  AccFor<T> rr, rz, mz, sr;
+};
+
+__device__ __forceinline__ void add_m(Acc64& acc, const Args& a, int row, double z) { acc.add_prod(__ldg(a.m + row), z); }
+__device__ __forceinline__ void add_m(DF& acc, const Args& a, int row, float z) {
+  const float2 m = __ldg(a.m2 + row);
+  acc.add_prod(m.x, z);
+  acc.add_prod(m.y, z);
+}
+
+// The vector that alpha p is added to: the FP64 iterate, or the FP32 correction of a mixed-precision solve.
+template <typename T>
+__device__ __forceinline__ T* iterate(const Args& a) {
+  if constexpr (std::is_same<T, double>::value) return a.x;
+  else return a.d;
+}
+// x += alpha p, p = z + beta p on one row.
+template <typename T>
+__device__ __forceinline__ void move_row(const Args& a, int row, T alpha, T beta, T z) {
+  T* p = static_cast<T*>(a.p);
+  T* x = iterate<T>(a);
+  const T pv = p[row];
+  x[row] = fma(alpha, pv, x[row]);
+  p[row] = fma(beta, pv, z);
+}
+
+// Constant operands of one row of a colour phase: its place, neighbour columns and factor row.
+template <typename T, int C, bool FWD>
+struct ColourRow {
+  static constexpr int kpar = C >> 2, cls = C & 3;
+  int row, k;
+  int nb[NNBR];
+  T f[NSLOT];
+  // The slots read: lower colours forward, higher ones backward.
+  static __host__ __device__ constexpr bool uses(int s) {
+    return s != DIAG_SLOT && (FWD ? (C ^ slot_flip(s)) < C : (C ^ slot_flip(s)) > C);
+  }
+  // t: place within the colour. Reads stay inside the arrays for t = 0 of an empty colour.
+  __device__ __forceinline__ void load(const Args& a, int t) {
+    const T* __restrict__ F = static_cast<const T*>(a.ic0);
+    const int i = fdiv(a.nlev[kpar], t), n = (int)a.g.n;
+    const int at = min(a.cls_off[cls] + i, a.g.ncols - 1), pos = min(a.cbase[C] + t, n - 1);
+    k = 2 * (t - i * a.nlev[kpar].d) + kpar;
+#pragma unroll
+    for (int q = 0; q < NNBR; ++q) nb[q] = cnbr_of(a, at, q);
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s)
+      if (uses(s) || s == DIAG_SLOT) f[s] = __ldg(F + (s * n + pos));
+    row = nb[0] * a.g.nz + k;
+  }
+  // (v - sum f_s y_s) / L_ii
+  __device__ __forceinline__ T value(int nz, T v, const T* y) const {
+    T yv[NSLOT];
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      if (!uses(s)) continue;
+      const int kk = k + slot_dk(s), q = slot_q(s);
+      bool ok = nb[q] >= 0;
+      if (slot_dk(s) < 0) ok = ok && kk >= 0;
+      if (slot_dk(s) > 0) ok = ok && kk < nz;
+      yv[s] = ok ? y[nb[q] * nz + kk] : (T)0;
+    }
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s)
+      if (uses(s)) v = fma(-f[s], yv[s], v);
+    return v * f[DIAG_SLOT];
+  }
+};
+
+// One colour phase over this block's share of the colour's rows. Forward (FWD): y_i = (r_i - sum L_ij y_j) / L_ii
+// over lower colours; colour 7 goes straight on to its backward value z_i = y_i / L_ii (no higher
+// colour exists). Backward: z_i = (y_i - sum L_ji z_j) / L_ii over higher colours, in place, and
+// (FUSEP) x_i += alpha p_i, p_i = z_i + beta p_i. The constant operands of a thread's first row are fetched before
+// the barrier that its neighbours' values wait for (SYNC). acc takes (y, y) on forward phases.
+template <typename T, int C, bool FWD, bool FUSEP, bool SYNC, bool CL, typename Acc>
+__device__ __forceinline__ bool colour_phase(const Args& a, Team<CL>& team, T alpha, T beta, Acc& acc) {
+  using Row = ColourRow<T, C, FWD>;
+  const T* r = static_cast<const T*>(a.r);
+  T* y = static_cast<T*>(a.z);
+  const int nz = a.g.nz;
+  const int tot = a.cls_cnt[Row::cls] * a.nlev[Row::kpar].d;
+  const int t0 = (int)((int64_t)tot * team.rank / team.G), t1 = (int)((int64_t)tot * (team.rank + 1) / team.G);
+  int t = t0 + (int)threadIdx.x;
+  Row w;
+  if (SYNC) {
+    // without a condition (a clamped place instead): loaded under one, the row went to local memory
+    w.load(a, max(0, min(t, tot - 1)));
+    if (!team.wait()) return false;
+  }
+#pragma unroll 1
+  for (bool first = SYNC; t < t1; t += NT, first = false) {
+    if (!first) w.load(a, t);
+    T v = w.value(nz, FWD ? r[w.row] : y[w.row], y);
+    if (FWD) {
+      acc.add_prod(v, v);
+      if (C == 7) v *= w.f[DIAG_SLOT];
+    }
+    y[w.row] = v;
+    if (FUSEP) move_row(a, w.row, alpha, beta, v);
+  }
+  return true;
+}
+
+// y of colour 0 for one row in natural order: r / L_ii (no lower colour). Other rows: nothing.
+template <typename T, typename Acc>
+__device__ __forceinline__ void colour0_y(const Args& a, int row, int col, int k, T ri, Acc& acc) {
+  if ((k | __ldg(a.coli + col) | __ldg(a.colj + col)) & 1) return;
+  const int t = __ldg(a.clsidx + col) * a.nlev[0].d + (k >> 1);
+  const T v = ri * __ldg(static_cast<const T*>(a.ic0) + DIAG_SLOT * (int)a.g.n + t);
+  static_cast<T*>(a.z)[row] = v;
+  acc.add_prod(v, v);
+}
+
+// Forward sweep after colour 0; (y, y) = (r, z) is summed over the team (a barrier).
+template <typename T, bool CL, typename Acc>
+__device__ __forceinline__ bool ic0_forward(const Args& a, Team<CL>& team, Acc& acc, double& yy) {
+  if (!colour_phase<T, 1, true, false, false>(a, team, (T)0, (T)0, acc)) return false;
+#define PM_FWD(C)                                                                          \
+  team.arrive();                                                                           \
+  if (!colour_phase<T, C, true, false, true>(a, team, (T)0, (T)0, acc)) return false;
+  PM_FWD(2) PM_FWD(3) PM_FWD(4) PM_FWD(5) PM_FWD(6) PM_FWD(7)
+#undef PM_FWD
+  double v[1] = {acc.value()};
+  if (!team.template sum<1>(v)) return false;
+  yy = v[0];
+  return true;
+}
+
+// Backward sweep from colour 6 on, with x and p when FUSEP, and the barrier after it.
+template <typename T, bool FUSEP, bool CL>
+__device__ __forceinline__ bool ic0_backward(const Args& a, Team<CL>& team, T alpha, T beta) {
+  Acc64 unused;
+  if (FUSEP) {   // rows of colour 7 have their z already: x and p where this block formed it
+    const int tot = a.cls_cnt[3] * a.nlev[1].d;
+    const int t1 = (int)((int64_t)tot * (team.rank + 1) / team.G);
+    for (int t = (int)((int64_t)tot * team.rank / team.G) + (int)threadIdx.x; t < t1; t += NT) {
+      const int i = fdiv(a.nlev[1], t);
+      const int row = __ldg(a.cnbr + a.cls_off[3] + i) * a.g.nz + 2 * (t - i * a.nlev[1].d) + 1;
+      move_row(a, row, alpha, beta, static_cast<const T*>(a.z)[row]);
+    }
+  }
+  if (!colour_phase<T, 6, false, FUSEP, false>(a, team, alpha, beta, unused)) return false;
+#define PM_BWD(C)                                                                          \
+  team.arrive();                                                                           \
+  if (!colour_phase<T, C, false, FUSEP, true>(a, team, alpha, beta, unused)) return false;
+  PM_BWD(5) PM_BWD(4) PM_BWD(3) PM_BWD(2) PM_BWD(1) PM_BWD(0)
+#undef PM_BWD
+  return team.barrier();
+}
+
+// ---- the update and the column-local preconditioners ------------------------------------------
+
+// r -= alpha w (UPDATE), then z by the preconditioner, on this block's columns [c0, c1). LINE: zt is the
+// block's tile of columns, ld apart (shared memory, or its part of the z vector).
+template <typename T, int PREC, bool UPDATE>
+__device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alpha, T* zt, int ld, Dots<T>& dots) {
+  const Geom& g = a.g;
+  const int nz = g.nz, row0 = c0 * nz, row1 = c1 * nz;
+  T* r = static_cast<T*>(a.r);
+  const T* w = static_cast<const T*>(a.w);
+  const T* dinv = static_cast<const T*>(a.dinv);
+  constexpr int U = 4;   // rows whose loads are in flight together
+  for (int i0 = row0 + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
+    T rv[U], wv[U], dv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = min(i0 + u * NT, row1 - 1);
+      rv[u] = r[row];
+      if (UPDATE) wv[u] = w[row];
+      if (PREC == PM_PREC_JACOBI) dv[u] = dinv ? __ldg(dinv + row) : (T)1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = i0 + u * NT;
+      if (row >= row1) break;
+      T ri = rv[u];
+      if (UPDATE) {
+        ri = fma(-alpha, wv[u], ri);
+        r[row] = ri;
+      }
+      dots.rr.add_prod(ri, ri);
+      if (a.proj) dots.sr.add(ri);
+      if (PREC == PM_PREC_JACOBI) {
+        const T zi = dv[u] * ri;
+        dots.rz.add_prod(ri, zi);
+        if (a.proj) add_m(dots.mz, a, row, zi);
+      } else {
+        const int col = fdiv(g.nzd, row), k = row - col * nz;
+        if (PREC == PM_PREC_LINE) zt[(col - c0) * ld + k] = ri;
+        else colour0_y(a, row, col, k, ri, dots.rz);
+      }
+    }
+  }
+  if (PREC != PM_PREC_LINE) return;
+  __syncthreads();
+  // Thomas solve of each column, one thread per column; (r, z) = sum_k t_k y_k (symmetric blocks)
+  const T* F = static_cast<const T*>(a.line);
+  const int nc = g.ncols, n = (int)g.n;
+  for (int col = c0 + (int)threadIdx.x; col < c1; col += NT) {
+    T* cs = zt + (col - c0) * ld;
+    T y = 0;
+#pragma unroll 8
+    for (int k = 0; k < nz; ++k) {
+      const int li = k * nc + col;
+      const T tk = fma(-__ldg(F + li), y, cs[k]);
+      y = tk * __ldg(F + n + li);
+      dots.rz.add_prod(tk, y);
+      cs[k] = y;
+    }
+    T zn = y;
+#pragma unroll 8
+    for (int k = nz - 2; k >= 0; --k) {
+      zn = fma(-__ldg(F + 2 * n + k * nc + col), zn, cs[k]);
+      cs[k] = zn;
+    }
+  }
+  __syncthreads();
+  if (!a.proj) return;
+  for (int row = row0 + (int)threadIdx.x; row < row1; row += NT) {
+    const int col = fdiv(g.nzd, row);
+    add_m(dots.mz, a, row, zt[(col - c0) * ld + row - col * nz]);
+  }
+}
+
+// x += alpha p and p = (z - c) + beta p on the block's rows. x moves here, a pass after r, because p is read
+// here anyway. FIRST: p = z - c.
+// LAST: x alone, when no further direction is needed.
+template <typename T, int PREC, bool FIRST, bool LAST>
+__device__ __forceinline__ void direction(const Args& a, int c0, int c1, T alpha, T beta, T c, const T* zt, int ld) {
+  const Geom& g = a.g;
+  const int nz = g.nz, row1 = c1 * nz;
+  T* p = static_cast<T*>(a.p);
+  T* x = iterate<T>(a);
+  const T* r = static_cast<const T*>(a.r);
+  const T* zv = static_cast<const T*>(a.z);
+  const T* dinv = static_cast<const T*>(a.dinv);
+  constexpr int U = 4;
+  for (int i0 = c0 * nz + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
+    T z[U], pv[U], xv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = min(i0 + u * NT, row1 - 1);
+      if (!LAST) {
+        if (PREC == PM_PREC_JACOBI) {
+          z[u] = (dinv ? __ldg(dinv + row) : (T)1) * r[row];
+        } else if (PREC == PM_PREC_LINE) {
+          const int col = fdiv(g.nzd, row);
+          z[u] = zt[(col - c0) * ld + row - col * nz];
+        } else {
+          z[u] = zv[row];
+        }
+      }
+      if (!FIRST) {
+        pv[u] = p[row];
+        xv[u] = x[row];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = i0 + u * NT;
+      if (row >= row1) break;
+      if (!FIRST) x[row] = fma(alpha, pv[u], xv[u]);
+      if (!LAST) p[row] = FIRST ? z[u] - c : fma(beta, pv[u], z[u] - c);
+    }
+  }
+}
+
+// State of the PCG recurrence, the same in every thread of the team.
+struct Cg {
+  double rho = 0.0, rr = 0.0;
+  int iter = 0, status = PM_OK;
+};
+
+// r -= alpha w (not FIRST), z = P^{-1} r, (r, r), then x += alpha p, rho, beta and p, and the barrier
+// after which every block may read p. FIRST: from r alone, beta = 0. STOP is asked once cg.rr = (r, r) is
+// known: true ends the step with x moved (the recursion has met its target). cg.status is PM_BREAKDOWN
+// when rho is not positive. Returns false when a wait ran out.
+template <typename T, int PREC, bool FIRST, bool CL, typename Stop>
+__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, int c0, int c1, T* zt, int ld, double alpha, Cg& cg,
+                                        bool& stopped, Stop stop) {
+  Dots<T> dots;
+  update_rows<T, PREC, !FIRST>(a, c0, c1, (T)alpha, zt, ld, dots);
+  double c = 0.0, rho = 0.0;
+  if (PREC == PM_PREC_IC0) {
+    double v[1] = {dots.rr.value()};
+    if (!team.template sum<1>(v)) return false;
+    cg.rr = v[0];
+    stopped = stop();
+    if (!stopped && !ic0_forward<T>(a, team, dots.rz, rho)) return false;
+    if (!stopped && a.proj) {   // the projection needs the whole z before p
+      if (!ic0_backward<T, false>(a, team, (T)0, (T)0)) return false;
+      const T* r = static_cast<const T*>(a.r);
+      const T* z = static_cast<const T*>(a.z);
+      AccFor<T> rz;
+      for (int row = c0 * a.g.nz + (int)threadIdx.x; row < c1 * a.g.nz; row += NT) {
+        rz.add_prod(r[row], z[row]);
+        add_m(dots.mz, a, row, z[row]);
+      }
+      double u[3] = {rz.value(), dots.mz.value(), dots.sr.value()};
+      if (!team.template sum<3>(u)) return false;
+      c = u[1] / a.one_m;
+      rho = u[0] - c * u[2];
+    }
+  } else if (a.proj) {
+    double v[4] = {dots.rr.value(), dots.rz.value(), dots.mz.value(), dots.sr.value()};
+    if (!team.template sum<4>(v)) return false;
+    cg.rr = v[0];
+    c = v[2] / a.one_m;
+    rho = v[1] - c * v[3];
+    stopped = stop();
+  } else {
+    double v[2] = {dots.rr.value(), dots.rz.value()};
+    if (!team.template sum<2>(v)) return false;
+    cg.rr = v[0];
+    rho = v[1];
+    stopped = stop();
+  }
+  const bool broken = !stopped && (!(rho > 0.0) || !isfinite(rho));
+  if (broken) cg.status = PM_BREAKDOWN;
+  if (stopped || broken) {
+    direction<T, PREC, FIRST, true>(a, c0, c1, (T)alpha, (T)0, (T)0, zt, ld);
+    return team.barrier();
+  }
+  const T beta = FIRST ? (T)0 : (T)(rho / cg.rho);
+  cg.rho = rho;
+  if (PREC == PM_PREC_IC0 && !a.proj) {
+    if (!FIRST) return ic0_backward<T, true>(a, team, (T)alpha, beta);
+    // p may hold anything yet (not a number included): set afterwards, not scaled by 0
+    if (!ic0_backward<T, false>(a, team, (T)0, (T)0)) return false;
+  }
+  direction<T, PREC, FIRST, false>(a, c0, c1, (T)alpha, beta, (T)c, zt, ld);
+  return team.barrier();
+}
+
+// w = A p on the block's rows; v = (p, w) over the team.
+template <typename T, typename TV, bool CL>
+__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, int c0, int c1, double& pw) {
+  const Geom& g = a.g;
+  const TV* val = static_cast<const TV*>(a.val);
+  const T* p = static_cast<const T*>(a.p);
+  T* w = static_cast<T*>(a.w);
+  AccFor<T> acc;
+  for (int row = c0 * g.nz + (int)threadIdx.x; row < c1 * g.nz; row += NT) {
+    const int col = fdiv(g.nzd, row);
+    const T wi = row_apply<T, TV>(g, val, p, a.mask, row, col, row - col * g.nz);
+    w[row] = wi;
+    acc.add_prod(p[row], wi);
+  }
+  double v[1] = {acc.value()};
+  if (!team.template sum<1>(v)) return false;
+  pw = v[0];
+  return true;
+}
+
+// r = b - A x (compensated), (r, r) and the floor's (|A||x| + |b|)^2 over the team.
+template <typename T, bool CL>
+__device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, int c0, int c1, const double* b, double& rr,
+                                              double& ff) {
+  const Geom& g = a.g;
+  T* r = static_cast<T*>(a.r);
+  double v[2] = {0.0, 0.0};
+  for (int row = c0 * g.nz + (int)threadIdx.x; row < c1 * g.nz; row += NT) {
+    const int col = fdiv(g.nzd, row);
+    double asum;
+    const double bi = b[row];
+    const double ri = row_residual(g, a.val64, a.x, a.mask, bi, row, col, row - col * g.nz, asum);
+    r[row] = (T)ri;
+    v[0] = fma(ri, ri, v[0]);
+    const double f = asum + fabs(bi);
+    v[1] = fma(f, f, v[1]);
+  }
+  if (!team.template sum<2>(v)) return false;
+  rr = v[0];
+  ff = v[1];
+  return true;
+}
+
+// Right-hand side, initial guess and first residual: (b', b') and (r, r). From x = 0 the residual is b' itself.
+template <typename T, bool CL>
+__device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, int c0, int c1, const double*& b, double& bb,
+                                            double& rr) {
+  const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
+  double lam = 0.0, xs = 0.0;
+  b = a.b;
+  if (a.proj) {
+    double v[2] = {0.0, 0.0};
+    for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) {
+      v[0] += b[i];
+      if (a.x0_is_guess) v[1] = fma(a.m[i], a.x[i], v[1]);
+    }
+    if (!team.template sum<2>(v)) return false;
+    lam = v[0] / a.one_m;
+    xs = a.x0_is_guess ? v[1] / a.one_m : 0.0;
+  }
+  T* r = static_cast<T*>(a.r);
+  double v[2] = {0.0, 0.0};
+  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) {
+    double bi = b[i];
+    if (a.proj) {
+      bi = bi - lam * a.m[i];
+      a.bw[i] = bi;
+    }
+    if (!a.x0_is_guess) {
+      a.x[i] = 0.0;
+      r[i] = (T)bi;
+    } else if (a.proj) {
+      a.x[i] = a.x[i] - xs;
+    }
+    v[0] = fma(bi, bi, v[0]);
+  }
+  if (a.proj) b = a.bw;
+  v[1] = v[0];
+  if (!team.template sum<1>(*reinterpret_cast<double(*)[1]>(v))) return false;
+  bb = v[0];
+  rr = bb;
+  double ff;
+  if (a.x0_is_guess && !true_residual<T>(a, team, c0, c1, b, rr, ff)) return false;
+  return true;
+}
+
+// The returned pressure has m'x = 0.
+template <bool CL>
+__device__ __forceinline__ bool zero_mean(const Args& a, Team<CL>& team, int c0, int c1) {
+  const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
+  double v[1] = {0.0};
+  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) v[0] = fma(a.m[i], a.x[i], v[0]);
+  if (!team.template sum<1>(v)) return false;
+  const double sh = v[0] / a.one_m;
+  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.x[i] -= sh;
+  return true;
+}
+
+// The FP64 solve: PCG on the recursive residual, then the true residual, restarts while they help.
+template <int PREC, bool CL>
+__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, int c1, double* zt, int ld, Out& o) {
+  const double* b;
+  double bb, rr;
+  if (!start_solve<double>(a, team, c0, c1, b, bb, rr)) return false;
+  const double tol2 = a.rtol * a.rtol * bb;
+  Cg cg;
+  int restarts = 0, first_pass = -1;
+  double rel_true = 0.0, floor = 0.0, prev_true = -1.0;
+  bool accepted = false;
+  bool skip = rr <= tol2;   // x0 already meets rtol
+  if (!skip && a.max_iter == 0 && bb != 0.0) cg.status = PM_NOT_CONVERGED;
+  cg.rr = rr;
+  if (bb == 0.0)
+    for (int i = c0 * a.g.nz + (int)threadIdx.x; i < c1 * a.g.nz; i += NT) a.x[i] = 0.0;
+  while (bb != 0.0) {
+    if (cg.status == PM_OK && !skip) {
+      bool converged = false, stopped;
+      if (!advance<double, PREC, true>(a, team, c0, c1, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
+      while (cg.status == PM_OK && cg.iter < a.max_iter) {
+        double pw;
+        if (!apply_dot<double, double>(a, team, c0, c1, pw)) return false;
+        if (!(pw > 0.0) || !isfinite(pw)) {
+          cg.status = PM_BREAKDOWN;
+          break;
+        }
+        const bool fine = advance<double, PREC, false>(a, team, c0, c1, zt, ld, cg.rho / pw, cg, stopped, [&] {
+          ++cg.iter;
+          converged = cg.rr <= tol2;
+          return converged || cg.iter >= a.max_iter;
+        });
+        if (!fine) return false;
+        if (stopped) break;
+      }
+      if (cg.status == PM_OK && !converged) cg.status = PM_NOT_CONVERGED;   // iteration cap
+    }
+    skip = false;
+    if (first_pass < 0) first_pass = cg.iter;
+    double tr, ff;
+    if (!true_residual<double>(a, team, c0, c1, b, tr, ff)) return false;
+    rel_true = sqrt(tr / bb);
+    floor = ldexp(1.0, -53) * sqrt(ff / bb);
+    const bool stalled = prev_true >= 0.0 && rel_true > 0.5 * prev_true;
+    const bool last = restarts >= a.max_restarts || cg.iter >= a.max_iter;
+    accepted = rel_true <= a.rtol || (rel_true <= floor && (stalled || last));
+    if (cg.status != PM_OK || accepted || last) break;
+    prev_true = rel_true;
+    cg.rr = tr;
+    ++restarts;
+  }
+  if (bb != 0.0 && cg.status == PM_OK && !accepted) cg.status = PM_NOT_CONVERGED;
+  if (a.proj && !zero_mean(a, team, c0, c1)) return false;
+  o.iters = cg.iter;
+  o.restarts = restarts;
+  o.first_pass = first_pass < 0 ? cg.iter : first_pass;
+  o.status = cg.status;
+  o.zero_rhs = bb == 0.0;
+  o.rel_true = bb == 0.0 ? 0.0 : rel_true;
+  o.rel_rec = bb == 0.0 ? 0.0 : sqrt(cg.rr / bb);
+  o.floor = floor;
+  return true;
+}
+
+// The mixed-precision solve: inner PCG with FP32 vectors on the difference-form values; each time the
+// recursive residual has dropped by inner_rtol, or claims convergence, the FP32 correction is folded into the
+// FP64 iterate, the true residual b - A x is formed (compensated) and a new inner solve starts from it.
+template <typename TV, int PREC, bool CL>
+__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c0, int c1, float* zt, int ld, Out& o) {
+  const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
+  const double* b;
+  double bb, rr;
+  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.d[i] = 0.f;
+  if (!start_solve<float>(a, team, c0, c1, b, bb, rr)) return false;
+  const double tol2 = a.rtol * a.rtol * bb, drop = a.inner_rtol * a.inner_rtol;
+  Cg cg;
+  int outer = 0, stalled = 0;
+  double rel_true = 0.0, floor = 0.0, prev_true = 1e300;
+  if (bb == 0.0) {
+    for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.x[i] = 0.0;
+  } else if (rr <= tol2 || a.max_iter == 0) {   // x0 already meets rtol, or no iteration is allowed
+    if (rr > tol2) cg.status = PM_NOT_CONVERGED;
+    rel_true = sqrt(rr / bb);
+  } else {
+    for (;;) {
+      const double target = fmax(tol2, drop * rr);
+      bool stopped;
+      if (!advance<float, PREC, true>(a, team, c0, c1, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
+      while (cg.status == PM_OK) {
+        double pw;
+        if (!apply_dot<float, TV>(a, team, c0, c1, pw)) return false;
+        if (!(pw > 0.0) || !isfinite(pw)) {
+          cg.status = PM_BREAKDOWN;
+          break;
+        }
+        const bool fine = advance<float, PREC, false>(a, team, c0, c1, zt, ld, cg.rho / pw, cg, stopped, [&] {
+          ++cg.iter;
+          return cg.rr <= target || cg.iter >= a.max_iter;
+        });
+        if (!fine) return false;
+        if (stopped) break;
+      }
+      for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) {
+        a.x[i] += (double)a.d[i];
+        a.d[i] = 0.f;
+      }
+      if (!team.barrier()) return false;
+      double ff;
+      if (!true_residual<float>(a, team, c0, c1, b, rr, ff)) return false;
+      ++outer;
+      rel_true = sqrt(rr / bb);
+      floor = ldexp(1.0, -53) * sqrt(ff / bb);
+      const bool stalled_now = rel_true > 0.5 * prev_true;   // this step did not halve the true residual
+      const bool broken = cg.status == PM_BREAKDOWN;
+      cg.status = PM_OK;
+      if (rel_true <= a.rtol || (rel_true <= floor && stalled_now)) break;
+      stalled = stalled_now ? stalled + 1 : 0;
+      prev_true = rel_true;
+      if (stalled >= 3) {   // stagnation above the floor
+        cg.status = PM_NOT_CONVERGED;
+        break;
+      }
+      if (broken) {
+        cg.status = PM_BREAKDOWN;
+        break;
+      }
+      if (cg.iter >= a.max_iter) {   // no iteration left: accepted only below the floor
+        if (rel_true > floor) cg.status = PM_NOT_CONVERGED;
+        break;
+      }
+    }
+  }
+  if (a.proj && !zero_mean(a, team, c0, c1)) return false;
+  o.iters = o.first_pass = cg.iter;
+  o.restarts = outer;
+  o.status = cg.status;
+  o.zero_rhs = bb == 0.0;
+  o.rel_true = o.rel_rec = bb == 0.0 ? 0.0 : rel_true;
+  o.floor = floor;
+  return true;
+}
+
+template <typename T, typename TV, int PREC, bool CL>
+__global__ void __launch_bounds__(NT, 1) k_resident(Args a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ Scratch scratch;
+  Team<CL> team(a, &scratch);
+  if (CL) team.barrier();   // every block of the cluster runs before one writes to another's shared memory
+  // whole columns, dealt evenly
+  const int c0 = (int)((int64_t)a.g.ncols * team.rank / team.G), c1 = (int)((int64_t)a.g.ncols * (team.rank + 1) / team.G);
+  T* zt;
+  int ld = a.g.nz | 1;   // odd: a warp's columns fall into different banks
+  if (a.z_in_smem) {
+    zt = reinterpret_cast<T*>(smem_raw);
+  } else {
+    zt = static_cast<T*>(a.z) + (int64_t)c0 * a.g.nz;
+    ld = a.g.nz;
+  }
+  Out o;
+  bool fine;
+  if constexpr (std::is_same<T, double>::value) fine = solve64<PREC>(a, team, c0, c1, zt, ld, o);
+  else fine = solve_mixed<TV, PREC>(a, team, c0, c1, zt, ld, o);
+  if (!fine) {
+    if (threadIdx.x == 0) *(volatile int32_t*)&a.out->status = PM_TIMEOUT;
+    return;
+  }
+  if (team.rank == 0 && threadIdx.x == 0) *a.out = o;
+  if (CL) team.barrier();   // no block of a cluster leaves while another may still write to its shared memory
+}
+
+// ---- launch ------------------------------------------------------------------------------------
+
+constexpr size_t TILE_LIMIT = 200 * 1024;   // shared memory of a block's tile of columns
+
+template <typename T, typename TV, int PREC, bool CL>
+inline int launch_one(Args& a, int grid, size_t smem, cudaStream_t s) {
+  const void* f = (const void*)k_resident<T, TV, PREC, CL>;
+  int st;
+  if (smem && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                               "resident shared memory")))
+    return st;
+  if (CL && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster size")))
+    return st;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (CL) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)grid;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if ((st = cuda_check(cudaMemsetAsync(a.ctl, 0, sizeof(Ctl), s), "resident barrier"))) return st;
+  st = cuda_check(cudaLaunchKernelEx(&cfg, k_resident<T, TV, PREC, CL>, a), "k_resident");
+  count_launch();
+  return st;
+}
+
+// Dynamic shared memory of a block's columns (line preconditioner), or 0 when they do not fit.
+inline size_t tile_bytes(int64_t ncols, int nz, int grid, size_t elem) {
+  const int64_t cols = (ncols + grid - 1) / grid;
+  const size_t b = (size_t)cols * (size_t)(nz | 1) * elem;
+  return b <= TILE_LIMIT ? b : 0;
+}
+
+template <typename T, typename TV, bool CL>
+int launch_prec(Args& a, int prec, int grid, cudaStream_t s) {
+  const size_t smem = prec == PM_PREC_LINE ? tile_bytes(a.g.ncols, a.g.nz, grid, sizeof(T)) : 0;
+  a.z_in_smem = smem > 0;
+  switch (prec) {
+    case PM_PREC_IC0: return launch_one<T, TV, PM_PREC_IC0, CL>(a, grid, smem, s);
+    case PM_PREC_LINE: return launch_one<T, TV, PM_PREC_LINE, CL>(a, grid, smem, s);
+    default: return launch_one<T, TV, PM_PREC_JACOBI, CL>(a, grid, smem, s);
+  }
+}
+
+template <typename T, typename TV>
+int launch(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s) {
+  return cluster ? launch_prec<T, TV, true>(a, prec, CLUSTER, s) : launch_prec<T, TV, false>(a, prec, num_sms, s);
+}
+
+// One file each (pm_resident.cu, pm_resident_fp32.cu, pm_resident_bf16.cu), so that they compile side by side.
+int launch_fp64(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s);
+int launch_fp32(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s);
+int launch_bf16(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s);
+
+}  // namespace resident
+}  // namespace pm

@@ -9,6 +9,8 @@
 //                    reductions (r, r), (r, z) [and m'z, 1'r for the pressure]; the last block
 //                    tests convergence and forms beta
 //   K3 k_cg_pupd   : p = z + beta p
+// This file's kernels run one phase each over the whole GPU (PM_KERNEL_STREAM, and large systems);
+// below resident_auto's lines one launch runs the whole solve (pm_resident.cuh).
 // IC0 replaces the inline z by 8 forward and 8 backward colour sweeps plus a (r, z) reduction.
 // Grid reductions are deterministic: each block reduces its rows in a fixed tree, writes one
 // partial, and the last block to arrive (atomic ticket) sums the partials in block order.
@@ -25,6 +27,7 @@
 #include <type_traits>
 
 #include "pm_internal.cuh"
+#include "pm_resident.cuh"
 
 namespace pm {
 
@@ -39,8 +42,8 @@ struct SolveCtx {
   float *r32 = nullptr, *p32 = nullptr, *w32 = nullptr, *z32 = nullptr, *d32 = nullptr;
   PcgScalars* sc_in = nullptr;
   PcgScalars* sc_in_host = nullptr;
-  void* small_out = nullptr;        // SmallOut of the resident solve (device)
-  void* small_out_host = nullptr;   // pinned host copy
+  void* res_ctl = nullptr;        // barrier of the resident solve (device)
+  void* res_out = nullptr;   // its results (pinned; the kernel writes them there)
 };
 
 struct ColourMap;  // pm_assemble.cu
@@ -1039,8 +1042,8 @@ int ensure_ctx(pm_operator* op) {
   e = e ? e : cudaMalloc((void**)&c->partials, (size_t)NPART * MAX_GRID * sizeof(double));
   e = e ? e : cudaMalloc((void**)&c->sc, sizeof(PcgScalars));
   e = e ? e : cudaMallocHost((void**)&c->sc_host, sizeof(PcgScalars));
-  e = e ? e : cudaMalloc(&c->small_out, 64);
-  e = e ? e : cudaMallocHost(&c->small_out_host, 64);
+  e = e ? e : cudaMalloc(&c->res_ctl, 64);
+  e = e ? e : cudaMallocHost(&c->res_out, 64);
   if (e == cudaSuccess) e = cudaMemset(c->sc, 0, sizeof(PcgScalars));
   op->ctx = c;
   if (e != cudaSuccess) return cuda_check(e, "solve workspace");
@@ -1309,273 +1312,18 @@ int pcg_run(pm_operator* op, int which, const double* b, double* x, const pm_sol
   return PM_OK;
 }
 
-// ---- resident solve of a small system: one block runs the whole PCG ----------------------------
-// The multi-kernel solve costs about twenty launches per IC0 iteration; on a few thousand rows each
-// of them is a few microseconds of launch latency around far less work. Here one block of
-// SMALL_TPB threads runs every step of the same PCG (the same preconditioners, projection,
-// stopping rule and true-residual restarts) with __syncthreads between phases, and writes its
-// statistics to device memory once. The FP64 work of one SM bounds it; it is used where that
-// is cheaper than the launches (n <= SMALL_AUTO_ROWS by default).
-constexpr int SMALL_TPB = 256;
-constexpr int64_t SMALL_AUTO_ROWS = 16384;   // automatic choice of the resident solve
-constexpr int64_t SMALL_MAX_ROWS = 1 << 20;  // accepted when requested explicitly
+// ---- resident solve: one launch runs the whole PCG (pm_resident.cuh) ---------------------------
+constexpr int64_t RESIDENT_MAX_ROWS = 1 << 20;    // accepted when requested explicitly
+// Automatic choice of the resident solve (measured lines: resident_auto).
+constexpr int64_t RESIDENT_AUTO_ROWS = 3 << 20, RESIDENT_AUTO_MIXED_LINE = 5 << 18;
+// Up to here by one cluster of blocks. Measured, us per iteration, cluster / grid: IC0 n = 2,048 40 / 49, 18,000
+// 50 / 49; line 11,803 18.3 / 18.1, 18,000 24 / 21; Jacobi 2,048 10 / 14, 11,803 15.5 / 14.2.
+constexpr int64_t RESIDENT_CLUSTER_ROWS = 8192, RESIDENT_CLUSTER_IC0 = 16384;
 
-struct SmallArgs {
-  double rtol, one_m;
-  int32_t max_iter, max_restarts, x0_is_guess, proj;
-  const double* dinv;     // Jacobi inverse diagonal (ones for PM_PREC_NONE)
-  const uint16_t* keep;   // keep mask of the velocity component (MASKC >= 0)
-  const double* m;        // M 1
-  const double* Fic;      // IC0 factor (colour-ordered rows)
-  const double* Fl;       // line factors (level-major)
-  const int32_t* cls_cols;
-  CMap cm;
-  int64_t cls_off[4], cls_cnt[4];
-};
+static_assert(sizeof(resident::Out) <= 64 && sizeof(resident::Ctl) <= 64, "resident buffers");
 
-struct SmallOut {
-  int32_t iters, restarts, first_pass, status, zero_rhs, pad;
-  double rel_true, rel_rec, floor;
-};
-
-// Sum of NV values over the block; every thread receives the totals. red: NV * 32 + NV doubles.
-// FP64 adds are what the reduction costs on this GPU (its FP64 pipe runs at 1/64 of FP32): the
-// warps' partials are added by one thread per value, in warp order (deterministic), and the
-// totals are read back from shared memory, rather than every thread adding them again.
-template <int NV>
-__device__ __forceinline__ void small_sum(double (&v)[NV], double* red) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    double t = warp_sum(v[i]);
-    if (lane == 0) red[i * 32 + wid] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    double t = 0.0;
-    for (int wv = 0; wv < nw; ++wv) t += red[threadIdx.x * 32 + wv];
-    red[NV * 32 + threadIdx.x] = t;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = red[NV * 32 + i];
-  __syncthreads();
-}
-
-template <int MASKC>
-__device__ __forceinline__ double small_row(const Geom& g, const double* __restrict__ val, const double* x,
-                                            const uint16_t* __restrict__ keep, int row) {
-  const int col = row / g.nz, k = row - col * g.nz;
-  bool d = false;
-  return MASKC >= 0 ? row_dot_keep(g, val, x, keep, row, col, k) : row_dot<MASKC>(g, val, x, row, col, k, d);
-}
-
-// z = P^{-1} r for the whole system; leaves (r, z), m'z and 1'r in v (block totals).
-template <int PREC>
-__device__ __forceinline__ void small_precond(const Geom& g, const SmallArgs& a, const double* r, double* z,
-                                              double (&v)[3], double* red) {
-  const int n = (int)g.n, T = blockDim.x, tid = threadIdx.x;
-  if (PREC == PM_PREC_IC0) {
-#define PM_SMALL_PHASE(C, FW)                                                                            \
-  {                                                                                                      \
-    const int64_t tot = a.cls_cnt[(C) & 3] * a.cm.nlev[(C) >> 2];                                        \
-    for (int64_t t = tid; t < tot; t += T) ic0_row<C, FW>(g, a.cm, a.cls_cols, a.cls_off[(C) & 3], t, a.Fic, r, z); \
-    __syncthreads();                                                                                     \
-  }
-    PM_SMALL_PHASE(0, 1) PM_SMALL_PHASE(1, 1) PM_SMALL_PHASE(2, 1) PM_SMALL_PHASE(3, 1)
-    PM_SMALL_PHASE(4, 1) PM_SMALL_PHASE(5, 1) PM_SMALL_PHASE(6, 1) PM_SMALL_PHASE(7, 1)
-    PM_SMALL_PHASE(7, 0) PM_SMALL_PHASE(6, 0) PM_SMALL_PHASE(5, 0) PM_SMALL_PHASE(4, 0)
-    PM_SMALL_PHASE(3, 0) PM_SMALL_PHASE(2, 0) PM_SMALL_PHASE(1, 0) PM_SMALL_PHASE(0, 0)
-#undef PM_SMALL_PHASE
-  } else if (PREC == PM_PREC_LINE) {
-    const int nz = g.nz, ncols = g.ncols;
-    for (int col = tid; col < ncols; col += T) {
-      double y = 0.0;
-      for (int k = 0; k < nz; ++k) {
-        const int li = k * ncols + col;
-        y = (r[col * nz + k] - a.Fl[li] * y) * a.Fl[n + li];
-        z[col * nz + k] = y;
-      }
-      double zn = y;
-      for (int k = nz - 2; k >= 0; --k) {
-        const int li = k * ncols + col;
-        zn = fma(-a.Fl[2 * n + li], zn, z[col * nz + k]);
-        z[col * nz + k] = zn;
-      }
-    }
-    __syncthreads();
-  } else {
-    for (int i = tid; i < n; i += T) z[i] = PREC == PM_PREC_NONE ? r[i] : a.dinv[i] * r[i];
-    __syncthreads();
-  }
-  v[0] = v[1] = v[2] = 0.0;
-  for (int i = tid; i < n; i += T) {
-    const double zi = z[i], ri = r[i];
-    v[0] = fma(ri, zi, v[0]);
-    if (a.proj) {
-      v[1] = fma(a.m[i], zi, v[1]);
-      v[2] += ri;
-    }
-  }
-  small_sum<3>(v, red);
-}
-
-template <int MASKC, int PREC>
-__global__ void __launch_bounds__(SMALL_TPB, 1) k_small_pcg(Geom g, const double* __restrict__ val,
-                                                           const double* __restrict__ b, double* x, double* r,
-                                                           double* p, double* w, double* z, double* bw,
-                                                           SmallArgs a, SmallOut* out) {
-  __shared__ double red[3 * 32 + 3];
-  const int n = (int)g.n, T = blockDim.x, tid = threadIdx.x;
-  // right-hand side and initial guess (pressure: b - (1'b / 1'm) m, x shifted to m'x = 0)
-  double v[3] = {0.0, 0.0, 0.0};
-  if (a.proj) {
-    for (int i = tid; i < n; i += T) {
-      v[0] += b[i];
-      if (a.x0_is_guess) v[1] = fma(a.m[i], x[i], v[1]);
-    }
-    small_sum<3>(v, red);
-  }
-  const double lam = a.proj ? v[0] / a.one_m : 0.0, xs = a.proj && a.x0_is_guess ? v[1] / a.one_m : 0.0;
-  const double* bb_ = b;
-  for (int i = tid; i < n; i += T) {
-    if (a.proj) bw[i] = b[i] - lam * a.m[i];
-    x[i] = a.x0_is_guess ? x[i] - xs : 0.0;
-  }
-  if (a.proj) bb_ = bw;
-  __syncthreads();
-  // r = b - A x (compensated), ||b||^2, ||r||^2
-  v[0] = v[1] = v[2] = 0.0;
-  for (int i = tid; i < n; i += T) {
-    const int col = i / g.nz, k = i - col * g.nz;
-    double asum;
-    const double bi = bb_[i];
-    const double ri = row_residual_dot2<MASKC>(g, val, x, bi, i, col, k, asum);
-    r[i] = ri;
-    v[0] = fma(bi, bi, v[0]);
-    v[1] = fma(ri, ri, v[1]);
-  }
-  small_sum<3>(v, red);
-  const double bb = v[0], tol2 = a.rtol * a.rtol * bb;
-  double rr = v[1];
-  int iter = 0, restarts = 0, first_pass = -1, status = PM_OK;
-  double rel_true = 0.0, floor = 0.0, prev_true = -1.0;
-  bool accepted = false;
-  // as pcg_run: x0 may already meet rtol (no iteration), max_iter = 0 allows none
-  bool skip = rr <= tol2;
-  if (!skip && a.max_iter == 0) status = PM_NOT_CONVERGED;
-  if (bb == 0.0) {
-    for (int i = tid; i < n; i += T) x[i] = 0.0;
-  }
-  while (bb != 0.0) {
-    if (status == PM_OK && !skip) {
-      // z = P^{-1} r, rho = (r, z'), p = z' (z' = z - c 1, c = m'z / 1'm for the pressure)
-      small_precond<PREC>(g, a, r, z, v, red);
-      double c = a.proj ? v[1] / a.one_m : 0.0;
-      double rho = v[0] - c * v[2];
-      if (!(rho > 0.0) || !isfinite(rho)) status = PM_BREAKDOWN;
-      for (int i = tid; i < n; i += T) p[i] = z[i] - c;
-      __syncthreads();
-      bool converged = false;
-      while (status == PM_OK && iter < a.max_iter) {
-        // w = A p, (p, w)
-        double pw[1] = {0.0};
-        for (int i = tid; i < n; i += T) {
-          const double wi = small_row<MASKC>(g, val, p, a.keep, i);
-          w[i] = wi;
-          pw[0] = fma(p[i], wi, pw[0]);
-        }
-        small_sum<1>(pw, red);
-        if (!(pw[0] > 0.0) || !isfinite(pw[0])) {
-          status = PM_BREAKDOWN;
-          break;
-        }
-        const double alpha = rho / pw[0];
-        double rv[1] = {0.0};
-        for (int i = tid; i < n; i += T) {
-          x[i] = fma(alpha, p[i], x[i]);
-          const double ri = fma(-alpha, w[i], r[i]);
-          r[i] = ri;
-          rv[0] = fma(ri, ri, rv[0]);
-        }
-        small_sum<1>(rv, red);
-        rr = rv[0];
-        ++iter;
-        if (rr <= tol2) {
-          converged = true;
-          break;
-        }
-        if (iter >= a.max_iter) break;
-        small_precond<PREC>(g, a, r, z, v, red);
-        c = a.proj ? v[1] / a.one_m : 0.0;
-        const double rho_new = v[0] - c * v[2];
-        if (!(rho_new > 0.0) || !isfinite(rho_new)) {
-          status = PM_BREAKDOWN;
-          break;
-        }
-        const double beta = rho_new / rho;
-        rho = rho_new;
-        for (int i = tid; i < n; i += T) p[i] = fma(beta, p[i], z[i] - c);
-        __syncthreads();
-      }
-      if (status == PM_OK && !converged) status = PM_NOT_CONVERGED;   // iteration cap
-    }
-    skip = false;
-    if (first_pass < 0) first_pass = iter;
-    // true residual, compensated (into r, the restart's starting residual), and the acceptance
-    // rule of pcg_run
-    v[0] = v[1] = v[2] = 0.0;
-    for (int i = tid; i < n; i += T) {
-      const int col = i / g.nz, k = i - col * g.nz;
-      double asum;
-      const double bi = bb_[i];
-      const double ri = row_residual_dot2<MASKC>(g, val, x, bi, i, col, k, asum);
-      r[i] = ri;
-      v[0] = fma(ri, ri, v[0]);
-      const double f = asum + fabs(bi);
-      v[1] = fma(f, f, v[1]);
-    }
-    small_sum<3>(v, red);
-    rel_true = sqrt(v[0] / bb);
-    floor = ldexp(1.0, -53) * sqrt(v[1] / bb);
-    const bool stalled = prev_true >= 0.0 && rel_true > 0.5 * prev_true;
-    const bool last = restarts >= a.max_restarts || iter >= a.max_iter;
-    accepted = rel_true <= a.rtol || (rel_true <= floor && (stalled || last));
-    if (status != PM_OK || accepted || last) break;
-    prev_true = rel_true;
-    ++restarts;
-  }
-  if (bb != 0.0 && status == PM_OK && !accepted) status = PM_NOT_CONVERGED;
-  if (a.proj) {   // the returned pressure has m'x = 0
-    __syncthreads();
-    v[0] = v[1] = v[2] = 0.0;
-    for (int i = tid; i < n; i += T) v[0] = fma(a.m[i], x[i], v[0]);
-    small_sum<3>(v, red);
-    const double sh = v[0] / a.one_m;
-    for (int i = tid; i < n; i += T) x[i] -= sh;
-  }
-  if (tid == 0) {
-    out->iters = iter;
-    out->restarts = restarts;
-    out->first_pass = first_pass < 0 ? iter : first_pass;
-    out->status = status;
-    out->zero_rhs = bb == 0.0;
-    out->rel_true = bb == 0.0 ? 0.0 : rel_true;
-    out->rel_rec = bb == 0.0 ? 0.0 : sqrt(rr / bb);
-    out->floor = floor;
-  }
-}
-
-static_assert(sizeof(SmallOut) <= 64, "SmallOut buffer");
-
-template <int MASKC>
-int small_run(pm_operator* op, int which, const double* b, double* x, const pm_solve_opts* o,
-              pm_solve_stats* stats, cudaStream_t s) {
-  auto t0 = std::chrono::steady_clock::now();
-  SolveCtx* c = op->ctx;
-  const bool proj = which == PM_OP_PRESSURE;
-  const int prec = o->prec;
+// Preconditioner data a solve reads: Jacobi diagonal, line or IC0 factor.
+int ensure_prec(pm_operator* op, int which, int prec, cudaStream_t s) {
   int st;
   if ((st = launch_dinv(op, which, s))) return st;
   if (prec == PM_PREC_IC0 && !op->ic0[which].ok) {
@@ -1586,61 +1334,46 @@ int small_run(pm_operator* op, int which, const double* b, double* x, const pm_s
     }
     if (bd) return set_error(PM_BREAKDOWN, "IC0 pivot failure after the shift limit");
   }
-  if (prec == PM_PREC_LINE && (st = line_factor(op, which, s))) return st;
-  SmallArgs a;
+  return prec == PM_PREC_LINE ? line_factor(op, which, s) : PM_OK;
+}
+
+// The operands of a resident solve that do not depend on its precision.
+resident::Args resident_args(pm_operator* op, int which, const double* b, double* x, const pm_solve_opts* o) {
+  SolveCtx* c = op->ctx;
+  resident::Args a;
   std::memset(&a, 0, sizeof(a));
-  a.rtol = o->rtol;
-  a.one_m = op->one_m;
-  a.max_iter = o->max_iter;
-  a.max_restarts = o->max_restarts;
-  a.x0_is_guess = o->x0_is_guess ? 1 : 0;
-  a.proj = proj ? 1 : 0;
-  a.dinv = op->d_dinv[which];
-  a.keep = MASKC >= 0 ? op->d_keep[MASKC < 0 ? 0 : MASKC] : nullptr;
+  const int mc = which_mask(which);
+  a.g = geom_of(op);
+  a.val64 = op->d_val[which_valset(which)];
+  a.mask = mc >= 0 ? op->d_keep[mc] : op->d_struct;
+  a.b = b;
+  a.x = x;
+  a.bw = c->bw;
   a.m = op->d_m;
-  a.Fic = op->ic0[which].F;
-  a.Fl = op->d_line[which];
-  a.cls_cols = op->d_cls_cols;
-  a.cm = cmap_of(op);
-  int64_t off = 0;
-  for (int q = 0; q < 4; ++q) {
+  a.cnbr = op->d_cnbr;
+  a.clsidx = op->d_cls_cols + op->ncols;
+  a.coli = a.clsidx + op->ncols;
+  a.colj = a.coli + op->ncols;
+  const CMap cm = cmap_of(op);
+  for (int q = 0, off = 0; q < 4; ++q) {
     a.cls_off[q] = off;
     a.cls_cnt[q] = op->cls_count[q];
     off += op->cls_count[q];
   }
-  Geom g = geom_of(op);
-  const double* val = op->d_val[which_valset(which)];
-  SmallOut* dout = static_cast<SmallOut*>(c->small_out);
-#define PM_SMALL(P) k_small_pcg<MASKC, P><<<1, SMALL_TPB, 0, s>>>(g, val, b, x, c->r, c->p, c->w, c->z, c->bw, a, dout)
-  switch (prec) {
-    case PM_PREC_IC0: PM_SMALL(PM_PREC_IC0); break;
-    case PM_PREC_LINE: PM_SMALL(PM_PREC_LINE); break;
-    case PM_PREC_NONE: PM_SMALL(PM_PREC_NONE); break;
-    default: PM_SMALL(PM_PREC_JACOBI); break;
-  }
-#undef PM_SMALL
-  count_launch();
-  if ((st = cuda_check(cudaGetLastError(), "k_small_pcg"))) return st;
-  if ((st = cuda_check(cudaMemcpyAsync(c->small_out_host, c->small_out, sizeof(SmallOut), cudaMemcpyDeviceToHost, s),
-                       "small stats")))
-    return st;
-  if ((st = cuda_check(cudaStreamSynchronize(s), "small pcg"))) return st;
-  const SmallOut& h = *static_cast<const SmallOut*>(c->small_out_host);
-  if (stats) {
-    stats->iters = h.iters;
-    stats->outer_iters = h.restarts;
-    stats->first_pass_iters = h.first_pass;
-    stats->status = h.status;
-    stats->rel_residual_true = h.rel_true;
-    stats->rel_residual_rec = h.rel_rec;
-    stats->rel_residual_floor = h.floor;
-    stats->bytes_moved = h.iters * bytes_per_iter(op, prec, proj);
-    stats->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-  }
-  if (h.status != PM_OK)
-    return set_error(h.status, h.status == PM_NOT_CONVERGED ? "PCG did not reach rtol within max_iter"
-                                                            : "PCG breakdown: (p, Ap) <= 0 or non-finite");
-  return PM_OK;
+  for (int q = 0; q < 8; ++q) a.cbase[q] = (int32_t)cm.cbase[q];
+  a.nlev[0] = fast_div(cm.nlev[0]);
+  a.nlev[1] = fast_div(cm.nlev[1]);
+  a.rtol = o->rtol;
+  a.inner_rtol = o->inner_rtol > 0.0 ? o->inner_rtol : 1e-2;
+  a.one_m = op->one_m;
+  a.max_iter = o->max_iter;
+  a.max_restarts = o->max_restarts;
+  a.x0_is_guess = o->x0_is_guess ? 1 : 0;
+  a.proj = which == PM_OP_PRESSURE ? 1 : 0;
+  a.ctl = static_cast<resident::Ctl*>(c->res_ctl);
+  a.part = c->partials;
+  a.out = static_cast<resident::Out*>(c->res_out);
+  return a;
 }
 
 // ---- mixed precision: FP32 / BF16 operator values, FP32 inner PCG, FP64 outer refinement -------
@@ -2290,6 +2023,83 @@ double bytes_per_inner(const pm_operator* op, int prec, int vbytes, bool proj) {
   return b;
 }
 
+// FP64 residual, and the fold of the correction into x, of one refinement step.
+double bytes_per_refine(const pm_operator* op) { return (double)op->n * (15 * 8 + 3 * 8 + 16 + 8); }
+
+// Whether the automatic choice runs a solve resident. Measured against the stream of kernels, us per
+// iteration, stream / resident:
+//   FP64  IC0 n = 0.12M 218 / 52, 0.29M 239 / 63, 0.99M 343 / 150, 2.0M 390 / 270, 4.9M 611 / 576;
+//         line 0.31M 64 / 35, 1.0M 110 / 88, 1.8M 152 / 130, 4.7M 319 / 327;
+//         Jacobi 2.0M 140 / 126, 5.1M 275 / 296
+//   FP32  IC0 0.12M 226 / 46, 2.0M 360 / 195, 4.9M 472 / 427 (BF16 values 0.85M 296 / 98);
+//         line 0.31M 66 / 27, 1.0M 69 / 67, 1.8M 93 / 98; Jacobi 0.31M 73 / 21, 5.1M 196 / 201.
+bool resident_auto(const pm_operator* op, int prec, bool mixed) {
+  return op->n <= (mixed && prec == PM_PREC_LINE ? RESIDENT_AUTO_MIXED_LINE : RESIDENT_AUTO_ROWS);
+}
+
+int resident_run(pm_operator* op, int which, const double* b, double* x, const pm_solve_opts* o,
+                 pm_solve_stats* stats, cudaStream_t s) {
+  auto t0 = std::chrono::steady_clock::now();
+  SolveCtx* c = op->ctx;
+  const int prec = o->prec;
+  const bool mixed = o->precision != PM_FP64;
+  int st;
+  if ((st = ensure_prec(op, which, prec, s))) return st;
+  if (mixed && (st = ensure_mixed(op, which, o->precision, prec, s))) return st;
+  resident::Args a = resident_args(op, which, b, x, o);
+  const int vs = which_valset(which);
+  const bool cluster = op->n <= (prec == PM_PREC_IC0 ? RESIDENT_CLUSTER_IC0 : RESIDENT_CLUSTER_ROWS);
+  a.out->status = -1;
+  if (mixed) {
+    a.val = o->precision == PM_FP32_REFINE ? (const void*)op->d_val32[vs] : (const void*)op->d_val16[vs];
+    a.r = c->r32;
+    a.p = c->p32;
+    a.w = c->w32;
+    a.z = c->z32;
+    a.d = c->d32;
+    a.m2 = op->d_m2f;
+    a.dinv = prec == PM_PREC_NONE ? nullptr : op->d_dinv32[which];
+    a.ic0 = op->d_ic0_32[which];
+    a.line = op->d_line32[which];
+    st = o->precision == PM_FP32_REFINE ? resident::launch_fp32(a, prec, cluster, op->num_sms, s)
+                                        : resident::launch_bf16(a, prec, cluster, op->num_sms, s);
+  } else {
+    a.val = a.val64;
+    a.r = c->r;
+    a.p = c->p;
+    a.w = c->w;
+    a.z = c->z;
+    a.dinv = prec == PM_PREC_NONE ? nullptr : op->d_dinv[which];
+    a.ic0 = op->ic0[which].F;
+    a.line = op->d_line[which];
+    st = resident::launch_fp64(a, prec, cluster, op->num_sms, s);
+  }
+  if (st) return st;
+  if ((st = cuda_check(cudaStreamSynchronize(s), "resident pcg"))) return st;
+  const resident::Out h = *a.out;
+  if (h.status == PM_TIMEOUT) return set_error(PM_TIMEOUT, "resident PCG: a grid barrier wait ran out");
+  if (h.status < 0) return set_error(PM_ECUDA, "resident PCG: the kernel reported nothing");
+  if (stats) {
+    stats->iters = h.iters;
+    stats->outer_iters = h.restarts;
+    stats->first_pass_iters = h.first_pass;
+    stats->status = h.status;
+    stats->rel_residual_true = h.rel_true;
+    stats->rel_residual_rec = h.rel_rec;
+    stats->rel_residual_floor = h.floor;
+    stats->bytes_moved = mixed ? h.iters * bytes_per_inner(op, prec, o->precision == PM_FP32_REFINE ? 4 : 2, a.proj) +
+                                     h.restarts * bytes_per_refine(op)
+                               : h.iters * bytes_per_iter(op, prec, a.proj);
+    stats->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+  }
+  if (h.status != PM_OK)
+    return set_error(h.status, h.status == PM_NOT_CONVERGED
+                                   ? mixed ? "mixed-precision PCG did not reach rtol" : "PCG did not reach rtol within max_iter"
+                               : mixed ? "mixed-precision PCG breakdown"
+                                       : "PCG breakdown: (p, Ap) <= 0 or non-finite");
+  return PM_OK;
+}
+
 template <int MASKC, typename TV>
 void inner_iter(pm_operator* op, int which, const TV* val32, bool proj, int prec, const float* dinv32,
                 cudaStream_t s) {
@@ -2370,16 +2180,7 @@ int mixed_run(pm_operator* op, int which, const double* b, double* x, const pm_s
   const int prec = o->prec;
   const double* val64 = op->d_val[which_valset(which)];
   int st;
-  if ((st = launch_dinv(op, which, s))) return st;
-  if (prec == PM_PREC_IC0 && !op->ic0[which].ok) {
-    int bd = 0;
-    for (int m = -1; m <= 10; ++m) {
-      if ((st = launch_ic0_factor(op, which, m < 0 ? 0.0 : 1e-3 * std::pow(2.0, m), &bd, s))) return st;
-      if (!bd) break;
-    }
-    if (bd) return set_error(PM_BREAKDOWN, "IC0 pivot failure after the shift limit");
-  }
-  if (prec == PM_PREC_LINE && (st = line_factor(op, which, s))) return st;
+  if ((st = ensure_prec(op, which, prec, s))) return st;
   if ((st = ensure_mixed(op, which, o->precision, prec, s))) return st;
   const int vs = which_valset(which);
   const TV* val32 = std::is_same<TV, float>::value ? reinterpret_cast<const TV*>(op->d_val32[vs])
@@ -2459,7 +2260,7 @@ int mixed_run(pm_operator* op, int which, const double* b, double* x, const pm_s
       launch_residual<MASKC>(op, val64, bw, x, o->rtol, 1, s);
       if ((st = read_scalars(c, s))) return st;
       ++outer;
-      bytes += (double)op->n * (15 * 8 + 3 * 8 + 16 + 8);   // FP64 residual; the fold of d into x
+      bytes += bytes_per_refine(op);
       rel_true = std::sqrt(c->sc_host->aux[0] / bb);
       rel_floor = std::ldexp(1.0, -53) * std::sqrt(c->sc_host->aux[1] / bb);
       // the refinement step did not halve the (compensated) true residual
@@ -2599,6 +2400,12 @@ int pcg_solve(pm_operator* op, int which, const double* b, double* x, const pm_s
   NvtxRange range(std::string("pcg ") + which_name(which) + " " + prec_name(o->prec) + " " + precision_name(o->precision));
   int r = ensure_ctx(op);
   if (r) return r;
+  // the kernel choice (and its limit) is of FP64 solves; a mixed-precision one runs as AUTO
+  const bool mixed = o->precision != PM_FP64;
+  if (!mixed && o->kernel == PM_KERNEL_RESIDENT && op->n > RESIDENT_MAX_ROWS)
+    return set_error(PM_EINVAL, "PM_KERNEL_RESIDENT: at most " + std::to_string(RESIDENT_MAX_ROWS) + " rows");
+  if (!mixed && o->kernel != PM_KERNEL_AUTO ? o->kernel == PM_KERNEL_RESIDENT : resident_auto(op, o->prec, mixed))
+    return resident_run(op, which, b, x, o, st, s);
   if (o->precision == PM_FP32_REFINE) {
     switch (which_mask(which)) {
       case 0: return mixed_run<0, float>(op, which, b, x, o, st, s);
@@ -2615,17 +2422,6 @@ int pcg_solve(pm_operator* op, int which, const double* b, double* x, const pm_s
       default: return mixed_run<-1, __nv_bfloat16>(op, which, b, x, o, st, s);
     }
   }
-  const bool resident = o->kernel == PM_KERNEL_RESIDENT || (o->kernel == PM_KERNEL_AUTO && op->n <= SMALL_AUTO_ROWS);
-  if (resident) {
-    if (op->n > SMALL_MAX_ROWS)
-      return set_error(PM_EINVAL, "PM_KERNEL_RESIDENT: at most " + std::to_string(SMALL_MAX_ROWS) + " rows");
-    switch (which_mask(which)) {
-      case 0: return small_run<0>(op, which, b, x, o, st, s);
-      case 1: return small_run<1>(op, which, b, x, o, st, s);
-      case 2: return small_run<2>(op, which, b, x, o, st, s);
-      default: return small_run<-1>(op, which, b, x, o, st, s);
-    }
-  }
   switch (which_mask(which)) {
     case 0: return pcg_run<0>(op, which, b, x, o, st, s);
     case 1: return pcg_run<1>(op, which, b, x, o, st, s);
@@ -2639,16 +2435,7 @@ int pcg_solve(pm_operator* op, int which, const double* b, double* x, const pm_s
 int prepare_for_batch(pm_operator* op, int which, int prec, int precision, cudaStream_t s) {
   int st = ensure_ctx(op);
   if (st) return st;
-  if ((st = launch_dinv(op, which, s))) return st;
-  if (prec == PM_PREC_LINE && (st = line_factor(op, which, s))) return st;
-  if (prec == PM_PREC_IC0 && !op->ic0[which].ok) {
-    int bd = 0;
-    for (int m = -1; m <= 10; ++m) {
-      if ((st = launch_ic0_factor(op, which, m < 0 ? 0.0 : 1e-3 * std::pow(2.0, m), &bd, s))) return st;
-      if (!bd) break;
-    }
-    if (bd) return set_error(PM_BREAKDOWN, "IC0 pivot failure after the shift limit");
-  }
+  if ((st = ensure_prec(op, which, prec, s))) return st;
   if (precision != PM_FP64 && (st = ensure_mixed(op, which, precision, prec, s))) return st;
   return PM_OK;
 }
@@ -2701,8 +2488,8 @@ void destroy_ctx(pm_operator* op) {
   cudaFree(c->d32);
   cudaFree(c->sc_in);
   if (c->sc_in_host) cudaFreeHost(c->sc_in_host);
-  cudaFree(c->small_out);
-  if (c->small_out_host) cudaFreeHost(c->small_out_host);
+  cudaFree(c->res_ctl);
+  if (c->res_out) cudaFreeHost(c->res_out);
   delete c;
   op->ctx = nullptr;
 }
