@@ -207,13 +207,12 @@ int pm_pcg_solve(pm_operator* op, pm_which which, const double* b, double* x,
  * owned by a framework allocator or a fixed pool (an allocation behind the pool's back escapes its
  * accounting, or fails against its reservation), and embedded users that must not grow the device
  * footprint after start-up.
- * All scratch (Krylov vectors, Jacobi diagonal, reduction partials, device scalars) lives in one
+ * All scratch (Krylov vectors, Jacobi diagonal, block sums, barrier, results) lives in one
  * static device array of PM_NOALLOC_MAX_ROWS rows (about 21 MB), held by every GPU that loads the
  * library until the process exits; no cudaMalloc, cudaFree or other allocating routine is called.
  * Errors: PM_EINVAL for systems with more than PM_NOALLOC_MAX_ROWS rows, another preconditioner
  * or precision, an operator that lives on a device other than the current one, or a stream that
- * is being captured (the call reads scalars back and synchronises the stream every few
- * iterations). The first call on a device looks up the array's address (cudaGetSymbolAddress)
+ * is being captured (the call reads its results back and synchronises the stream). The first call on a device looks up the array's address (cudaGetSymbolAddress)
  * with that device current. Every call shares the one array and re-initialises what must start
  * at zero; calls that overlap on the GPU (other streams or threads) race. max_iter = 0 runs no
  * iteration (PM_NOT_CONVERGED unless x already meets rtol). The operator itself must already be
