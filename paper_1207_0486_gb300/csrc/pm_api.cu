@@ -138,7 +138,7 @@ int64_t pm_operator_bytes(const pm_mesh_desc* d) {
   b += 3 * (int64_t)NSLOT * np * 4;            // FP32 copies of the solved operators (mixed precision)
   b += 3 * (int64_t)NSLOT * n * 8;             // IC0 factors of the three BDF2 velocity systems
   b += 4 * n * 12;                             // Jacobi diagonals
-  b += n * (8 + 2 + 3 * 2) + ncols * (14 * 4 + 8 + 8 + 2 + 16);   // m, structure, keep masks; columns
+  b += n * (8 + 2 + 3 * 2) + ncols * (23 * 4 + 8 + 8 + 2 + 16);   // m, structure, keep masks; columns
   b += 5 * n * 8 + (int64_t)NPART * MAX_GRID * 8;   // PCG workspace
   return b;
 }
@@ -183,14 +183,30 @@ int pm_assemble_operator(const pm_mesh_desc* mesh, const pm_physics* phys, pm_op
       }
   const int nc = hm.ncols;
   std::vector<int32_t> packed;
-  packed.reserve((size_t)(4 + NNBR) * nc);
+  packed.reserve((size_t)(6 + 2 * NNBR) * nc);
   packed.insert(packed.end(), cls_cols.begin(), cls_cols.end());
   packed.insert(packed.end(), clsidx.begin(), clsidx.end());
   packed.insert(packed.end(), hm.col_i.begin(), hm.col_i.end());
   packed.insert(packed.end(), hm.col_j.begin(), hm.col_j.end());
-  // neighbour columns in class order, entry by entry
+  // neighbour columns in class order, entry by entry; the same by their index within their own class
+  // (-1: none); first colour-ordered position of each column's even and odd levels
   for (int q = 0; q < NNBR; ++q)
     for (int i = 0; i < nc; ++i) packed.push_back(q == 0 ? cls_cols[i] : hm.nbr[(size_t)cls_cols[i] * NNBR + q]);
+  for (int q = 0; q < NNBR; ++q)
+    for (int i = 0; i < nc; ++i) {
+      const int nb = packed[(size_t)(4 + q) * nc + i];
+      packed.push_back(nb < 0 ? -1 : clsidx[nb]);
+    }
+  const int nlev[2] = {(mesh->nz + 1) / 2, mesh->nz / 2};
+  for (int par = 0; par < 2; ++par) {
+    int64_t base[4], acc = par ? (int64_t)nc * nlev[0] : 0;
+    for (int cls = 0; cls < 4; ++cls) {
+      base[cls] = acc;
+      acc += (int64_t)op->cls_count[cls] * nlev[par];
+    }
+    for (int c = 0; c < nc; ++c)
+      packed.push_back((int32_t)(base[(hm.col_i[c] & 1) | ((hm.col_j[c] & 1) << 1)] + (int64_t)clsidx[c] * nlev[par]));
+  }
 #define PM_TRY(x)           \
   do {                      \
     int _e = (x);           \
@@ -204,8 +220,10 @@ int pm_assemble_operator(const pm_mesh_desc* mesh, const pm_physics* phys, pm_op
   PM_TRY(dalloc(op, &op->d_cellmask, (size_t)nc));
   PM_TRY(dalloc(op, &op->d_colflag, (size_t)nc));
   PM_TRY(dalloc(op, &op->d_coriolis, (size_t)nc));
-  PM_TRY(dalloc(op, &op->d_cls_cols, (size_t)(4 + NNBR) * nc));
+  PM_TRY(dalloc(op, &op->d_cls_cols, (size_t)(6 + 2 * NNBR) * nc));
   op->d_cnbr = op->d_cls_cols + (size_t)4 * nc;
+  op->d_ccls = op->d_cnbr + (size_t)NNBR * nc;
+  op->d_colpos = op->d_ccls + (size_t)NNBR * nc;
   PM_TRY(dalloc(op, &op->d_struct, (size_t)op->n));
   PM_TRY(dalloc(op, &op->d_m, (size_t)op->n));
   for (int v = 0; v < VS_COUNT; ++v) PM_TRY(dalloc(op, &op->d_val[v], (size_t)NSLOT * op->npad));

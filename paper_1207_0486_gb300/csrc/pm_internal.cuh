@@ -346,6 +346,8 @@ struct pm_operator {
                                     // class, i and j of each column, [ncols] each
   int32_t* d_cnbr = nullptr;        // [7][ncols]: neighbour columns of the i-th column in class order
                                     // (entry 0: that column itself); part of d_cls_cols' allocation
+  int32_t* d_ccls = nullptr;        // [7][ncols]: the same neighbours by their index within their class
+  int32_t* d_colpos = nullptr;      // [2][ncols]: first colour-ordered position of a column's even / odd levels
   uint16_t* d_struct = nullptr;     // structural slot bits per row
   uint16_t* d_keep[3] = {};         // per velocity component: bit s = slot s kept (neighbour present and
                                     // not in the component's Dirichlet set), bit 15 = Dirichlet row

@@ -11,7 +11,7 @@
 //   K3 k_cg_pupd   : p = z + beta p
 // This file's kernels run one phase each over the whole GPU (PM_KERNEL_STREAM, and large systems);
 // below resident_auto's lines one launch runs the whole solve (pm_resident.cuh).
-// IC0 replaces the inline z by 8 forward and 8 backward colour sweeps plus a (r, z) reduction.
+// IC0 replaces the inline z by 8 forward and 7 backward colour sweeps, with (r, z) = (y, y) between them.
 // Grid reductions are deterministic: each block reduces its rows in a fixed tree, writes one
 // partial, and the last block to arrive (atomic ticket) sums the partials in block order.
 // All scalars (alpha, beta, rho, status) stay on the device; the host reads one small struct
@@ -329,17 +329,15 @@ __global__ void __launch_bounds__(TPB) k_cg_residual(Geom g, const double* __res
   }
 }
 
-// First preconditioned residual (Jacobi or stored z): rho = (r, z') with z' = z - c 1,
-// c = m'z / 1'm for the pressure (PROJ), p = z'. STORED: z read from zbuf.
-template <int PROJ, int STORED>
+// First preconditioned residual (Jacobi): rho = (r, z') with z' = z - c 1,
+// c = m'z / 1'm for the pressure (PROJ), p = z'; beta = 0.
+template <int PROJ>
 __global__ void __launch_bounds__(TPB) k_cg_rho(int64_t n, const double* __restrict__ r, const double* __restrict__ dinv,
-                                                const double* __restrict__ zbuf, const double* __restrict__ m,
-                                                double* partials, PcgScalars* sc, int is_first) {
-  if (!is_first && sc_done(sc)) return;
+                                                const double* __restrict__ m, double* partials, PcgScalars* sc) {
   double v[3] = {0.0, 0.0, 0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double ri = r[i];
-    const double zi = STORED ? zbuf[i] : dinv[i] * ri;
+    const double zi = dinv[i] * ri;
     v[0] = fma(ri, zi, v[0]);
     if (PROJ) {
       v[1] = fma(m[i], zi, v[1]);
@@ -350,18 +348,11 @@ __global__ void __launch_bounds__(TPB) k_cg_rho(int64_t n, const double* __restr
     const double c = PROJ ? v[1] / sc->one_m : 0.0;
     const double rho_new = v[0] - c * v[2];
     sc->proj_c = c;
-    if (is_first) {
-      sc->rho = rho_new;
-      sc->beta = 0.0;
-    } else {
-      sc->beta = rho_new / sc->rho;
-      sc->rho = rho_new;
-    }
-    if (!(rho_new > 0.0) || !isfinite(rho_new)) {
-      if (!sc->done) {
-        sc->status = PM_BREAKDOWN;
-        sc->done = 1;
-      }
+    sc->rho = rho_new;
+    sc->beta = 0.0;
+    if ((!(rho_new > 0.0) || !isfinite(rho_new)) && !sc->done) {
+      sc->status = PM_BREAKDOWN;
+      sc->done = 1;
     }
   }
 }
@@ -457,72 +448,147 @@ __global__ void __launch_bounds__(TPB) k_cg_update(int64_t n, double* __restrict
 }
 
 // ---- IC0 colour sweeps -------------------------------------------------------------------------
-struct CMap {
-  int64_t cbase[8];
-  int32_t nlev[2];
+// The sweeps' work vector y (then z) is kept in colour order, the order of the factor's rows: position
+// cbase[colour] + (index of the column in its parity class) * levels + level / 2. A colour's rows are every
+// other level of their columns, so in the natural order each gathered or stored sector would be half
+// used; in colour order a warp's accesses to every neighbour are runs. The neighbours' class indices
+// come from a table in class order (d_ccls), one load each. Before (natural order, 64-bit index
+// divisions, two dependent index loads per neighbour): 23.8 us per colour phase at 4.9M rows, now 18.9.
+struct SweepGeo {
+  int32_t n, nz, ncols;
+  const int32_t* cnbr;
+  const int32_t* ccls;
+  const int32_t* colpos;
+  int32_t cbase[8], cls_off[4], cls_cnt[4];
+  FastDiv nlev[2], nzd;
 };
 
-// Forward (FWD = 1): y_i = (r_i - sum_{colour(j) < c} L_ij y_j) / L_ii over rows of colour c.
-// Backward (FWD = 0): z_i = (y_i - sum_{colour(j) > c} L_ji z_j) / L_ii, in place on y.
-// The factor's diagonal slot holds 1 / L_ii (a multiply instead of an FP64 division).
-// Position t of colour COLOUR: column cls_cols[cls_off + t / nlev], level 2 (t % nlev) + parity.
-// ic0_value returns the row's new value and its index; ic0_row stores it.
-template <int COLOUR, int FWD, typename T>
-__device__ __forceinline__ T ic0_value(const Geom& g, const CMap& cm, const int32_t* __restrict__ cls_cols,
-                                       int64_t cls_off, int64_t t, const T* __restrict__ F,
-                                       const T* __restrict__ r, const T* y, int64_t* row_out) {
-  constexpr int kpar = COLOUR >> 2;
-  const int nlev = cm.nlev[kpar];
-  const int nz = g.nz;
-  const int col = __ldg(cls_cols + cls_off + t / nlev);
-  const int k = 2 * (int)(t % nlev) + kpar;
-  const int64_t row = (int64_t)col * nz + k;
-  const int64_t pi = cm.cbase[COLOUR] + t;
-  T acc = FWD ? r[row] : y[row];
-#pragma unroll
-  for (int s = 0; s < NSLOT; ++s) {
-    if (s == DIAG_SLOT) continue;
-    const int cj = COLOUR ^ slot_flip(s);
-    if (FWD ? (cj > COLOUR) : (cj < COLOUR)) continue;
-    const int q = slot_q(s);
-    const int kk = k + slot_dk(s);
-    if (kk < 0 || kk >= nz) continue;
-    const int nb = q == 0 ? col : nbr_of(g, col, q);
-    if (nb < 0) continue;
-    acc = fma(-F[(int64_t)s * g.n + pi], y[(int64_t)nb * nz + kk], acc);
+__device__ __forceinline__ int ccls_of(const SweepGeo& g, int i, int q) {
+  const int nb = __ldg(g.ccls + q * g.ncols + i);
+#ifdef PM_CHECKED
+  if (nb < -1 || nb >= g.ncols) {
+    record_bad_index(SITE_NBR, nb, g.ncols);
+    return -1;
   }
-  *row_out = row;
-  return acc * F[(int64_t)DIAG_SLOT * g.n + pi];
+#endif
+  return nb;
 }
 
-template <int COLOUR, int FWD>
-__device__ __forceinline__ void ic0_row(const Geom& g, const CMap& cm, const int32_t* __restrict__ cls_cols,
-                                        int64_t cls_off, int64_t t, const double* __restrict__ F,
-                                        const double* __restrict__ r, double* __restrict__ y) {
-  int64_t row;
-  const double v = ic0_value<COLOUR, FWD>(g, cm, cls_cols, cls_off, t, F, r, y, &row);
-  y[row] = v;
+// Colour-ordered position of a row in natural order.
+__device__ __forceinline__ int colour_pos(const SweepGeo& g, int row) {
+  const int col = fdiv(g.nzd, row), k = row - col * g.nz;
+  return __ldg(g.colpos + (k & 1) * g.ncols + col) + (k >> 1);
 }
 
-// One colour phase: two rows per thread (t and t + stride), both computed before either is
-// stored (no row of a colour reads another row of that colour), so that each thread has both
-// rows' neighbour gathers in flight. Launched over half the rows.
-template <int COLOUR, int FWD, typename T>
-__global__ void __launch_bounds__(TPB) k_ic0_sweep(Geom g, CMap cm, const int32_t* __restrict__ cls_cols,
-                                                   int64_t cls_off, int64_t cls_cnt, const T* __restrict__ F,
-                                                   const T* __restrict__ r, T* __restrict__ y,
-                                                   const PcgScalars* sc, int check_done) {
+// Forward (FWD = 1): y_i = (r_i - sum_{colour(j) < C} L_ij y_j) / L_ii over rows of colour C.
+// Backward (FWD = 0): z_i = (y_i - sum_{colour(j) > C} L_ji z_j) / L_ii, in place on y.
+// The factor's diagonal slot holds 1 / L_ii (a multiply instead of an FP64 division).
+// Position t of colour C: column t / nlev of its class, level 2 (t % nlev) + parity. All of a row's
+// loads but the neighbours' values are independent of one another.
+template <int C, int FWD, typename T>
+__global__ void __launch_bounds__(TPB, 4) k_ic0_sweep(SweepGeo g, const T* __restrict__ F, const T* __restrict__ r,
+                                                      T* y, const PcgScalars* sc, int check_done) {
   if (check_done && sc_done(sc)) return;
-  const int64_t total = cls_cnt * cm.nlev[COLOUR >> 2];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += 2 * stride) {
-    const bool two = t + stride < total;
-    int64_t r0, r1 = 0;
-    const T v0 = ic0_value<COLOUR, FWD>(g, cm, cls_cols, cls_off, t, F, r, y, &r0);
-    T v1 = 0;
-    if (two) v1 = ic0_value<COLOUR, FWD>(g, cm, cls_cols, cls_off, t + stride, F, r, y, &r1);
-    y[r0] = v0;
-    if (two) y[r1] = v1;
+  constexpr int kpar = C >> 2, cls = C & 3;
+  const int total = g.cls_cnt[cls] * g.nlev[kpar].d;
+  const int n = g.n;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const int i = fdiv(g.nlev[kpar], t), kk = t - i * g.nlev[kpar].d, at = g.cls_off[cls] + i, pos = g.cbase[C] + t;
+    T f[NSLOT], v[NSLOT];
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      const int cj = C ^ slot_flip(s);
+      if (s == DIAG_SLOT || (FWD ? cj < C : cj > C)) f[s] = __ldg(F + s * n + pos);
+    }
+    T acc = FWD ? r[__ldg(g.cnbr + at) * g.nz + 2 * kk + kpar] : y[pos];
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      const int cj = C ^ slot_flip(s);
+      if (s == DIAG_SLOT || !(FWD ? cj < C : cj > C)) continue;
+      const int dk = slot_dk(s), q = slot_q(s);
+      const int lv = kk + (dk == 0 ? 0 : dk > 0 ? kpar : kpar - 1);   // the neighbour's level / 2
+      const int nl = g.nlev[cj >> 2].d;
+      const int nb = q == 0 ? i : ccls_of(g, at, q);
+      const bool ok = nb >= 0 && lv >= 0 && lv < nl;
+      v[s] = ok ? y[g.cbase[cj] + nb * nl + lv] : (T)0;
+    }
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      const int cj = C ^ slot_flip(s);
+      if (s == DIAG_SLOT || !(FWD ? cj < C : cj > C)) continue;
+      acc = fma(-f[s], v[s], acc);
+    }
+    y[pos] = acc * f[DIAG_SLOT];
+  }
+}
+
+// Between the sweeps: (y, y), which is (r, z) since y = L^-1 r and z = L^-T y, and colour 7's backward rows
+// z = y / L_ii (no higher colour). FINISH: rho, beta, breakdown test, as k_cg_rho.
+template <typename T, int FINISH>
+__global__ void __launch_bounds__(TPB) k_ic0_mid(SweepGeo g, const T* __restrict__ F, T* __restrict__ y, double* partials,
+                                                 PcgScalars* sc, int is_first) {
+  if (!is_first && sc_done(sc)) return;
+  AccFor<T> a;
+  const int n = g.n, last = g.cbase[7];
+  for (int i = (FINISH ? 0 : last) + blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const T yi = y[i];
+    if (FINISH) a.add_prod(yi, yi);
+    if (i >= last) y[i] = yi * __ldg(F + DIAG_SLOT * n + i);
+  }
+  if (!FINISH) return;
+  double v[1] = {a.value()};
+  if (grid_sum<1>(v, partials, &sc->count[2]) && threadIdx.x == 0) {
+    sc->proj_c = 0.0;
+    sc->beta = is_first ? 0.0 : v[0] / sc->rho;
+    sc->rho = v[0];
+    if ((!(v[0] > 0.0) || !isfinite(v[0])) && !sc->done) {
+      sc->status = PM_BREAKDOWN;
+      sc->done = 1;
+    }
+  }
+}
+
+__device__ __forceinline__ void ic0_add_m(Acc64& acc, const double* m, int i, double z) { acc.add_prod(m[i], z); }
+__device__ __forceinline__ void ic0_add_m(DF& acc, const float2* m, int i, float z) {
+  acc.add_prod(m[i].x, z);
+  acc.add_prod(m[i].y, z);
+}
+
+// Pressure: rho = (r, z'), z' = z - c, c = m'z / 1'm, with z in colour order (k_cg_rho otherwise).
+template <typename T, typename TM>
+__global__ void __launch_bounds__(TPB) k_ic0_rho_proj(SweepGeo g, const T* __restrict__ r, const T* __restrict__ z,
+                                                      const TM* __restrict__ m, double* partials, PcgScalars* sc,
+                                                      int is_first) {
+  if (!is_first && sc_done(sc)) return;
+  AccFor<T> a0, a1, a2;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.n; i += gridDim.x * blockDim.x) {
+    const T ri = r[i], zi = z[colour_pos(g, i)];
+    a0.add_prod(ri, zi);
+    ic0_add_m(a1, m, i, zi);
+    a2.add(ri);
+  }
+  double v[3] = {a0.value(), a1.value(), a2.value()};
+  if (grid_sum<3>(v, partials, &sc->count[2]) && threadIdx.x == 0) {
+    const double c = v[1] / sc->one_m, rho = v[0] - c * v[2];
+    sc->proj_c = c;
+    sc->beta = is_first ? 0.0 : rho / sc->rho;
+    sc->rho = rho;
+    if ((!(rho > 0.0) || !isfinite(rho)) && !sc->done) {
+      sc->status = PM_BREAKDOWN;
+      sc->done = 1;
+    }
+  }
+}
+
+// p = (z - c) + beta p with z in colour order; FIRST step: p = z - c.
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_ic0_pupd(SweepGeo g, const T* __restrict__ z, T* __restrict__ p,
+                                                  const PcgScalars* sc, int is_first) {
+  if (!is_first && sc_done(sc)) return;
+  const T beta = (T)sc->beta, c = (T)sc->proj_c;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.n; i += gridDim.x * blockDim.x) {
+    const T zi = z[colour_pos(g, i)] - c;
+    p[i] = is_first ? zi : fma(beta, p[i], zi);
   }
 }
 
@@ -992,6 +1058,10 @@ int grid_for(int64_t n, int threads, int sms) {
   return (int)gsz;
 }
 
+struct CMap {
+  int64_t cbase[8];
+  int32_t nlev[2];
+};
 CMap cmap_of(const pm_operator* op) {
   CMap cm;
   cm.nlev[0] = (op->nz + 1) / 2;
@@ -1004,28 +1074,54 @@ CMap cmap_of(const pm_operator* op) {
   return cm;
 }
 
-void ic0_apply(pm_operator* op, int which, const double* r, double* z, const PcgScalars* sc,
-               int check_done, cudaStream_t s) {
-  Geom g = geom_of(op);
-  CMap cm = cmap_of(op);
-  const double* F = op->ic0[which].F;
-  int64_t off[5] = {0, 0, 0, 0, 0};
-  for (int c = 0; c < 4; ++c) off[c + 1] = off[c] + op->cls_count[c];
-#define PM_SWEEP(C, FW)                                                                        \
-  {                                                                                            \
-    const int64_t cnt = op->cls_count[(C) & 3];                                                \
-    const int64_t tot = cnt * cm.nlev[(C) >> 2];                                               \
-    if (tot > 0) {                                                                             \
-      k_ic0_sweep<C, FW, double><<<grid_for((tot + 1) / 2, TPB, op->num_sms), TPB, 0, s>>>(     \
-          g, cm, op->d_cls_cols, off[(C) & 3], cnt, F, r, z, sc, check_done);                  \
-      count_launch();                                                                          \
-    }                                                                                          \
+SweepGeo sweep_geo(const pm_operator* op) {
+  SweepGeo g;
+  const CMap cm = cmap_of(op);
+  g.n = (int32_t)op->n;
+  g.nz = op->nz;
+  g.ncols = op->ncols;
+  g.cnbr = op->d_cnbr;
+  g.ccls = op->d_ccls;
+  g.colpos = op->d_colpos;
+  for (int c = 0; c < 8; ++c) g.cbase[c] = (int32_t)cm.cbase[c];
+  for (int q = 0, off = 0; q < 4; ++q) {
+    g.cls_off[q] = off;
+    g.cls_cnt[q] = op->cls_count[q];
+    off += op->cls_count[q];
   }
-  PM_SWEEP(0, 1) PM_SWEEP(1, 1) PM_SWEEP(2, 1) PM_SWEEP(3, 1)
-  PM_SWEEP(4, 1) PM_SWEEP(5, 1) PM_SWEEP(6, 1) PM_SWEEP(7, 1)
-  PM_SWEEP(7, 0) PM_SWEEP(6, 0) PM_SWEEP(5, 0) PM_SWEEP(4, 0)
-  PM_SWEEP(3, 0) PM_SWEEP(2, 0) PM_SWEEP(1, 0) PM_SWEEP(0, 0)
+  g.nlev[0] = fast_div(cm.nlev[0]);
+  g.nlev[1] = fast_div(cm.nlev[1]);
+  g.nzd = fast_div(op->nz);
+  return g;
+}
+
+// z = (L L^T)^{-1} r into z (colour order), and rho, beta (m: the projection's mass vector, null: none).
+// is_first: the step that starts a recurrence; its kernels run whatever the done flag says.
+template <typename T, typename TM>
+void ic0_apply(pm_operator* op, const T* F, const T* r, T* z, const TM* m, double* partials, PcgScalars* sc, int is_first,
+               cudaStream_t s) {
+  const SweepGeo g = sweep_geo(op);
+  const int G = grid_for(op->n, TPB, op->num_sms), check = is_first ? 0 : 1;
+#define PM_SWEEP(C, FW)                                                                                         \
+  {                                                                                                             \
+    const int64_t tot = (int64_t)g.cls_cnt[(C) & 3] * g.nlev[(C) >> 2].d;                                       \
+    if (tot > 0) {                                                                                              \
+      k_ic0_sweep<C, FW, T><<<(int)((tot + TPB - 1) / TPB), TPB, 0, s>>>(g, F, r, z, sc, check);                \
+      count_launch();                                                                                           \
+    }                                                                                                           \
+  }
+  {
+    KtScope t(PM_KT_IC0, 16, s);
+    PM_SWEEP(0, 1) PM_SWEEP(1, 1) PM_SWEEP(2, 1) PM_SWEEP(3, 1)
+    PM_SWEEP(4, 1) PM_SWEEP(5, 1) PM_SWEEP(6, 1) PM_SWEEP(7, 1)
+    if (m) k_ic0_mid<T, 0><<<G, TPB, 0, s>>>(g, F, z, partials, sc, is_first);
+    else k_ic0_mid<T, 1><<<G, TPB, 0, s>>>(g, F, z, partials, sc, is_first);
+    PM_SWEEP(6, 0) PM_SWEEP(5, 0) PM_SWEEP(4, 0)
+    PM_SWEEP(3, 0) PM_SWEEP(2, 0) PM_SWEEP(1, 0) PM_SWEEP(0, 0)
+  }
 #undef PM_SWEEP
+  if (m) k_ic0_rho_proj<T, TM><<<G, TPB, 0, s>>>(g, r, z, m, partials, sc, is_first);
+  count_launch(m ? 2 : 1);
 }
 
 int ensure_ctx(pm_operator* op) {
@@ -1093,18 +1189,10 @@ void launch_iter(pm_operator* op, int which, const double* val, double* x, bool 
       k_cg_update<0, 0><<<G, TPB, 0, s>>>(op->n, x, c->r, c->p, c->w, dinv, op->d_m, c->partials, c->sc);
     }
     count_launch(1);
+    ic0_apply(op, op->ic0[which].F, c->r, c->z, proj ? op->d_m : nullptr, c->partials, c->sc, 0, s);
     {
-      KtScope t(PM_KT_IC0, 16, s);
-      ic0_apply(op, which, c->r, c->z, c->sc, 1, s);
-    }
-    {
-      KtScope t(PM_KT_PUPDATE, 2, s);
-      if (proj) {
-        k_cg_rho<1, 1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, c->z, op->d_m, c->partials, c->sc, 0);
-      } else {
-        k_cg_rho<0, 1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, c->z, op->d_m, c->partials, c->sc, 0);
-      }
-      k_cg_pupd<1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, c->z, c->p, c->sc, 0);
+      KtScope t(PM_KT_PUPDATE, 1, s);
+      k_ic0_pupd<<<G, TPB, 0, s>>>(sweep_geo(op), c->z, c->p, c->sc, 0);
     }
     count_launch(2);
   }
@@ -1135,13 +1223,11 @@ void launch_first(pm_operator* op, int which, bool proj, int prec, const double*
     return;
   }
   if (prec == PM_PREC_IC0) {
-    ic0_apply(op, which, c->r, c->z, c->sc, 0, s);
-    if (proj) k_cg_rho<1, 1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, c->z, op->d_m, c->partials, c->sc, 1);
-    else k_cg_rho<0, 1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, c->z, op->d_m, c->partials, c->sc, 1);
-    k_cg_pupd<1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, c->z, c->p, c->sc, 1);
+    ic0_apply(op, op->ic0[which].F, c->r, c->z, proj ? op->d_m : nullptr, c->partials, c->sc, 1, s);
+    k_ic0_pupd<<<G, TPB, 0, s>>>(sweep_geo(op), c->z, c->p, c->sc, 1);
   } else {
-    if (proj) k_cg_rho<1, 0><<<G, TPB, 0, s>>>(op->n, c->r, dinv, nullptr, op->d_m, c->partials, c->sc, 1);
-    else k_cg_rho<0, 0><<<G, TPB, 0, s>>>(op->n, c->r, dinv, nullptr, op->d_m, c->partials, c->sc, 1);
+    if (proj) k_cg_rho<1><<<G, TPB, 0, s>>>(op->n, c->r, dinv, op->d_m, c->partials, c->sc);
+    else k_cg_rho<0><<<G, TPB, 0, s>>>(op->n, c->r, dinv, op->d_m, c->partials, c->sc);
     k_cg_pupd<0><<<G, TPB, 0, s>>>(op->n, c->r, dinv, nullptr, c->p, c->sc, 1);
   }
   count_launch(2);
@@ -1573,16 +1659,14 @@ __global__ void __launch_bounds__(TPB) k32_update(int64_t n, float* __restrict__
   }
 }
 
-// rho = (r, z') with z' = z - c (pressure) from stored or inline z; first: beta = 0.
-template <int PROJ, int STORED>
+// First preconditioned residual: rho = (r, z') with z' = z - c (pressure), z = dinv r; beta = 0.
+template <int PROJ>
 __global__ void __launch_bounds__(TPB) k32_rho(int64_t n, const float* __restrict__ r, const float* __restrict__ dinv,
-                                               const float* __restrict__ zbuf, const float2* __restrict__ m2,
-                                               double* partials, PcgScalars* sc, int is_first) {
-  if (!is_first && sc_done(sc)) return;
+                                               const float2* __restrict__ m2, double* partials, PcgScalars* sc) {
   DF a[3];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float ri = r[i];
-    const float zi = STORED ? zbuf[i] : dinv[i] * ri;
+    const float zi = dinv[i] * ri;
     a[0].add_prod(ri, zi);
     if (PROJ) {
       add_mz(a[1], m2[i], zi);
@@ -1594,13 +1678,8 @@ __global__ void __launch_bounds__(TPB) k32_rho(int64_t n, const float* __restric
     const double c = PROJ ? v[1] / sc->one_m : 0.0;
     const double rho_new = v[0] - c * v[2];
     sc->proj_c = c;
-    if (is_first) {
-      sc->rho = rho_new;
-      sc->beta = 0.0;
-    } else {
-      sc->beta = rho_new / sc->rho;
-      sc->rho = rho_new;
-    }
+    sc->rho = rho_new;
+    sc->beta = 0.0;
     if ((!(rho_new > 0.0) || !isfinite(rho_new)) && !sc->done) {
       sc->status = PM_BREAKDOWN;
       sc->done = 1;
@@ -1917,31 +1996,6 @@ void update_line32(pm_operator* op, int which, bool proj, int mode, cudaStream_t
                                                       op->d_m2f, c->partials, c->sc_in, mode);
 }
 
-// FP32 IC0 apply: the same colour sweeps (k_ic0_sweep<.., float>) on the FP32 copy of the factor.
-void ic0_apply32(pm_operator* op, int which, const float* r, float* z, const PcgScalars* sc, int check_done,
-                 cudaStream_t s) {
-  Geom g = geom_of(op);
-  CMap cm = cmap_of(op);
-  const float* F = op->d_ic0_32[which];
-  int64_t off[5] = {0, 0, 0, 0, 0};
-  for (int c = 0; c < 4; ++c) off[c + 1] = off[c] + op->cls_count[c];
-#define PM_SWEEP32(C, FW)                                                                      \
-  {                                                                                            \
-    const int64_t cnt = op->cls_count[(C) & 3];                                                \
-    const int64_t tot = cnt * cm.nlev[(C) >> 2];                                               \
-    if (tot > 0) {                                                                             \
-      k_ic0_sweep<C, FW, float><<<grid_for((tot + 1) / 2, TPB, op->num_sms), TPB, 0, s>>>(     \
-          g, cm, op->d_cls_cols, off[(C) & 3], cnt, F, r, z, sc, check_done);                  \
-      count_launch();                                                                          \
-    }                                                                                          \
-  }
-  PM_SWEEP32(0, 1) PM_SWEEP32(1, 1) PM_SWEEP32(2, 1) PM_SWEEP32(3, 1)
-  PM_SWEEP32(4, 1) PM_SWEEP32(5, 1) PM_SWEEP32(6, 1) PM_SWEEP32(7, 1)
-  PM_SWEEP32(7, 0) PM_SWEEP32(6, 0) PM_SWEEP32(5, 0) PM_SWEEP32(4, 0)
-  PM_SWEEP32(3, 0) PM_SWEEP32(2, 0) PM_SWEEP32(1, 0) PM_SWEEP32(0, 0)
-#undef PM_SWEEP32
-}
-
 int ensure_mixed(pm_operator* op, int which, int precision, int prec, cudaStream_t s) {
   SolveCtx* c = op->ctx;
   const size_t fb = (size_t)op->n * sizeof(float);
@@ -2126,17 +2180,12 @@ void inner_iter(pm_operator* op, int which, const TV* val32, bool proj, int prec
       KtScope t(PM_KT_UPDATE, 1, s);
       k32_update<0, 0><<<G, TPB, 0, s>>>(op->n, c->d32, c->r32, c->p32, c->w32, dinv32, op->d_m2f, c->partials, c->sc_in);
     }
+    ic0_apply(op, op->d_ic0_32[which], c->r32, c->z32, proj ? op->d_m2f : nullptr, c->partials, c->sc_in, 0, s);
     {
-      KtScope t(PM_KT_IC0, 16, s);
-      ic0_apply32(op, which, c->r32, c->z32, c->sc_in, 1, s);
+      KtScope t(PM_KT_PUPDATE, 1, s);
+      k_ic0_pupd<<<G, TPB, 0, s>>>(sweep_geo(op), c->z32, c->p32, c->sc_in, 0);
     }
-    {
-      KtScope t(PM_KT_PUPDATE, 2, s);
-      if (proj) k32_rho<1, 1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, op->d_m2f, c->partials, c->sc_in, 0);
-      else k32_rho<0, 1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, op->d_m2f, c->partials, c->sc_in, 0);
-      k32_pupd<1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, c->p32, c->sc_in, 0);
-    }
-    count_launch(4);
+    count_launch(3);
   } else {
     {
       KtScope t(PM_KT_UPDATE, 1, s);
@@ -2159,13 +2208,11 @@ void inner_first(pm_operator* op, int which, bool proj, int prec, const float* d
     update_line32(op, which, proj, 0, s);
     k32_pupd<1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, c->p32, c->sc_in, 1);
   } else if (prec == PM_PREC_IC0) {
-    ic0_apply32(op, which, c->r32, c->z32, c->sc_in, 0, s);
-    if (proj) k32_rho<1, 1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, op->d_m2f, c->partials, c->sc_in, 1);
-    else k32_rho<0, 1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, op->d_m2f, c->partials, c->sc_in, 1);
-    k32_pupd<1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, c->p32, c->sc_in, 1);
+    ic0_apply(op, op->d_ic0_32[which], c->r32, c->z32, proj ? op->d_m2f : nullptr, c->partials, c->sc_in, 1, s);
+    k_ic0_pupd<<<G, TPB, 0, s>>>(sweep_geo(op), c->z32, c->p32, c->sc_in, 1);
   } else {
-    if (proj) k32_rho<1, 0><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, nullptr, op->d_m2f, c->partials, c->sc_in, 1);
-    else k32_rho<0, 0><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, nullptr, op->d_m2f, c->partials, c->sc_in, 1);
+    if (proj) k32_rho<1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, op->d_m2f, c->partials, c->sc_in);
+    else k32_rho<0><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, op->d_m2f, c->partials, c->sc_in);
     k32_pupd<0><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, nullptr, c->p32, c->sc_in, 1);
   }
   count_launch(2);
