@@ -73,10 +73,9 @@ struct Args {
   const float2* m2;       // M 1 as two floats (mixed precision)
   const void* ic0;        // IC0 factor, colour-ordered rows, 1 / L_ii in the diagonal slot
   const void* line;       // line factors, level-major
-  const int32_t* cnbr;    // neighbour columns in class order
-  const int32_t* clsidx;  // index of a column within its class
-  const int32_t* coli;
-  const int32_t* colj;
+  const int32_t* cnbr;    // columns in class order
+  const int32_t* ccls;    // [7][ncols]: their neighbours' indices within their classes
+  const int32_t* colpos;  // [2][ncols]: first colour-ordered position of a column's even / odd levels
   int32_t cls_off[4], cls_cnt[4];
   int32_t cbase[8];
   FastDiv nlev[2];        // levels of even / odd parity
@@ -113,6 +112,7 @@ struct Scratch {
   double res[4];
   double xch[2][4][CLUSTER];   // cluster team: the blocks' sums
   int ok;
+  int first[8], past[8];       // this block's share of each colour's rows
 };
 
 template <bool CL>
@@ -212,8 +212,9 @@ struct Team {
   }
 };
 
-__device__ __forceinline__ int cnbr_of(const Args& a, int i, int q) {
-  const int nb = __ldg(a.cnbr + q * a.g.ncols + i);
+// Neighbour q, by its index within its class, of the column at place i in class order (-1: none).
+__device__ __forceinline__ int ccls_of(const Args& a, int i, int q) {
+  const int nb = __ldg(a.ccls + q * a.g.ncols + i);
 #ifdef PM_CHECKED
   if (nb < -1 || nb >= a.g.ncols) {
     record_bad_index(SITE_NBR, nb, a.g.ncols);
@@ -328,11 +329,19 @@ __device__ __forceinline__ void move_row(const Args& a, int row, T alpha, T beta
   p[row] = fma(beta, pv, z);
 }
 
-// Constant operands of one row of a colour phase: its place, neighbour columns and factor row.
+// The sweeps' work vector (y, then z) is in colour order, as the factor's rows are: position cbase[colour] +
+// (index of the column in its parity class) * levels + level / 2. A colour's rows are every other level of
+// their columns; in colour order a warp's reads of each neighbour are runs, in the natural order every other
+// entry of each sector.
+__device__ __forceinline__ int colour_pos(const Args& a, int col, int k) {
+  return __ldg(a.colpos + (k & 1) * a.g.ncols + col) + (k >> 1);
+}
+
+// Constant operands of one row of a colour phase: its places, neighbours and factor row.
 template <typename T, int C, bool FWD>
 struct ColourRow {
   static constexpr int kpar = C >> 2, cls = C & 3;
-  int row, k;
+  int row, pos, kk;   // in natural order, in colour order; level / 2
   int nb[NNBR];
   T f[NSLOT];
   // The slots read: lower colours forward, higher ones backward.
@@ -343,26 +352,27 @@ struct ColourRow {
   __device__ __forceinline__ void load(const Args& a, int t) {
     const T* __restrict__ F = static_cast<const T*>(a.ic0);
     const int i = fdiv(a.nlev[kpar], t), n = (int)a.g.n;
-    const int at = min(a.cls_off[cls] + i, a.g.ncols - 1), pos = min(a.cbase[C] + t, n - 1);
-    k = 2 * (t - i * a.nlev[kpar].d) + kpar;
+    const int at = min(a.cls_off[cls] + i, a.g.ncols - 1);
+    pos = min(a.cbase[C] + t, n - 1);
+    kk = t - i * a.nlev[kpar].d;
+    nb[0] = i;
 #pragma unroll
-    for (int q = 0; q < NNBR; ++q) nb[q] = cnbr_of(a, at, q);
+    for (int q = 1; q < NNBR; ++q) nb[q] = ccls_of(a, at, q);
 #pragma unroll
     for (int s = 0; s < NSLOT; ++s)
       if (uses(s) || s == DIAG_SLOT) f[s] = __ldg(F + (s * n + pos));
-    row = nb[0] * a.g.nz + k;
+    row = __ldg(a.cnbr + at) * a.g.nz + 2 * kk + kpar;
   }
   // (v - sum f_s y_s) / L_ii
-  __device__ __forceinline__ T value(int nz, T v, const T* y) const {
+  __device__ __forceinline__ T value(const Args& a, T v, const T* y) const {
     T yv[NSLOT];
 #pragma unroll
     for (int s = 0; s < NSLOT; ++s) {
       if (!uses(s)) continue;
-      const int kk = k + slot_dk(s), q = slot_q(s);
-      bool ok = nb[q] >= 0;
-      if (slot_dk(s) < 0) ok = ok && kk >= 0;
-      if (slot_dk(s) > 0) ok = ok && kk < nz;
-      yv[s] = ok ? y[nb[q] * nz + kk] : (T)0;
+      const int cj = C ^ slot_flip(s), dk = slot_dk(s), nl = a.nlev[cj >> 2].d;
+      const int lv = kk + (dk == 0 ? 0 : dk > 0 ? kpar : kpar - 1);   // the neighbour's level / 2
+      const bool ok = nb[slot_q(s)] >= 0 && lv >= 0 && lv < nl;
+      yv[s] = ok ? y[a.cbase[cj] + nb[slot_q(s)] * nl + lv] : (T)0;
     }
 #pragma unroll
     for (int s = 0; s < NSLOT; ++s)
@@ -381,25 +391,23 @@ __device__ __forceinline__ bool colour_phase(const Args& a, Team<CL>& team, T al
   using Row = ColourRow<T, C, FWD>;
   const T* r = static_cast<const T*>(a.r);
   T* y = static_cast<T*>(a.z);
-  const int nz = a.g.nz;
-  const int tot = a.cls_cnt[Row::cls] * a.nlev[Row::kpar].d;
-  const int t0 = (int)((int64_t)tot * team.rank / team.G), t1 = (int)((int64_t)tot * (team.rank + 1) / team.G);
-  int t = t0 + (int)threadIdx.x;
+  const int t1 = team.s->past[C];
+  int t = team.s->first[C] + (int)threadIdx.x;
   Row w;
   if (SYNC) {
     // without a condition (a clamped place instead): loaded under one, the row went to local memory
-    w.load(a, max(0, min(t, tot - 1)));
+    w.load(a, max(0, min(t, t1 - 1)));
     if (!team.wait()) return false;
   }
 #pragma unroll 1
   for (bool first = SYNC; t < t1; t += NT, first = false) {
     if (!first) w.load(a, t);
-    T v = w.value(nz, FWD ? r[w.row] : y[w.row], y);
+    T v = w.value(a, FWD ? r[w.row] : y[w.pos], y);
     if (FWD) {
       acc.add_prod(v, v);
       if (C == 7) v *= w.f[DIAG_SLOT];
     }
-    y[w.row] = v;
+    y[w.pos] = v;
     if (FUSEP) move_row(a, w.row, alpha, beta, v);
   }
   return true;
@@ -407,11 +415,12 @@ __device__ __forceinline__ bool colour_phase(const Args& a, Team<CL>& team, T al
 
 // y of colour 0 for one row in natural order: r / L_ii (no lower colour). Other rows: nothing.
 template <typename T, typename Acc>
-__device__ __forceinline__ void colour0_y(const Args& a, int row, int col, int k, T ri, Acc& acc) {
-  if ((k | __ldg(a.coli + col) | __ldg(a.colj + col)) & 1) return;
-  const int t = __ldg(a.clsidx + col) * a.nlev[0].d + (k >> 1);
-  const T v = ri * __ldg(static_cast<const T*>(a.ic0) + DIAG_SLOT * (int)a.g.n + t);
-  static_cast<T*>(a.z)[row] = v;
+__device__ __forceinline__ void colour0_y(const Args& a, int col, int k, T ri, Acc& acc) {
+  if (k & 1) return;
+  const int pos = colour_pos(a, col, k);
+  if (pos >= a.cbase[1]) return;
+  const T v = ri * __ldg(static_cast<const T*>(a.ic0) + DIAG_SLOT * (int)a.g.n + pos);
+  static_cast<T*>(a.z)[pos] = v;
   acc.add_prod(v, v);
 }
 
@@ -435,12 +444,10 @@ template <typename T, bool FUSEP, bool CL>
 __device__ __forceinline__ bool ic0_backward(const Args& a, Team<CL>& team, T alpha, T beta) {
   Acc64 unused;
   if (FUSEP) {   // rows of colour 7 have their z already: x and p where this block formed it
-    const int tot = a.cls_cnt[3] * a.nlev[1].d;
-    const int t1 = (int)((int64_t)tot * (team.rank + 1) / team.G);
-    for (int t = (int)((int64_t)tot * team.rank / team.G) + (int)threadIdx.x; t < t1; t += NT) {
+    for (int t = team.s->first[7] + (int)threadIdx.x; t < team.s->past[7]; t += NT) {
       const int i = fdiv(a.nlev[1], t);
       const int row = __ldg(a.cnbr + a.cls_off[3] + i) * a.g.nz + 2 * (t - i * a.nlev[1].d) + 1;
-      move_row(a, row, alpha, beta, static_cast<const T*>(a.z)[row]);
+      move_row(a, row, alpha, beta, static_cast<const T*>(a.z)[a.cbase[7] + t]);
     }
   }
   if (!colour_phase<T, 6, false, FUSEP, false>(a, team, alpha, beta, unused)) return false;
@@ -491,7 +498,7 @@ __device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alp
       } else {
         const int col = fdiv(g.nzd, row), k = row - col * nz;
         if (PREC == PM_PREC_LINE) zt[(col - c0) * ld + k] = ri;
-        else colour0_y(a, row, col, k, ri, dots.rz);
+        else colour0_y(a, col, k, ri, dots.rz);
       }
     }
   }
@@ -551,7 +558,8 @@ __device__ __forceinline__ void direction(const Args& a, int c0, int c1, T alpha
           const int col = fdiv(g.nzd, row);
           z[u] = zt[(col - c0) * ld + row - col * nz];
         } else {
-          z[u] = zv[row];
+          const int col = fdiv(g.nzd, row);
+          z[u] = zv[colour_pos(a, col, row - col * nz)];
         }
       }
       if (!FIRST) {
@@ -597,8 +605,10 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, int c0, i
       const T* z = static_cast<const T*>(a.z);
       AccFor<T> rz;
       for (int row = c0 * a.g.nz + (int)threadIdx.x; row < c1 * a.g.nz; row += NT) {
-        rz.add_prod(r[row], z[row]);
-        add_m(dots.mz, a, row, z[row]);
+        const int col = fdiv(a.g.nzd, row);
+        const T zi = z[colour_pos(a, col, row - col * a.g.nz)];
+        rz.add_prod(r[row], zi);
+        add_m(dots.mz, a, row, zi);
       }
       double u[3] = {rz.value(), dots.mz.value(), dots.sr.value()};
       if (!team.template sum<3>(u)) return false;
@@ -880,6 +890,13 @@ template <typename T, typename TV, int PREC, bool CL>
 __global__ void __launch_bounds__(NT, 1) k_resident(Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Scratch scratch;
+  if (PREC == PM_PREC_IC0 && threadIdx.x < 8) {   // 64-bit divisions: once, not in every phase
+    const int c = threadIdx.x;
+    const int64_t tot = (int64_t)a.cls_cnt[c & 3] * (c >> 2 ? a.nlev[1].d : a.nlev[0].d);
+    scratch.first[c] = (int)(tot * blockIdx.x / gridDim.x);
+    scratch.past[c] = (int)(tot * (blockIdx.x + 1) / gridDim.x);
+  }
+  __syncthreads();
   Team<CL> team(a, &scratch);
   if (CL) team.barrier();   // every block of the cluster runs before one writes to another's shared memory
   // whole columns, dealt evenly

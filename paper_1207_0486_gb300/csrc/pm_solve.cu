@@ -1437,9 +1437,8 @@ resident::Args resident_args(pm_operator* op, int which, const double* b, double
   a.bw = c->bw;
   a.m = op->d_m;
   a.cnbr = op->d_cnbr;
-  a.clsidx = op->d_cls_cols + op->ncols;
-  a.coli = a.clsidx + op->ncols;
-  a.colj = a.coli + op->ncols;
+  a.ccls = op->d_ccls;
+  a.colpos = op->d_colpos;
   const CMap cm = cmap_of(op);
   for (int q = 0, off = 0; q < 4; ++q) {
     a.cls_off[q] = off;
