@@ -164,10 +164,16 @@ __host__ __device__ __forceinline__ int fdiv(const FastDiv& f, int t) {
 // ---- compensated residual (Ogita, Rump & Oishi, "Accurate sum and dot product", 2005) --------
 // Error-free transformations in FP64. The _rn intrinsics are never contracted into an FMA, which
 // would change what the transformations compute.
+//
+// a + b = s + err exactly. Dekker's three additions need the exponent of the first operand to be at least
+// the second's; Knuth's six need nothing. An FP64 addition holds this GPU's FP64 pipe for 64 cycles a warp, an
+// integer comparison of the high words and the selects that order the operands take a few, so the
+// operands are ordered: the same s and err with half the additions.
 __device__ __forceinline__ double two_sum(double a, double b, double& err) {
-  const double s = __dadd_rn(a, b);
-  const double bv = __dsub_rn(s, a);
-  err = __dadd_rn(__dsub_rn(a, __dsub_rn(s, bv)), __dsub_rn(b, bv));
+  const bool swap = (__double2hiint(b) & 0x7fffffff) > (__double2hiint(a) & 0x7fffffff);
+  const double big = swap ? b : a, small = swap ? a : b;
+  const double s = __dadd_rn(big, small);
+  err = __dsub_rn(small, __dsub_rn(s, big));
   return s;
 }
 // a * b = p + err exactly (one FMA gives the rounding error of the product).
@@ -245,9 +251,9 @@ __device__ __forceinline__ int nbr_of(const Geom& g, int64_t col, int q) {
 // accurate as b_i - (A x)_i formed in twice the working precision and rounded once; the plain
 // FP64 residual of a nearly converged x is wrong by up to u (|A||x|)_i, which for the thin
 // basins' pressure operator is of the order of the residuals a solve aims for.
-// abs_sum receives (|A||x|)_i (the FP64 floor). MASKC >= 0: component MASKC's symmetric
+// abs_sum receives (|A||x|)_i (the FP64 floor) when WANT_ABS. MASKC >= 0: component MASKC's symmetric
 // Dirichlet elimination (identity row, zero column), as the solvers apply it.
-template <int MASKC>
+template <int MASKC, bool WANT_ABS = true>
 __device__ __forceinline__ double row_residual_dot2(const Geom& g, const double* __restrict__ val,
                                                     const double* x, double bi, int row, int col, int k,
                                                     double& abs_sum) {
@@ -282,7 +288,7 @@ __device__ __forceinline__ double row_residual_dot2(const Geom& g, const double*
     const double p = two_product(av, xv, pe);
     s = two_sum(s, -p, se);
     c = __dadd_rn(c, __dsub_rn(se, pe));
-    asum += fabs(p);
+    if (WANT_ABS) asum += fabs(p);
   }
   abs_sum = asum;
   return __dadd_rn(s, c);

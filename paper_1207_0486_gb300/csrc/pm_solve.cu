@@ -274,15 +274,50 @@ __global__ void __launch_bounds__(TPB) k_cg_press_sums(int64_t n, const double* 
   }
 }
 
-// bw = b - lam m (pressure) and x = x - xshift (pressure) or x = 0 (no guess).
+// Pressure with a guess: bw = b - lam m and x = x - xshift.
 __global__ void k_cg_prepare(int64_t n, const double* __restrict__ b, const double* __restrict__ m,
-                             double* __restrict__ bw, double* __restrict__ x, int press, int use_x,
-                             const PcgScalars* sc) {
-  const double lam = press ? sc->lam : 0.0, xs = press ? sc->xshift : 0.0;
+                             double* __restrict__ bw, double* __restrict__ x, const PcgScalars* sc) {
+  const double lam = sc->lam, xs = sc->xshift;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (press) bw[i] = b[i] - lam * m[i];
-    x[i] = use_x ? x[i] - xs : 0.0;
+    bw[i] = b[i] - lam * m[i];
+    x[i] = x[i] - xs;
   }
+}
+
+// Scalars of a solve from ||b||^2 and the first ||r||^2: target, zero right-hand side, first convergence test.
+__device__ __forceinline__ void start_scalars(PcgScalars* sc, double rtol, double bb, double rr) {
+  sc->bb = bb;
+  sc->rr = rr;
+  sc->tol2 = rtol * rtol * bb;
+  sc->zero_rhs = bb == 0.0;
+  sc->iter = 0;
+  sc->status = PM_OK;
+  sc->done = (bb == 0.0 || rr <= sc->tol2) ? 1 : 0;
+  if (!sc->done && sc->max_iter == 0) {  // no iteration allowed: report the initial residual
+    sc->status = PM_NOT_CONVERGED;
+    sc->done = 1;
+  }
+}
+
+// A solve from x = 0: bw = b - lam m (pressure), r = bw itself, (bw, bw). The residual kernel would spend 1.5 ms at
+// 5M rows on forming b - A 0.
+__global__ void __launch_bounds__(TPB) k_cg_start_zero(int64_t n, const double* __restrict__ b, const double* __restrict__ m,
+                                                       double* __restrict__ bw, double* __restrict__ x,
+                                                       double* __restrict__ r, int press, double rtol, double* partials,
+                                                       PcgScalars* sc) {
+  const double lam = press ? sc->lam : 0.0;
+  double v[1] = {0.0};
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double bi = b[i];
+    if (press) {
+      bi = bi - lam * m[i];
+      bw[i] = bi;
+    }
+    x[i] = 0.0;
+    r[i] = bi;
+    v[0] = fma(bi, bi, v[0]);
+  }
+  if (grid_sum<1>(v, partials, &sc->count[1]) && threadIdx.x == 0) start_scalars(sc, rtol, v[0], v[0]);
 }
 
 // r = bw - A x, row by row in compensated arithmetic (row_residual_dot2); grid sums (bw, bw),
@@ -300,7 +335,7 @@ __global__ void __launch_bounds__(TPB) k_cg_residual(Geom g, const double* __res
     const int k = row - col * g.nz;
     double asum = 0.0;
     const double bi = bw[row];
-    const double ri = row_residual_dot2<MASKC>(g, val, x, bi, row, col, k, asum);
+    const double ri = row_residual_dot2<MASKC, MODE == 1>(g, val, x, bi, row, col, k, asum);
     r[row] = ri;
     v[0] = fma(bi, bi, v[0]);
     v[1] = fma(ri, ri, v[1]);
@@ -311,17 +346,7 @@ __global__ void __launch_bounds__(TPB) k_cg_residual(Geom g, const double* __res
   }
   if (grid_sum<3>(v, partials, &sc->count[1]) && threadIdx.x == 0) {
     if (MODE == 0) {
-      sc->bb = v[0];
-      sc->rr = v[1];
-      sc->tol2 = rtol * rtol * v[0];
-      sc->zero_rhs = v[0] == 0.0;
-      sc->iter = 0;
-      sc->status = PM_OK;
-      sc->done = (v[0] == 0.0 || v[1] <= sc->tol2) ? 1 : 0;
-      if (!sc->done && sc->max_iter == 0) {  // no iteration allowed: report the initial residual
-        sc->status = PM_NOT_CONVERGED;
-        sc->done = 1;
-      }
+      start_scalars(sc, rtol, v[0], v[1]);
     } else {
       sc->aux[0] = v[1];
       sc->aux[1] = v[2];
@@ -1211,6 +1236,31 @@ void launch_residual(pm_operator* op, const double* val, const double* bw, const
   count_launch();
 }
 
+// Projected right-hand side (pressure: returned in the workspace), initial guess, first residual in c->r and the
+// scalars that start a solve.
+template <int MASKC>
+const double* launch_start(pm_operator* op, const double* val, const double* b, double* x, bool proj, const pm_solve_opts* o,
+                           cudaStream_t s) {
+  SolveCtx* c = op->ctx;
+  const int G = grid_for(op->n, TPB, op->num_sms), guess = o->x0_is_guess ? 1 : 0;
+  if (proj) {
+    k_cg_press_sums<<<G, TPB, 0, s>>>(op->n, b, x, op->d_m, guess, c->partials, c->sc);
+    count_launch();
+  }
+  const double* bw = proj ? c->bw : b;
+  if (!guess) {
+    k_cg_start_zero<<<G, TPB, 0, s>>>(op->n, b, op->d_m, c->bw, x, c->r, proj ? 1 : 0, o->rtol, c->partials, c->sc);
+    count_launch();
+    return bw;
+  }
+  if (proj) {
+    k_cg_prepare<<<G, TPB, 0, s>>>(op->n, b, op->d_m, c->bw, x, c->sc);
+    count_launch();
+  }
+  launch_residual<MASKC>(op, val, bw, x, o->rtol, 0, s);
+  return bw;
+}
+
 // z, p, rho from the current r (first step or restart). The kernels run even when "done" is
 // set by the setup so that a zero initial residual still leaves consistent scalars.
 void launch_first(pm_operator* op, int which, bool proj, int prec, const double* dinv, cudaStream_t s) {
@@ -1309,17 +1359,7 @@ int pcg_run(pm_operator* op, int which, const double* b, double* x, const pm_sol
   init.one_m = op->one_m;
   init.max_iter = o->max_iter;
   if ((st = cuda_check(cudaMemcpyAsync(c->sc, &init, sizeof(init), cudaMemcpyHostToDevice, s), "scalars init"))) return st;
-  const double* bw = b;
-  if (proj) {
-    k_cg_press_sums<<<G, TPB, 0, s>>>(op->n, b, x, op->d_m, o->x0_is_guess ? 1 : 0, c->partials, c->sc);
-    k_cg_prepare<<<G, TPB, 0, s>>>(op->n, b, op->d_m, c->bw, x, 1, o->x0_is_guess ? 1 : 0, c->sc);
-    count_launch(2);
-    bw = c->bw;
-  } else if (!o->x0_is_guess) {
-    k_cg_prepare<<<G, TPB, 0, s>>>(op->n, b, op->d_m, nullptr, x, 0, 0, c->sc);
-    count_launch();
-  }
-  launch_residual<MASKC>(op, val, bw, x, o->rtol, 0, s);
+  const double* bw = launch_start<MASKC>(op, val, b, x, proj, o, s);
   launch_first(op, which, proj, prec, dinv, s);
   if ((st = read_scalars(c, s))) return st;
   int restarts = 0;
@@ -2245,17 +2285,7 @@ int mixed_run(pm_operator* op, int which, const double* b, double* x, const pm_s
   init.one_m = op->one_m;
   init.max_iter = o->max_iter;
   if ((st = cuda_check(cudaMemcpyAsync(c->sc, &init, sizeof(init), cudaMemcpyHostToDevice, s), "scalars init"))) return st;
-  const double* bw = b;
-  if (proj) {
-    k_cg_press_sums<<<G, TPB, 0, s>>>(op->n, b, x, op->d_m, o->x0_is_guess ? 1 : 0, c->partials, c->sc);
-    k_cg_prepare<<<G, TPB, 0, s>>>(op->n, b, op->d_m, c->bw, x, 1, o->x0_is_guess ? 1 : 0, c->sc);
-    count_launch(2);
-    bw = c->bw;
-  } else if (!o->x0_is_guess) {
-    k_cg_prepare<<<G, TPB, 0, s>>>(op->n, b, op->d_m, nullptr, x, 0, 0, c->sc);
-    count_launch();
-  }
-  launch_residual<MASKC>(op, val64, bw, x, o->rtol, 0, s);
+  const double* bw = launch_start<MASKC>(op, val64, b, x, proj, o, s);
   if ((st = read_scalars(c, s))) return st;
   const double bb = c->sc_host->bb;
   int outer = 0, inner_total = 0, status = PM_OK;
