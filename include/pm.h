@@ -120,7 +120,7 @@ typedef struct pm_solve_opts {
   int32_t x0_is_guess;   /* 1: x holds the initial guess; 0: start from x = 0               */
   int32_t max_restarts;  /* true-residual restarts after the recursive test passes (FP64)   */
   double inner_rtol;     /* mixed precision: relative reduction asked of each inner solve  */
-  int32_t kernel;        /* FP64 solves: PM_KERNEL_AUTO (resident up to about 3M rows),
+  int32_t kernel;        /* FP64 solves: PM_KERNEL_AUTO (resident up to 2M to 3M rows),
                             PM_KERNEL_STREAM (one launch per PCG phase), or
                             PM_KERNEL_RESIDENT (one launch runs the whole solve, n <= 2^20).
                             Mixed-precision solves run as AUTO                              */
@@ -387,7 +387,7 @@ int64_t pm_kernel_launch_count(void);
 enum { PM_KT_SPMV = 0,    /* SpMV + (p, Ap) reduction, one launch per PCG iteration      */
        PM_KT_UPDATE = 1,  /* x, r update + residual reductions                           */
        PM_KT_PUPDATE = 2, /* search-direction update (with the (r, z) reduction for IC0) */
-       PM_KT_IC0 = 3,     /* the 16 IC0 colour sweeps of one preconditioner apply        */
+       PM_KT_IC0 = 3,     /* the IC0 colour sweeps of one preconditioner apply (16 kernels) */
        PM_KT_LINE = 4,    /* the vertical-line solve fused with the (r, z) reduction     */
        PM_KT_COUNT = 5 };
 int pm_kernel_timing(int32_t enable);

@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(TPB) k_cg_update(int64_t n, double* __restrict
 // other level of their columns, so in the natural order each gathered or stored sector would be half
 // used; in colour order a warp's accesses to every neighbour are runs. The neighbours' class indices
 // come from a table in class order (d_ccls), one load each. Before (natural order, 64-bit index
-// divisions, two dependent index loads per neighbour): 23.8 us per colour phase at 4.9M rows, now 18.9.
+// divisions, two dependent index loads per neighbour): 23.8 us per colour phase at 4.9M rows; 18.9 with this
+// layout, 16.1 launched ahead (below).
 struct SweepGeo {
   int32_t n, nz, ncols;
   const int32_t* cnbr;
@@ -510,41 +511,50 @@ __device__ __forceinline__ int colour_pos(const SweepGeo& g, int row) {
 // The factor's diagonal slot holds 1 / L_ii (a multiply instead of an FP64 division).
 // Position t of colour C: column t / nlev of its class, level 2 (t % nlev) + parity. All of a row's
 // loads but the neighbours' values are independent of one another.
+//
+// Launched ahead of the previous kernel's end (programmatic dependent launch): a block that finds room
+// while that kernel's last blocks run fetches its factor row and neighbour indices, which no kernel of a solve
+// writes, and waits for the previous kernel only then.
 template <int C, int FWD, typename T>
 __global__ void __launch_bounds__(TPB, 4) k_ic0_sweep(SweepGeo g, const T* __restrict__ F, const T* __restrict__ r,
                                                       T* y, const PcgScalars* sc, int check_done) {
-  if (check_done && sc_done(sc)) return;
+  asm volatile("griddepcontrol.launch_dependents;");
   constexpr int kpar = C >> 2, cls = C & 3;
   const int total = g.cls_cnt[cls] * g.nlev[kpar].d;
   const int n = g.n;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int i = fdiv(g.nlev[kpar], t), kk = t - i * g.nlev[kpar].d, at = g.cls_off[cls] + i, pos = g.cbase[C] + t;
-    T f[NSLOT], v[NSLOT];
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, tc = min(t, total - 1);   // the grid covers the rows
+  const int i = fdiv(g.nlev[kpar], tc), kk = tc - i * g.nlev[kpar].d, at = g.cls_off[cls] + i, pos = g.cbase[C] + tc;
+  T f[NSLOT], v[NSLOT];
+  int nb[NNBR];
+  nb[0] = i;
 #pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-      const int cj = C ^ slot_flip(s);
-      if (s == DIAG_SLOT || (FWD ? cj < C : cj > C)) f[s] = __ldg(F + s * n + pos);
-    }
-    T acc = FWD ? r[__ldg(g.cnbr + at) * g.nz + 2 * kk + kpar] : y[pos];
+  for (int q = 1; q < NNBR; ++q) nb[q] = ccls_of(g, at, q);
+  const int own = FWD ? __ldg(g.cnbr + at) * g.nz + 2 * kk + kpar : pos;
 #pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-      const int cj = C ^ slot_flip(s);
-      if (s == DIAG_SLOT || !(FWD ? cj < C : cj > C)) continue;
-      const int dk = slot_dk(s), q = slot_q(s);
-      const int lv = kk + (dk == 0 ? 0 : dk > 0 ? kpar : kpar - 1);   // the neighbour's level / 2
-      const int nl = g.nlev[cj >> 2].d;
-      const int nb = q == 0 ? i : ccls_of(g, at, q);
-      const bool ok = nb >= 0 && lv >= 0 && lv < nl;
-      v[s] = ok ? y[g.cbase[cj] + nb * nl + lv] : (T)0;
-    }
-#pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-      const int cj = C ^ slot_flip(s);
-      if (s == DIAG_SLOT || !(FWD ? cj < C : cj > C)) continue;
-      acc = fma(-f[s], v[s], acc);
-    }
-    y[pos] = acc * f[DIAG_SLOT];
+  for (int s = 0; s < NSLOT; ++s) {
+    const int cj = C ^ slot_flip(s);
+    if (s == DIAG_SLOT || (FWD ? cj < C : cj > C)) f[s] = __ldg(F + s * n + pos);
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (check_done && sc_done(sc)) return;
+  T acc = FWD ? r[own] : y[own];
+#pragma unroll
+  for (int s = 0; s < NSLOT; ++s) {
+    const int cj = C ^ slot_flip(s);
+    if (s == DIAG_SLOT || !(FWD ? cj < C : cj > C)) continue;
+    const int dk = slot_dk(s);
+    const int lv = kk + (dk == 0 ? 0 : dk > 0 ? kpar : kpar - 1);   // the neighbour's level / 2
+    const int nl = g.nlev[cj >> 2].d;
+    const bool ok = nb[slot_q(s)] >= 0 && lv >= 0 && lv < nl;
+    v[s] = ok ? y[g.cbase[cj] + nb[slot_q(s)] * nl + lv] : (T)0;
+  }
+#pragma unroll
+  for (int s = 0; s < NSLOT; ++s) {
+    const int cj = C ^ slot_flip(s);
+    if (s == DIAG_SLOT || !(FWD ? cj < C : cj > C)) continue;
+    acc = fma(-f[s], v[s], acc);
+  }
+  if (t < total) y[pos] = acc * f[DIAG_SLOT];
 }
 
 // Between the sweeps: (y, y), which is (r, z) since y = L^-1 r and z = L^-T y, and colour 7's backward rows
@@ -1127,11 +1137,20 @@ void ic0_apply(pm_operator* op, const T* F, const T* r, T* z, const TM* m, doubl
                cudaStream_t s) {
   const SweepGeo g = sweep_geo(op);
   const int G = grid_for(op->n, TPB, op->num_sms), check = is_first ? 0 : 1;
+  cudaLaunchAttribute ahead;
+  ahead.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  ahead.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(TPB);
+  cfg.stream = s;
+  cfg.attrs = &ahead;
+  cfg.numAttrs = 1;
 #define PM_SWEEP(C, FW)                                                                                         \
   {                                                                                                             \
     const int64_t tot = (int64_t)g.cls_cnt[(C) & 3] * g.nlev[(C) >> 2].d;                                       \
     if (tot > 0) {                                                                                              \
-      k_ic0_sweep<C, FW, T><<<(int)((tot + TPB - 1) / TPB), TPB, 0, s>>>(g, F, r, z, sc, check);                \
+      cfg.gridDim = dim3((unsigned)((tot + TPB - 1) / TPB));                                                    \
+      cudaLaunchKernelEx(&cfg, k_ic0_sweep<C, FW, T>, g, F, r, z, (const PcgScalars*)sc, check);                \
       count_launch();                                                                                           \
     }                                                                                                           \
   }
@@ -1441,7 +1460,7 @@ int pcg_run(pm_operator* op, int which, const double* b, double* x, const pm_sol
 // ---- resident solve: one launch runs the whole PCG (pm_resident.cuh) ---------------------------
 constexpr int64_t RESIDENT_MAX_ROWS = 1 << 20;    // accepted when requested explicitly
 // Automatic choice of the resident solve (measured lines: resident_auto).
-constexpr int64_t RESIDENT_AUTO_ROWS = 3 << 20, RESIDENT_AUTO_MIXED_LINE = 5 << 18;
+constexpr int64_t RESIDENT_AUTO_ROWS = 3 << 20, RESIDENT_AUTO_IC0 = 2 << 20, RESIDENT_AUTO_MIXED_LINE = 5 << 18;
 // Up to here by one cluster of blocks. Measured, us per iteration, cluster / grid: IC0 n = 2,048 40 / 49, 18,000
 // 50 / 49; line 11,803 18.3 / 18.1, 18,000 24 / 21; Jacobi 2,048 10 / 14, 11,803 15.5 / 14.2.
 constexpr int64_t RESIDENT_CLUSTER_ROWS = 8192, RESIDENT_CLUSTER_IC0 = 16384;
@@ -1620,6 +1639,85 @@ __global__ void k_cvt_diff(int64_t n, int64_t npad, const double* __restrict__ v
   }
 }
 
+// Four consecutive rows of one slot's values.
+__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+}
+__device__ __forceinline__ void ld4(const __nv_bfloat16* p, float (&v)[4]) {
+  const uint2 t = __ldg(reinterpret_cast<const uint2*>(p));   // bf16 is the upper half of an FP32 number
+  v[0] = __uint_as_float(t.x << 16), v[1] = __uint_as_float(t.x & 0xffff0000u);
+  v[2] = __uint_as_float(t.y << 16), v[3] = __uint_as_float(t.y & 0xffff0000u);
+}
+
+// k32_spmv for level counts that are multiples of 4: four consecutive rows of a column per thread, so that a
+// slot's values and a neighbour column's entries are one 16-byte load each (the entry above or below the four is a
+// load of its own): 45 loads for four rows instead of 148. The FP32 SpMV is bound by load instructions,
+// not by its 68 bytes a row. Slots by the mask (structural slots, or a component's kept ones): a clear
+// bit's value is 0 or, eliminated, goes to the drop term.
+template <typename TV>
+__global__ void __launch_bounds__(TPB, 2) k32_spmv4(Geom g, const TV* __restrict__ val, const float* __restrict__ p,
+                                                    float* __restrict__ w, const uint16_t* __restrict__ mask,
+                                                    double* partials, PcgScalars* sc) {
+  if (sc_done(sc)) return;
+  DF dot;
+  const int n4 = (int)(g.n >> 2), nz = g.nz, npad = (int)g.npad;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n4; j += gridDim.x * blockDim.x) {
+    const int row = 4 * j, col = fdiv(g.nzd, row), k = row - col * nz;
+    const uint2 mk = __ldg(reinterpret_cast<const uint2*>(mask + row));
+    const uint32_t km[4] = {mk.x & 0xffffu, mk.x >> 16, mk.y & 0xffffu, mk.y >> 16};
+    float x[NNBR][6];   // entries k - 1 .. k + 4 of each neighbour column (unused ones never loaded)
+#pragma unroll
+    for (int q = 0; q < NNBR; ++q) {
+      const int nb = q == 0 ? col : nbr_of(g, col, q);
+      const bool up = q == 0 || (q & 1), down = q == 0 || !(q & 1);   // slots with dk = +1, dk = -1
+      const float* c = p + (nb >= 0 ? nb * nz + k : row);
+      float t[4];
+      ld4(c, t);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[q][u + 1] = t[u];
+      x[q][0] = down && k > 0 ? (nb >= 0 ? c[-1] : 0.f) : 0.f;
+      x[q][5] = up && k + 4 < nz ? (nb >= 0 ? c[4] : 0.f) : 0.f;
+    }
+    float sum[4] = {0.f, 0.f, 0.f, 0.f}, drop[4] = {0.f, 0.f, 0.f, 0.f}, diag[4];
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      float a[4];
+      ld4(val + s * npad + row, a);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (s == DIAG_SLOT) {
+          diag[u] = a[u];
+          continue;
+        }
+        const bool keep = (km[u] >> s) & 1u;
+        drop[u] += keep ? 0.f : a[u];
+        sum[u] = fmaf(keep ? a[u] : 0.f, x[slot_q(s)][u + 1 + slot_dk(s)] - x[0][u + 1], sum[u]);
+      }
+    }
+    float4 out;
+    float* o = &out.x;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float xi = x[0][u + 1];
+      o[u] = (km[u] & 0x8000u) ? xi : fmaf(diag[u] - drop[u], xi, sum[u]);
+      dot.add_prod(xi, o[u]);
+    }
+    *reinterpret_cast<float4*>(w + row) = out;
+  }
+  double v[1] = {dot.value()};
+  if (grid_sum<1>(v, partials, &sc->count[3]) && threadIdx.x == 0) {
+    const double pap = v[0];
+    sc->pAp = pap;
+    if (!(pap > 0.0) || !isfinite(pap)) {
+      sc->status = PM_BREAKDOWN;
+      sc->done = 1;
+    } else {
+      sc->alpha = sc->rho / pap;
+    }
+  }
+}
+
 template <int MASKC, typename TV>
 __global__ void __launch_bounds__(TPB, 4) k32_spmv(Geom g, const TV* __restrict__ val, const float* __restrict__ p,
                                                    float* __restrict__ w, const uint16_t* __restrict__ keep,
@@ -1736,6 +1834,22 @@ __global__ void __launch_bounds__(TPB) k32_pupd(int64_t n, const float* __restri
     const float zi = (STORED ? zbuf[i] : dinv[i] * r[i]) - c;
     p[i] = is_first ? zi : fmaf(beta, p[i], zi);
   }
+}
+
+// k32_pupd<1> after the first step, four entries per thread (16-byte loads: 4.7M rows 18.5 -> 13.8 us).
+__global__ void __launch_bounds__(TPB) k32_pupd4(int n, const float* __restrict__ z, float* __restrict__ p,
+                                                 const PcgScalars* sc) {
+  if (sc_done(sc)) return;
+  const float beta = (float)sc->beta, c = (float)sc->proj_c;
+  const int n4 = n >> 2, stride = gridDim.x * blockDim.x, t = blockIdx.x * blockDim.x + threadIdx.x;
+  const float4* z4 = reinterpret_cast<const float4*>(z);
+  float4* p4 = reinterpret_cast<float4*>(p);
+  for (int i = t; i < n4; i += stride) {
+    const float4 zi = z4[i], pi = p4[i];
+    p4[i] = make_float4(fmaf(beta, pi.x, zi.x - c), fmaf(beta, pi.y, zi.y - c), fmaf(beta, pi.z, zi.z - c),
+                        fmaf(beta, pi.w, zi.w - c));
+  }
+  for (int i = 4 * n4 + t; i < n; i += stride) p[i] = fmaf(beta, p[i], z[i] - c);
 }
 
 // m = hi + lo as two floats (hi = fl32(m), lo = fl32(m - hi)) for the FP32 kernels' m'z.
@@ -1873,25 +1987,27 @@ __global__ void __launch_bounds__(LINE_UCOLS) k32_update_line(Geom g, const floa
   }
 }
 
-// FP32 version of k_update_line_w (32-level columns, warp tasks of TC columns, no block
-// barriers); the FP32 correction d takes alpha p (folded into the FP64 x at each refinement) and
-// the dots are accumulated in compensated FP32. mode as k32_update_line: 0 first step, 1 a full
-// iteration. (r, z) = sum_k t_k y_k from the sweep (symmetric column blocks, see k_update_line_w).
-template <int PROJ, int TC>
+// FP32 version of k_update_line_w (warp tasks of TC columns, no block barriers), for any number of
+// levels that fits (NZ = 0: g.nz, rows of a task taken flat); the FP32 correction d takes alpha p (folded into
+// the FP64 x at each refinement) and the dots are accumulated in compensated FP32. mode as k32_update_line: 0
+// first step, 1 a full iteration. (r, z) = sum_k t_k y_k from the sweep (symmetric column blocks, see
+// k_update_line_w). Half-wide tasks (TC = 16): the FP32 pipe has room for idle lanes, and more tasks per warp keep
+// some warps streaming while others sweep.
+template <int PROJ, int TC, int NZ>
 __global__ void __launch_bounds__(LINE_WTPB, 4) k32_update_line_w(Geom g, const float* __restrict__ F,
                                                               float* __restrict__ d, float* __restrict__ r,
                                                               const float* __restrict__ p, const float* __restrict__ w,
                                                               float* __restrict__ z, const float2* __restrict__ m2,
                                                               double* partials, PcgScalars* sc, int mode) {
-  constexpr int NZ = LINE_WNZ, LD = NZ + 1;
   extern __shared__ float smf[];
   const int update = mode == 1;
   if (mode != 0 && sc_done(sc)) return;
   const double alpha_d = update ? sc->alpha : 0.0;
   const float alpha = (float)alpha_d;
+  const int nz = NZ > 0 ? NZ : g.nz, ld = nz | 1;
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
-  float* ws = smf + wib * (TC * LD);
+  float* ws = smf + wib * (TC * ld);
   const int ncols = g.ncols;
   const int n = (int)g.n;
   const int nwarps = gridDim.x * (LINE_WTPB / 32);
@@ -1899,31 +2015,37 @@ __global__ void __launch_bounds__(LINE_WTPB, 4) k32_update_line_w(Geom g, const 
   const int ntask = (ncols + TC - 1) / TC;
   const int tbeg = (int)((int64_t)ntask * wg / nwarps);
   const int tend = (int)((int64_t)ntask * (wg + 1) / nwarps);
+  // place of the task's i-th row in the tile of columns
+  const auto at = [&](int i) {
+    if (NZ > 0) return (i / (NZ > 0 ? NZ : 1)) * ld + i % (NZ > 0 ? NZ : 1);
+    const int c = fdiv(g.nzd, i);
+    return c * ld + i - c * nz;
+  };
   DF a[4];   // (r, r), (r, z), m'z, 1'r
   for (int t = tbeg; t < tend; ++t) {
     const int c0 = t * TC;
     const int cc = min(TC, ncols - c0);
-    const int row0 = c0 * NZ + lane;
+    const int row0 = c0 * nz, rows = cc * nz;
 #pragma unroll 8
-    for (int j = 0; j < cc; ++j) {
-      const int row = row0 + j * NZ;
+    for (int i = lane; i < rows; i += 32) {
+      const int row = row0 + i;
       float ri = r[row];
       if (update) {
         d[row] = fmaf(alpha, p[row], d[row]);
         ri = fmaf(-alpha, w[row], ri);
         r[row] = ri;
       }
-      ws[j * LD + lane] = ri;
+      ws[at(i)] = ri;
       a[0].add_prod(ri, ri);
       if (PROJ) a[3].add(ri);
     }
     __syncwarp();
     if (lane < cc) {
       const int col = c0 + lane;
-      float* cs = ws + lane * LD;
+      float* cs = ws + lane * ld;
       float y = 0.f;
 #pragma unroll 8
-      for (int k = 0; k < NZ; ++k) {
+      for (int k = 0; k < nz; ++k) {
         const int li = k * ncols + col;
         const float tk = fmaf(-F[li], y, cs[k]);
         y = tk * F[n + li];
@@ -1932,7 +2054,7 @@ __global__ void __launch_bounds__(LINE_WTPB, 4) k32_update_line_w(Geom g, const 
       }
       float zn = y;
 #pragma unroll 8
-      for (int k = NZ - 2; k >= 0; --k) {
+      for (int k = nz - 2; k >= 0; --k) {
         const int li = k * ncols + col;
         zn = fmaf(-F[2 * n + li], zn, cs[k]);
         cs[k] = zn;
@@ -1940,9 +2062,9 @@ __global__ void __launch_bounds__(LINE_WTPB, 4) k32_update_line_w(Geom g, const 
     }
     __syncwarp();
 #pragma unroll 8
-    for (int j = 0; j < cc; ++j) {
-      const int row = row0 + j * NZ;
-      const float zi = ws[j * LD + lane];
+    for (int i = lane; i < rows; i += 32) {
+      const int row = row0 + i;
+      const float zi = ws[at(i)];
       z[row] = zi;
       if (PROJ) add_mz(a[2], m2[row], zi);
     }
@@ -1983,45 +2105,34 @@ __global__ void __launch_bounds__(LINE_WTPB, 4) k32_update_line_w(Geom g, const 
   }
 }
 
-// The FP32 fused update + line solve (mode as k32_update_line): warp tasks for 32-level columns,
-// the block kernel otherwise. One launch; the caller counts it.
+// The FP32 fused update + line solve (mode as k32_update_line): warp tasks while a block's tiles fit
+// (LINE32_TILE), the block kernel for taller columns. One launch; the caller counts it.
+constexpr int LINE32_TC = 16;
+constexpr size_t LINE32_TILE = 100 * 1024;   // shared memory of a block's warp tiles: up to 199 levels
+
+template <int PROJ, int NZ>
+void launch_line32_w(pm_operator* op, int which, int mode, cudaStream_t s) {
+  SolveCtx* c = op->ctx;
+  const void* kern = (const void*)k32_update_line_w<PROJ, LINE32_TC, NZ>;
+  const size_t smem = (size_t)(LINE_WTPB / 32) * LINE32_TC * (op->nz | 1) * sizeof(float);
+  static const bool attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LINE32_TILE) == cudaSuccess;
+  (void)attr;
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, LINE_WTPB, smem);
+  // the resident blocks, capped by the partials buffer (4 lanes per block) and by one task per warp
+  const int64_t ntask = (op->ncols + LINE32_TC - 1) / LINE32_TC;
+  int64_t blocks = std::min<int64_t>((int64_t)std::max(1, per_sm) * op->num_sms, (int64_t)NPART * MAX_GRID / 4);
+  blocks = std::min<int64_t>(blocks, (ntask + LINE_WTPB / 32 - 1) / (LINE_WTPB / 32));
+  k32_update_line_w<PROJ, LINE32_TC, NZ><<<(int)std::max<int64_t>(1, blocks), LINE_WTPB, smem, s>>>(
+      geom_of(op), op->d_line32[which], c->d32, c->r32, c->p32, c->w32, c->z32, op->d_m2f, c->partials, c->sc_in, mode);
+}
+
 void update_line32(pm_operator* op, int which, bool proj, int mode, cudaStream_t s) {
   SolveCtx* c = op->ctx;
   Geom g = geom_of(op);
-  if (op->nz == LINE_WNZ) {
-    static int slots32 = 0, slots16 = 0;
-    auto slots_of = [&](const void* kern, int tc) {
-      const size_t sm = (size_t)(LINE_WTPB / 32) * tc * (LINE_WNZ + 1) * sizeof(float);
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      int per_sm = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, LINE_WTPB, sm);
-      return std::max(1, per_sm) * op->num_sms;
-    };
-    if (!slots32) {
-      slots32 = slots_of((const void*)k32_update_line_w<1, 32>, 32);
-      slots_of((const void*)k32_update_line_w<0, 32>, 32);
-      slots16 = slots_of((const void*)k32_update_line_w<1, 16>, 16);
-      slots_of((const void*)k32_update_line_w<0, 16>, 16);
-    }
-    // 32-column tasks while they fill the resident warps, else 16 (as update_line_w)
-    const bool wide = (op->ncols + 31) / 32 >= (int64_t)slots32 * (LINE_WTPB / 32);
-    const int tc = wide ? 32 : 16;
-    const size_t smem = (size_t)(LINE_WTPB / 32) * tc * (LINE_WNZ + 1) * sizeof(float);
-    int64_t blocks = std::min<int64_t>(wide ? slots32 : slots16, (int64_t)NPART * MAX_GRID / 4);
-    const int64_t ntask = (op->ncols + tc - 1) / tc;
-    blocks = std::min<int64_t>(blocks, (ntask + LINE_WTPB / 32 - 1) / (LINE_WTPB / 32));
-    const int grid = (int)std::max<int64_t>(1, blocks);
-#define PM_UL32(P, TCV)                                                                                   \
-  k32_update_line_w<P, TCV><<<grid, LINE_WTPB, smem, s>>>(g, op->d_line32[which], c->d32, c->r32, c->p32, c->w32, \
-                                                           c->z32, op->d_m2f, c->partials, c->sc_in, mode)
-    if (wide) {
-      if (proj) PM_UL32(1, 32);
-      else PM_UL32(0, 32);
-    } else {
-      if (proj) PM_UL32(1, 16);
-      else PM_UL32(0, 16);
-    }
-#undef PM_UL32
+  if ((size_t)(LINE_WTPB / 32) * LINE32_TC * (op->nz | 1) * sizeof(float) <= LINE32_TILE) {
+    if (op->nz == LINE_WNZ) proj ? launch_line32_w<1, LINE_WNZ>(op, which, mode, s) : launch_line32_w<0, LINE_WNZ>(op, which, mode, s);
+    else proj ? launch_line32_w<1, 0>(op, which, mode, s) : launch_line32_w<0, 0>(op, which, mode, s);
     return;
   }
   const int64_t ntiles = (op->ncols + LINE_UCOLS - 1) / LINE_UCOLS;
@@ -2121,13 +2232,15 @@ double bytes_per_refine(const pm_operator* op) { return (double)op->n * (15 * 8 
 
 // Whether the automatic choice runs a solve resident. Measured against the stream of kernels, us per
 // iteration, stream / resident:
-//   FP64  IC0 n = 0.12M 218 / 52, 0.29M 239 / 63, 0.99M 343 / 150, 2.0M 390 / 270, 4.9M 611 / 576;
-//         line 0.31M 64 / 35, 1.0M 110 / 88, 1.8M 152 / 130, 4.7M 319 / 327;
+//   FP64  IC0 n = 0.12M 132 / 51, 0.29M 170 / 63, 0.99M 231 / 150, 2.0M 266 / 269, 3.0M 336 / 362;
+//         line 0.31M 64 / 35, 1.0M 110 / 88, 1.8M 152 / 130, 4.7M 316 / 327;
 //         Jacobi 2.0M 140 / 126, 5.1M 275 / 296
-//   FP32  IC0 0.12M 226 / 46, 2.0M 360 / 195, 4.9M 472 / 427 (BF16 values 0.85M 296 / 98);
-//         line 0.31M 66 / 27, 1.0M 69 / 67, 1.8M 93 / 98; Jacobi 0.31M 73 / 21, 5.1M 196 / 201.
+//   FP32  IC0 0.12M 226 / 46, 2.0M 198 / 190, 3.0M 231 / 258; line 0.31M 40 / 25, 0.63M 48 / 32, 1.0M 67 / 62,
+//         4.7M 150 / 218; Jacobi 1.0M 77 / 41, 2.25M 112 / 98, 5.1M 196 / 201.
 bool resident_auto(const pm_operator* op, int prec, bool mixed) {
-  return op->n <= (mixed && prec == PM_PREC_LINE ? RESIDENT_AUTO_MIXED_LINE : RESIDENT_AUTO_ROWS);
+  return op->n <= (prec == PM_PREC_IC0             ? RESIDENT_AUTO_IC0
+                   : mixed && prec == PM_PREC_LINE ? RESIDENT_AUTO_MIXED_LINE
+                                                   : RESIDENT_AUTO_ROWS);
 }
 
 int resident_run(pm_operator* op, int which, const double* b, double* x, const pm_solve_opts* o,
@@ -2201,8 +2314,12 @@ void inner_iter(pm_operator* op, int which, const TV* val32, bool proj, int prec
   const int G = grid_for(op->n, TPB, op->num_sms);
   {
     KtScope t(PM_KT_SPMV, 1, s);
-    k32_spmv<MASKC, TV><<<G, TPB, 0, s>>>(g, val32, c->p32, c->w32, MASKC >= 0 ? op->d_keep[MASKC < 0 ? 0 : MASKC] : nullptr,
-                                          c->partials, c->sc_in);
+    if (op->nz % 4 == 0)
+      k32_spmv4<TV><<<grid_for(op->n / 4, TPB, op->num_sms), TPB, 0, s>>>(
+          g, val32, c->p32, c->w32, MASKC >= 0 ? op->d_keep[MASKC < 0 ? 0 : MASKC] : op->d_struct, c->partials, c->sc_in);
+    else
+      k32_spmv<MASKC, TV><<<G, TPB, 0, s>>>(g, val32, c->p32, c->w32, MASKC >= 0 ? op->d_keep[MASKC < 0 ? 0 : MASKC] : nullptr,
+                                            c->partials, c->sc_in);
   }
   if (prec == PM_PREC_LINE) {
     {
@@ -2211,7 +2328,7 @@ void inner_iter(pm_operator* op, int which, const TV* val32, bool proj, int prec
     }
     {
       KtScope t(PM_KT_PUPDATE, 1, s);
-      k32_pupd<1><<<G, TPB, 0, s>>>(op->n, c->r32, dinv32, c->z32, c->p32, c->sc_in, 0);
+      k32_pupd4<<<grid_for(op->n / 4 + 1, TPB, op->num_sms), TPB, 0, s>>>((int)op->n, c->z32, c->p32, c->sc_in);
     }
     count_launch(3);
   } else if (prec == PM_PREC_IC0) {
