@@ -183,36 +183,13 @@ int pm_assemble_operator(const pm_mesh_desc* mesh, const pm_physics* phys, pm_op
         cls_cols.push_back(c);
       }
   const int nc = hm.ncols;
-  // columns class by class, index within the class, i, j; neighbour columns in class order, entry by entry; the
-  // same by their index within their own class (-1: none); first colour-ordered position of each
-  // column's even and odd levels
-  std::vector<int32_t> packed((size_t)(6 + 2 * NNBR) * nc);
-  std::copy(cls_cols.begin(), cls_cols.end(), packed.begin());
-  std::copy(clsidx.begin(), clsidx.end(), packed.begin() + nc);
-  std::copy(hm.col_i.begin(), hm.col_i.end(), packed.begin() + 2 * (size_t)nc);
-  std::copy(hm.col_j.begin(), hm.col_j.end(), packed.begin() + 3 * (size_t)nc);
-  int32_t* cn = packed.data() + 4 * (size_t)nc;
-  int32_t* cc = cn + (size_t)NNBR * nc;
-  int32_t* cp = cc + (size_t)NNBR * nc;
-  for (int i = 0; i < nc; ++i) {
-    const int32_t* nb = hm.nbr.data() + (size_t)cls_cols[i] * NNBR;
-    for (int q = 0; q < NNBR; ++q) {
-      const int32_t c = q == 0 ? cls_cols[i] : nb[q];
-      cn[(size_t)q * nc + i] = c;
-      cc[(size_t)q * nc + i] = c < 0 ? -1 : clsidx[c];
-    }
-  }
-  const int nlev[2] = {(mesh->nz + 1) / 2, mesh->nz / 2};
-  for (int par = 0; par < 2; ++par) {
-    int64_t base[4], acc = par ? (int64_t)nc * nlev[0] : 0;
-    for (int cls = 0; cls < 4; ++cls) {
-      base[cls] = acc;
-      acc += (int64_t)op->cls_count[cls] * nlev[par];
-    }
-    for (int c = 0; c < nc; ++c)
-      cp[(size_t)par * nc + c] =
-          (int32_t)(base[(hm.col_i[c] & 1) | ((hm.col_j[c] & 1) << 1)] + (int64_t)clsidx[c] * nlev[par]);
-  }
+  // columns class by class, index within the class, i, j (the tables in class order follow on the device)
+  std::vector<int32_t> packed;
+  packed.reserve((size_t)4 * nc);
+  packed.insert(packed.end(), cls_cols.begin(), cls_cols.end());
+  packed.insert(packed.end(), clsidx.begin(), clsidx.end());
+  packed.insert(packed.end(), hm.col_i.begin(), hm.col_i.end());
+  packed.insert(packed.end(), hm.col_j.begin(), hm.col_j.end());
 #define PM_TRY(x)           \
   do {                      \
     int _e = (x);           \

@@ -308,6 +308,26 @@ __global__ void k_keep_masks(Geom g, uint16_t* __restrict__ k0, uint16_t* __rest
   }
 }
 
+// Tables of the IC0 sweeps: neighbour columns of the i-th column in class order (entry 0: that column), the same by
+// their index within their class (-1: none), and each column's first colour-ordered positions.
+__global__ void k_class_tables(Geom g, ColourMap cm, const int32_t* __restrict__ cls_cols, int32_t* __restrict__ cnbr,
+                               int32_t* __restrict__ ccls, int32_t* __restrict__ colpos) {
+  const int nc = g.ncols;
+  const int32_t* clsidx = cls_cols + nc;
+  const int32_t* coli = clsidx + nc;
+  const int32_t* colj = coli + nc;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
+    const int col = cls_cols[i];
+    for (int q = 0; q < NNBR; ++q) {
+      const int nb = q == 0 ? col : nbr_of(g, col, q);
+      cnbr[q * nc + i] = nb;
+      ccls[q * nc + i] = nb < 0 ? -1 : clsidx[nb];
+    }
+    const int cls = (coli[i] & 1) | ((colj[i] & 1) << 1);
+    for (int par = 0; par < 2; ++par) colpos[par * nc + i] = (int)node_pos(cm, clsidx, i, cls, par);
+  }
+}
+
 __global__ void k_recip(double* __restrict__ d, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     d[i] = 1.0 / d[i];
@@ -337,6 +357,9 @@ ColourMap colour_map(const pm_operator* op) {
 
 int launch_assemble(pm_operator* op, cudaStream_t s) {
   Geom g = geom_of(op);
+  k_class_tables<<<grid_for(op->ncols, 128, op->num_sms), 128, 0, s>>>(g, colour_map(op), op->d_cls_cols, op->d_cnbr,
+                                                                       op->d_ccls, op->d_colpos);
+  count_launch();
   const int threads = 128;
   const int grid = grid_for(op->n, threads, op->num_sms);
   const double a2 = 1.5 / op->dt, a1 = 1.0 / op->dt;
