@@ -115,37 +115,38 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sm) {
   __syncthreads();
 }
 
-constexpr long long SPIN_LIMIT = 1ll << 24;  // x ~100 ns sleep: about 2 s
+constexpr uint32_t SPIN_LIMIT = 1u << 22;  // polls of about half a microsecond: about 2 s
 
 // Bounded grid barrier; returns false (and records PM_TIMEOUT) when the wait expires or another
-// block already gave up.
+// block already gave up. Thread 0's release after the block barrier publishes the whole block's stores and its
+// acquire covers the block's later loads, so no other thread fences; the waiting thread polls without a sleep.
+// (With a fence in every thread, a 100 ns sleep between polls and a last look at the error word, a
+// 24-system batch of 4.5M rows took 188.6 ms, 185.2 without.)
 __device__ bool grid_barrier(Ctl* ctl) {
   __shared__ int ok_s;
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    volatile uint32_t* genp = &ctl->bar_gen;
-    const uint32_t g0 = *genp;
-    __threadfence();
-    const uint32_t arrived = atomicAdd(&ctl->bar_count, 1u) + 1u;
-    if (arrived == gridDim.x) {
+    uint32_t g0, arrived, g;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(g0) : "l"(&ctl->bar_gen) : "memory");
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(&ctl->bar_count) : "memory");
+    if (arrived + 1 == gridDim.x) {
       ctl->bar_count = 0;
-      __threadfence();
-      atomicAdd(&ctl->bar_gen, 1u);
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar_gen) : "memory");
     } else {
-      long long spins = 0;
-      while (*genp == g0) {
-        if (*((volatile int32_t*)&ctl->err) != 0 || ++spins > SPIN_LIMIT) {
+      uint32_t spins = 0;
+      for (;;) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&ctl->bar_gen) : "memory");
+        if (g != g0) break;
+        ++spins;
+        if (spins > SPIN_LIMIT || ((spins & 1023u) == 0 && *((volatile int32_t*)&ctl->err) != 0)) {
           atomicExch(&ctl->err, PM_TIMEOUT);
           ok = 0;
           break;
         }
-        __nanosleep(100);
       }
     }
-    __threadfence();
-    ok_s = ok && *((volatile int32_t*)&ctl->err) == 0;
+    ok_s = ok;
   }
   __syncthreads();
   return ok_s != 0;
@@ -486,16 +487,14 @@ __device__ __forceinline__ bool owns_ic0_chunk(const Sys& S, int c) {
     if (!grid_barrier(ctl)) return;                                                                 \
   }
 
-// Resident blocks of 256 threads per SM the register budget is sized for: 3 (80 registers, about
-// 1 KB of spills per thread) keeps 24 warps per SM in flight. The kernel is latency-bound, and on
-// the batched 64-basin workloads 3 measured faster than 2 (128 registers, no spills): IC0 mass
-// systems 0.41 -> 0.36 s, the FP32 line batch 8.84 -> 8.49 s.
-#ifndef PM_BATCH_MINB
-#define PM_BATCH_MINB 3
-#endif
-
-template <typename T>
-__global__ void __launch_bounds__(256, PM_BATCH_MINB) k_batch(const Sys* __restrict__ sys, Scal* scal, int nsys,
+// MINB: resident blocks of 256 threads per SM that the register budget is sized for. 3 (80 registers, about
+// 1 KB of spills per thread) keeps 24 warps per SM in flight, 2 (128 registers) spills almost nothing. With many
+// tiles for each block 3 measured faster (64-basin batches: IC0 mass systems 0.41 -> 0.36 s, FP32 line
+// 8.84 -> 8.49 s); with few, when a phase is one tile's chain of loads and arithmetic, 2 is: 24 FP32 systems of 4.5M rows
+// (1200 tiles) 300 us per iteration either way, and 160 -> 110 us once only six systems iterate.
+constexpr int64_t FEW_TILES = 2400;   // up to about eight per block of the two-block kernel
+template <typename T, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys, Scal* scal, int nsys,
                                                int ntiles, double* part, Ctl* ctl,
                                                int quantum, int init, int ic0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -961,10 +960,16 @@ int prepare_for_batch(pm_operator* op, int which, int prec, int precision, cudaS
 namespace batch {
 namespace {
 
-template <typename T>
-int max_blocks(int block, size_t smem) {
+using Kernel = void (*)(const Sys*, Scal*, int, int, double*, Ctl*, int, int, int);
+Kernel kernel_of(int precision, bool few_tiles) {
+  if (precision == PM_FP64) return few_tiles ? &k_batch<double, 2> : &k_batch<double, 3>;
+  return few_tiles ? &k_batch<float, 2> : &k_batch<float, 3>;
+}
+// Resident blocks per SM (0: the shape does not fit).
+int max_blocks(Kernel k, int block, size_t smem) {
+  cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
   int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<T>, block, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, smem);
   return nb;
 }
 
@@ -1101,8 +1106,7 @@ int build_layout(pm_batch* bt) {
   return st;
 }
 
-template <typename T>
-cudaError_t launch_k(int grid, int block, size_t smem, const Sys* d_sys, Scal* d_scal, int nsys, int ntiles, double* d_part, Ctl* d_ctl, int quantum, int init, int ic0, cudaStream_t s) {
+cudaError_t launch_k(Kernel k, int grid, int block, size_t smem, const Sys* d_sys, Scal* d_scal, int nsys, int ntiles, double* d_part, Ctl* d_ctl, int quantum, int init, int ic0, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
@@ -1114,12 +1118,13 @@ cudaError_t launch_k(int grid, int block, size_t smem, const Sys* d_sys, Scal* d
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   count_launch();
-  return cudaLaunchKernelEx(&cfg, k_batch<T>, d_sys, d_scal, nsys, ntiles, d_part, d_ctl, quantum, init, ic0);
+  return cudaLaunchKernelEx(&cfg, k, d_sys, d_scal, nsys, ntiles, d_part, d_ctl, quantum, init, ic0);
 }
 
-template <typename T>
+Kernel kernel_of(const pm_batch* bt) { return kernel_of(bt->precision, bt->ntiles <= FEW_TILES && !bt->any_ic0); }
+
 cudaError_t launch(pm_batch* bt, int quantum, int init, cudaStream_t s) {
-  return launch_k<T>(bt->grid, bt->block, smem_bytes(bt), bt->d_sys, bt->d_scal, (int)bt->count,
+  return launch_k(kernel_of(bt), bt->grid, bt->block, smem_bytes(bt), bt->d_sys, bt->d_scal, (int)bt->count,
                      (int)bt->ntiles, bt->d_part, bt->d_ctl, quantum, init, bt->any_ic0 ? 1 : 0, s);
 }
 
@@ -1148,9 +1153,7 @@ int capture_graph(cudaGraphExec_t* exec, F fn) {
 
 int set_grid(pm_batch* bt) {
   const size_t smem = smem_bytes(bt);
-  cudaFuncSetAttribute(k_batch<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-  cudaFuncSetAttribute(k_batch<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-  const int per_sm = bt->precision == PM_FP64 ? max_blocks<double>(bt->block, smem) : max_blocks<float>(bt->block, smem);
+  const int per_sm = max_blocks(kernel_of(bt), bt->block, smem);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device);
   if (per_sm <= 0) return set_error(PM_EINVAL, "batched kernel cannot be resident with this block / tile shape");
@@ -1173,7 +1176,7 @@ int start(pm_batch* bt, cudaStream_t s) {
   if (!st) st = cuda_check(cudaMemcpyAsync(bt->d_scal, hs.data(), bt->count * sizeof(Scal), cudaMemcpyHostToDevice, s), "scal");
   if (!st) st = cuda_check(cudaMemcpyAsync(bt->d_ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s), "ctl");
   if (st) return st;
-  const cudaError_t e = bt->precision == PM_FP64 ? launch<double>(bt, 0, 1, s) : launch<float>(bt, 0, 1, s);
+  const cudaError_t e = launch(bt, 0, 1, s);
   return cuda_check(e, "batched PCG init launch");
 }
 
@@ -1181,7 +1184,7 @@ int run_to_completion(pm_batch* bt, cudaStream_t s, int quantum) {
   // capture one quantum launch in a CUDA graph once, replay it until no system is active
   if (!bt->graph || bt->graph_quantum != quantum) {
     const int st = capture_graph(&bt->graph, [&](cudaStream_t cs) {
-      return bt->precision == PM_FP64 ? launch<double>(bt, quantum, 0, cs) : launch<float>(bt, quantum, 0, cs);
+      return launch(bt, quantum, 0, cs);
     });
     if (st) return st;
     bt->graph_quantum = quantum;
@@ -1279,7 +1282,7 @@ int autotune(pm_batch* bt, cudaStream_t s) {
       }
       if (start(bt, s)) continue;
       cudaEventRecord(e0, s);
-      const cudaError_t le = bt->precision == PM_FP64 ? launch<double>(bt, 8, 0, s) : launch<float>(bt, 8, 0, s);
+      const cudaError_t le = launch(bt, 8, 0, s);
       cudaEventRecord(e1, s);
       if (le != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) continue;
       Ctl h;
@@ -1545,9 +1548,7 @@ extern "C" int pm_server_create(int32_t slots, int32_t nz_cap, const pm_solve_op
   const size_t smem = server_smem(sv);
   int st = smem > 160 * 1024 ? set_error(PM_EINVAL, "tile_cols x (nz_cap + 1) does not fit in shared memory") : PM_OK;
   if (!st) {
-    cudaFuncSetAttribute(k_batch<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    cudaFuncSetAttribute(k_batch<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    const int per_sm = sv->precision == PM_FP64 ? max_blocks<double>(block, smem) : max_blocks<float>(block, smem);
+    const int per_sm = max_blocks(kernel_of(sv->precision, false), block, smem);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, sv->device);
     if (per_sm <= 0) st = set_error(PM_EINVAL, "server kernel cannot be resident with this block / tile shape");
@@ -1669,11 +1670,8 @@ extern "C" int pm_server_run(pm_server* sv, int32_t quantum, int32_t* active, pm
   if (!sv->graph || sv->graph_quantum != quantum || sv->graph_tcap != sv->tcap || sv->graph_ic0 != ic0) {
     const size_t smem = server_smem(sv);
     st = capture_graph(&sv->graph, [&](cudaStream_t cs) {
-      return sv->precision == PM_FP64
-                 ? launch_k<double>(sv->grid, sv->block, smem, sv->d_sys, sv->d_scal, sv->cap,
-                                    (int)sv->tcap, sv->d_part, sv->d_ctl, quantum, 0, ic0, cs)
-                 : launch_k<float>(sv->grid, sv->block, smem, sv->d_sys, sv->d_scal, sv->cap,
-                                   (int)sv->tcap, sv->d_part, sv->d_ctl, quantum, 0, ic0, cs);
+      return launch_k(kernel_of(sv->precision, false), sv->grid, sv->block, smem, sv->d_sys, sv->d_scal, sv->cap,
+                      (int)sv->tcap, sv->d_part, sv->d_ctl, quantum, 0, ic0, cs);
     });
     if (st) return st;
     sv->graph_quantum = quantum;
