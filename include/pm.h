@@ -120,10 +120,10 @@ typedef struct pm_solve_opts {
   int32_t x0_is_guess;   /* 1: x holds the initial guess; 0: start from x = 0               */
   int32_t max_restarts;  /* true-residual restarts after the recursive test passes (FP64)   */
   double inner_rtol;     /* mixed precision: relative reduction asked of each inner solve  */
-  int32_t kernel;        /* FP64 solves: PM_KERNEL_AUTO (resident up to 2M to 3M rows),
+  int32_t kernel;        /* PM_KERNEL_AUTO (resident up to 1.3M to 3M rows),
                             PM_KERNEL_STREAM (one launch per PCG phase), or
-                            PM_KERNEL_RESIDENT (one launch runs the whole solve, n <= 2^20).
-                            Mixed-precision solves run as AUTO                              */
+                            PM_KERNEL_RESIDENT (one launch runs the whole solve, n <= 2^20;
+                            mixed-precision solves run as AUTO)                             */
   int32_t pad;
 } pm_solve_opts;
 
@@ -380,7 +380,8 @@ int pm_last_error(char* buf, int32_t len);
 int64_t pm_kernel_launch_count(void);
 
 /* Live kernel timing. When enabled, the PCG driver brackets every launch of the kernel classes
- * below with CUDA events on the solve's stream and accumulates their elapsed times at its own
+ * below (stream solves; a resident solve is one launch of none of these classes) with CUDA events
+ * on the solve's stream and accumulates their elapsed times at its own
  * synchronisation points. pm_kernel_timing(enable) switches it and resets the totals;
  * pm_kernel_timing_get returns the total milliseconds and launch count of one class. Process-
  * global and not thread-safe; a measurement aid, off by default. */

@@ -29,8 +29,8 @@
 // sweep can form p at once. The pressure's projection needs m'z first: its IC0 sums and p follow the
 // sweeps as passes of their own.
 //
-// What bounds it: barriers and load latency below about 0.3M rows (IC0 52 us per iteration at 0.12M rows, where the
-// stream of kernels takes 218), the FP64 pipe (64 cycles per warp instruction and sub-core) above.
+// What bounds it: barriers and load latency below about 0.3M rows (IC0 51 us per iteration at 0.12M rows, where a
+// stream of kernels took 218), the FP64 pipe (64 cycles per warp instruction and sub-core) above.
 #pragma once
 
 #include <cuda_bf16.h>

@@ -740,11 +740,10 @@ __global__ void __launch_bounds__(LINE_TPB) k_line_rho(Geom g, const double* __r
 }
 
 // One PCG iteration's update with the vertical-line preconditioner fused in:
-//   x += alpha p, r -= alpha w (rows of LINE_UCOLS whole columns, staged in shared memory),
+//   x += alpha p, r -= alpha w (rows of LINE_FCOLS whole columns, staged in shared memory),
 //   z = P^{-1} r column by column (one thread per column, in place), then the reductions
 //   (r, r), (r, z) [m'z, 1'r]. The last block tests convergence on (r, r) and forms beta, as
 //   k_cg_update + k_line_rho would; the z of the converged iteration is simply not used.
-constexpr int LINE_UCOLS = 128;   // FP32 fused kernel: columns (= threads) per block
 #ifndef PM_LINE_FCOLS
 #define PM_LINE_FCOLS 64
 #endif
@@ -1885,112 +1884,10 @@ __global__ void k_cvt(int64_t n, const double* __restrict__ in, T* __restrict__ 
   }
 }
 
-// FP32 vertical-line solve fused with the inner update (as k_update_line).
-template <int PROJ>
-__global__ void __launch_bounds__(LINE_UCOLS) k32_update_line(Geom g, const float* __restrict__ F,
-                                                            float* __restrict__ d, float* __restrict__ r,
-                                                            const float* __restrict__ p, const float* __restrict__ w,
-                                                            float* __restrict__ z, const float2* __restrict__ m2,
-                                                            double* partials, PcgScalars* sc, int mode) {
-  // mode 0: first step (z, rho, beta = 0); 1: a full iteration (d, r update, z, rho, beta)
-  extern __shared__ float smf[];
-  const int update = mode == 1;
-  if (mode != 0 && sc_done(sc)) return;
-  const double alpha_d = update ? sc->alpha : 0.0;
-  const float alpha = (float)alpha_d;
-  const int nz = g.nz, ld = nz + 1;
-  const int ncols = g.ncols;
-  const int n = (int)g.n;
-  const int ntiles = (ncols + LINE_UCOLS - 1) / LINE_UCOLS;
-  DF a[4];
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int c0 = tile * LINE_UCOLS;
-    const int cc = min(LINE_UCOLS, ncols - c0);
-    const int row0 = c0 * nz;
-    const int rows = cc * nz;
-    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-      const int row = row0 + i;
-      float ri = r[row];
-      if (update) {
-        d[row] = fmaf(alpha, p[row], d[row]);
-        ri = fmaf(-alpha, w[row], ri);
-        r[row] = ri;
-      }
-      smf[(i / nz) * ld + i % nz] = ri;
-      a[0].add_prod(ri, ri);
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < cc) {
-      const int col = c0 + threadIdx.x;
-      float* col_s = smf + threadIdx.x * ld;
-      float y = 0.f;
-#pragma unroll 4
-      for (int k = 0; k < nz; ++k) {
-        const int li = k * ncols + col;
-        y = (col_s[k] - F[li] * y) * F[n + li];
-        col_s[k] = y;
-      }
-      float zn = y;
-#pragma unroll 4
-      for (int k = nz - 2; k >= 0; --k) {
-        const int li = k * ncols + col;
-        zn = fmaf(-F[2 * n + li], zn, col_s[k]);
-        col_s[k] = zn;
-      }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-      const int row = row0 + i;
-      const float zi = smf[(i / nz) * ld + i % nz];
-      const float ri = r[row];
-      z[row] = zi;
-      a[1].add_prod(ri, zi);
-      if (PROJ) {
-        add_mz(a[2], m2[row], zi);
-        a[3].add(ri);
-      }
-    }
-    __syncthreads();
-  }
-  double v[4] = {a[0].value(), a[1].value(), a[2].value(), a[3].value()};
-  if (grid_sum<4>(v, partials, &sc->count[4]) && threadIdx.x == 0) {
-    const double c = PROJ ? v[2] / sc->one_m : 0.0;
-    const double rho_new = v[1] - c * v[3];
-    if (mode == 0) {
-      sc->proj_c = c;
-      sc->rho = rho_new;
-      sc->beta = 0.0;
-      if ((!(rho_new > 0.0) || !isfinite(rho_new)) && !sc->done) {
-        sc->status = PM_BREAKDOWN;
-        sc->done = 1;
-      }
-    } else {
-      sc->iter += 1;
-      sc->rr = v[0];
-      if (v[0] <= sc->tol2) {
-        sc->done = 1;
-      } else if (sc->iter >= sc->max_iter) {
-        sc->status = PM_NOT_CONVERGED;
-        sc->done = 1;
-      } else if (v[0] <= sc->aux[2]) {
-        sc->done = 2;
-      } else {
-        sc->proj_c = c;
-        sc->beta = rho_new / sc->rho;
-        sc->rho = rho_new;
-        if (!(rho_new > 0.0) || !isfinite(rho_new)) {
-          sc->status = PM_BREAKDOWN;
-          sc->done = 1;
-        }
-      }
-    }
-  }
-}
-
 // FP32 version of k_update_line_w (warp tasks of TC columns, no block barriers), for any number of
 // levels that fits (NZ = 0: g.nz, rows of a task taken flat); the FP32 correction d takes alpha p (folded into
-// the FP64 x at each refinement) and the dots are accumulated in compensated FP32. mode as k32_update_line: 0
-// first step, 1 a full iteration. (r, z) = sum_k t_k y_k from the sweep (symmetric column blocks, see
+// the FP64 x at each refinement) and the dots are accumulated in compensated FP32. mode 0: first step (z,
+// rho, beta = 0); 1: a full iteration (d, r update, z, rho, beta). (r, z) = sum_k t_k y_k from the sweep (symmetric column blocks, see
 // k_update_line_w). Half-wide tasks (TC = 16): the FP32 pipe has room for idle lanes, and more tasks per warp keep
 // some warps streaming while others sweep.
 template <int PROJ, int TC, int NZ>
@@ -2105,16 +2002,16 @@ __global__ void __launch_bounds__(LINE_WTPB, 4) k32_update_line_w(Geom g, const 
   }
 }
 
-// The FP32 fused update + line solve (mode as k32_update_line): warp tasks while a block's tiles fit
-// (LINE32_TILE), the block kernel for taller columns. One launch; the caller counts it.
+// The FP32 fused update + line solve (mode as k32_update_line_w). One launch; the caller counts it.
 constexpr int LINE32_TC = 16;
-constexpr size_t LINE32_TILE = 100 * 1024;   // shared memory of a block's warp tiles: up to 199 levels
+constexpr size_t LINE32_TILE = 200 * 1024;   // shared memory of a block's warp tiles: up to 399 levels
+size_t line32_tile(int nz) { return (size_t)(LINE_WTPB / 32) * LINE32_TC * (nz | 1) * sizeof(float); }
 
 template <int PROJ, int NZ>
 void launch_line32_w(pm_operator* op, int which, int mode, cudaStream_t s) {
   SolveCtx* c = op->ctx;
   const void* kern = (const void*)k32_update_line_w<PROJ, LINE32_TC, NZ>;
-  const size_t smem = (size_t)(LINE_WTPB / 32) * LINE32_TC * (op->nz | 1) * sizeof(float);
+  const size_t smem = line32_tile(op->nz);
   static const bool attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LINE32_TILE) == cudaSuccess;
   (void)attr;
   int per_sm = 0;
@@ -2128,22 +2025,8 @@ void launch_line32_w(pm_operator* op, int which, int mode, cudaStream_t s) {
 }
 
 void update_line32(pm_operator* op, int which, bool proj, int mode, cudaStream_t s) {
-  SolveCtx* c = op->ctx;
-  Geom g = geom_of(op);
-  if ((size_t)(LINE_WTPB / 32) * LINE32_TC * (op->nz | 1) * sizeof(float) <= LINE32_TILE) {
-    if (op->nz == LINE_WNZ) proj ? launch_line32_w<1, LINE_WNZ>(op, which, mode, s) : launch_line32_w<0, LINE_WNZ>(op, which, mode, s);
-    else proj ? launch_line32_w<1, 0>(op, which, mode, s) : launch_line32_w<0, 0>(op, which, mode, s);
-    return;
-  }
-  const int64_t ntiles = (op->ncols + LINE_UCOLS - 1) / LINE_UCOLS;
-  int grid = (int)std::min<int64_t>(ntiles, std::min<int64_t>((int64_t)op->num_sms * 8, MAX_GRID));
-  const size_t smem = (size_t)LINE_UCOLS * (op->nz + 1) * sizeof(float);
-  if (proj)
-    k32_update_line<1><<<grid, LINE_UCOLS, smem, s>>>(g, op->d_line32[which], c->d32, c->r32, c->p32, c->w32, c->z32,
-                                                      op->d_m2f, c->partials, c->sc_in, mode);
-  else
-    k32_update_line<0><<<grid, LINE_UCOLS, smem, s>>>(g, op->d_line32[which], c->d32, c->r32, c->p32, c->w32, c->z32,
-                                                      op->d_m2f, c->partials, c->sc_in, mode);
+  if (op->nz == LINE_WNZ) proj ? launch_line32_w<1, LINE_WNZ>(op, which, mode, s) : launch_line32_w<0, LINE_WNZ>(op, which, mode, s);
+  else proj ? launch_line32_w<1, 0>(op, which, mode, s) : launch_line32_w<0, 0>(op, which, mode, s);
 }
 
 int ensure_mixed(pm_operator* op, int which, int precision, int prec, cudaStream_t s) {
@@ -2383,6 +2266,8 @@ int mixed_run(pm_operator* op, int which, const double* b, double* x, const pm_s
   const int prec = o->prec;
   const double* val64 = op->d_val[which_valset(which)];
   int st;
+  if (prec == PM_PREC_LINE && line32_tile(op->nz) > LINE32_TILE)
+    return set_error(PM_ECUDA, "line preconditioner: columns too tall for shared memory");
   if ((st = ensure_prec(op, which, prec, s))) return st;
   if ((st = ensure_mixed(op, which, o->precision, prec, s))) return st;
   const int vs = which_valset(which);
@@ -2593,11 +2478,11 @@ int pcg_solve(pm_operator* op, int which, const double* b, double* x, const pm_s
   NvtxRange range(std::string("pcg ") + which_name(which) + " " + prec_name(o->prec) + " " + precision_name(o->precision));
   int r = ensure_ctx(op);
   if (r) return r;
-  // the kernel choice (and its limit) is of FP64 solves; a mixed-precision one runs as AUTO
-  const bool mixed = o->precision != PM_FP64;
-  if (!mixed && o->kernel == PM_KERNEL_RESIDENT && op->n > RESIDENT_MAX_ROWS)
+  // PM_KERNEL_RESIDENT (and its limit) is of FP64 solves; a mixed-precision one runs as AUTO then
+  const bool mixed = o->precision != PM_FP64, asked = !mixed && o->kernel == PM_KERNEL_RESIDENT;
+  if (asked && op->n > RESIDENT_MAX_ROWS)
     return set_error(PM_EINVAL, "PM_KERNEL_RESIDENT: at most " + std::to_string(RESIDENT_MAX_ROWS) + " rows");
-  if (!mixed && o->kernel != PM_KERNEL_AUTO ? o->kernel == PM_KERNEL_RESIDENT : resident_auto(op, o->prec, mixed))
+  if (asked || (o->kernel != PM_KERNEL_STREAM && resident_auto(op, o->prec, mixed)))
     return resident_run(op, which, b, x, o, st, s);
   if (o->precision == PM_FP32_REFINE) {
     switch (which_mask(which)) {
