@@ -514,10 +514,12 @@ __device__ __forceinline__ int colour_pos(const SweepGeo& g, int row) {
 //
 // Launched ahead of the previous kernel's end (programmatic dependent launch): a block that finds room
 // while that kernel's last blocks run fetches its factor row and neighbour indices, which no kernel of a solve
-// writes, and waits for the previous kernel only then.
+// writes, and waits for the previous kernel only then. r and y are not __restrict__: earlier kernels write them
+// while this one is already resident, so neither may be read as constant for the kernel's life (ld.global.nc,
+// or a load moved above the wait).
 template <int C, int FWD, typename T>
-__global__ void __launch_bounds__(TPB, 4) k_ic0_sweep(SweepGeo g, const T* __restrict__ F, const T* __restrict__ r,
-                                                      T* y, const PcgScalars* sc, int check_done) {
+__global__ void __launch_bounds__(TPB, 4) k_ic0_sweep(SweepGeo g, const T* __restrict__ F, const T* r, T* y,
+                                                      const PcgScalars* sc, int check_done) {
   asm volatile("griddepcontrol.launch_dependents;");
   constexpr int kpar = C >> 2, cls = C & 3;
   const int total = g.cls_cnt[cls] * g.nlev[kpar].d;
