@@ -929,7 +929,9 @@ template <typename T, typename TV, int PREC, bool CL>
 inline int launch_one(Args& a, int grid, size_t smem, cudaStream_t s) {
   const void* f = (const void*)k_resident<T, TV, PREC, CL>;
   int st;
-  if (smem && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+  // the limit belongs to the function, not to the launch: always the same value, since other threads launch tiles
+  // of other sizes between this call and the launch
+  if (smem && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_LIMIT),
                                "resident shared memory")))
     return st;
   if (CL && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster size")))
