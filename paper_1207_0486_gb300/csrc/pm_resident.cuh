@@ -825,7 +825,7 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c
   if (bb == 0.0) {
     for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.x[i] = 0.0;
   } else if (rr <= tol2 || a.max_iter == 0) {   // x0 already meets rtol, or no iteration is allowed
-    if (rr > tol2) cg.status = PM_NOT_CONVERGED;
+    if (!(rr <= tol2)) cg.status = PM_NOT_CONVERGED;   // not a number included
     rel_true = sqrt(rr / bb);
   } else {
     for (;;) {
@@ -871,7 +871,7 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c
         break;
       }
       if (cg.iter >= a.max_iter) {   // no iteration left: accepted only below the floor
-        if (rel_true > floor) cg.status = PM_NOT_CONVERGED;
+        if (!(rel_true <= floor)) cg.status = PM_NOT_CONVERGED;
         break;
       }
     }
