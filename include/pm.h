@@ -252,8 +252,9 @@ int pm_batch_info(const pm_batch* batch, int32_t* tile_cols, int32_t* block, int
 void pm_batch_destroy(pm_batch* batch);
 /* Test aid for failure detection: launches a two-block cooperative kernel in which one block
  * leaves without reaching the grid barrier, so the other block's bounded wait expires (about 2 s).
- * Returns the status that wait recorded: PM_TIMEOUT. Nothing faults, traps or hangs, and the
- * context stays usable. */
+ * Then a resident solve's barrier (pm_pcg_solve) waits for a block that never arrives, and a result
+ * is reported after that wait has run out. Returns the status of the two: PM_TIMEOUT. Nothing
+ * faults, traps or hangs, and the context stays usable. */
 int pm_debug_barrier_timeout(pm_stream stream);
 /* One-shot: create (no autotuning), solve, destroy. */
 int pm_pcg_solve_batched(pm_operator* const* ops, const pm_which* which, const double* const* b,

@@ -1774,6 +1774,6 @@ extern "C" int pm_debug_barrier_timeout(pm_stream stream) {
   if (!st) st = cuda_check(cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s), "probe copy");
   if (!st) st = cuda_check(cudaStreamSynchronize(s), "probe sync");
   cudaFree(d);
-  if (st) return st;
-  return h.err;
+  if (st || h.err != PM_TIMEOUT) return st ? st : h.err;
+  return pm::resident::debug_timeout(s);
 }

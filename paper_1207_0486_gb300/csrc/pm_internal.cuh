@@ -392,6 +392,10 @@ namespace pm {
 
 // error reporting (pm_api.cu)
 int set_error(int status, const std::string& msg);
+namespace resident {
+// Test aid: what a resident solve returns when one block's wait runs out and rank 0 reports a result after it.
+int debug_timeout(cudaStream_t s);
+}  // namespace resident
 int cuda_check(cudaError_t e, const char* what);
 void count_launch(int n = 1);
 

@@ -132,11 +132,11 @@ int run(pm_operator* op, int which, const double* b, double* x, const pm_solve_o
   int st = cuda_check(cudaMemsetAsync(a.out, 0xff, sizeof(resident::Out), s), "noalloc results");
   if (st) return st;
   if ((st = resident::launch_fp64(a, PM_PREC_JACOBI, n <= CLUSTER_ROWS, op->num_sms, s))) return st;
-  resident::Out h;
-  if ((st = cuda_check(cudaMemcpyAsync(&h, a.out, sizeof(h), cudaMemcpyDeviceToHost, s), "noalloc results"))) return st;
+  resident::Out got;
+  if ((st = cuda_check(cudaMemcpyAsync(&got, a.out, sizeof(got), cudaMemcpyDeviceToHost, s), "noalloc results"))) return st;
   if ((st = cuda_check(cudaStreamSynchronize(s), "noalloc pcg"))) return st;
-  if (h.status == PM_TIMEOUT) return set_error(PM_TIMEOUT, "resident PCG: a grid barrier wait ran out");
-  if (h.status < 0) return set_error(PM_ECUDA, "resident PCG: the kernel reported nothing");
+  if ((st = resident::outcome(got))) return st;
+  const resident::Result& h = got.res;
   stats->iters = h.iters;
   stats->outer_iters = h.restarts;
   stats->first_pass_iters = h.first_pass;

@@ -53,9 +53,15 @@ struct Ctl {
   int32_t err;       // set by a wait that ran out
 };
 
-struct Out {
+struct Result {
   int32_t iters, restarts, first_pass, status, zero_rhs, pad;
   double rel_true, rel_rec, floor;
+};
+// Rank 0 writes the result. A block whose wait ran out writes the other field: rank 0 may have passed the last
+// barrier all the same and report its result after that, but the block that left did not do its rows.
+struct Out {
+  Result res;
+  int32_t timeout, pad;
 };
 
 struct Args {
@@ -746,7 +752,7 @@ __device__ __forceinline__ bool zero_mean(const Args& a, Team<CL>& team, int c0,
 
 // The FP64 solve: PCG on the recursive residual, then the true residual, restarts while they help.
 template <int PREC, bool CL>
-__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, int c1, double* zt, int ld, Out& o) {
+__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, int c1, double* zt, int ld, Result& o) {
   const double* b;
   double bb, rr;
   if (!start_solve<double>(a, team, c0, c1, b, bb, rr)) return false;
@@ -812,7 +818,7 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, i
 // recursive residual has dropped by inner_rtol, or claims convergence, the FP32 correction is folded into the
 // FP64 iterate, the true residual b - A x is formed (compensated) and a new inner solve starts from it.
 template <typename TV, int PREC, bool CL>
-__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c0, int c1, float* zt, int ld, Out& o) {
+__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c0, int c1, float* zt, int ld, Result& o) {
   const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
   const double* b;
   double bb, rr;
@@ -886,6 +892,19 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c
   return true;
 }
 
+__device__ __forceinline__ void report(Out* out, int rank, bool fine, const Result& o) {
+  if (threadIdx.x != 0) return;
+  if (!fine) *(volatile int32_t*)&out->timeout = 1;
+  else if (rank == 0) out->res = o;
+}
+
+// Host: whether the results of a finished launch are a solve's.
+inline int outcome(const Out& h) {
+  if (h.timeout > 0) return set_error(PM_TIMEOUT, "resident PCG: a grid barrier wait ran out");
+  if (h.res.status < 0) return set_error(PM_ECUDA, "resident PCG: the kernel reported nothing");
+  return PM_OK;
+}
+
 template <typename T, typename TV, int PREC, bool CL>
 __global__ void __launch_bounds__(NT, 1) k_resident(Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -909,15 +928,12 @@ __global__ void __launch_bounds__(NT, 1) k_resident(Args a) {
     zt = static_cast<T*>(a.z) + (int64_t)c0 * a.g.nz;
     ld = a.g.nz;
   }
-  Out o;
+  Result o;
   bool fine;
   if constexpr (std::is_same<T, double>::value) fine = solve64<PREC>(a, team, c0, c1, zt, ld, o);
   else fine = solve_mixed<TV, PREC>(a, team, c0, c1, zt, ld, o);
-  if (!fine) {
-    if (threadIdx.x == 0) *(volatile int32_t*)&a.out->status = PM_TIMEOUT;
-    return;
-  }
-  if (team.rank == 0 && threadIdx.x == 0) *a.out = o;
+  report(a.out, team.rank, fine, o);
+  if (!fine) return;
   if (CL) team.barrier();   // no block of a cluster leaves while another may still write to its shared memory
 }
 

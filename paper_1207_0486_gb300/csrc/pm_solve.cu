@@ -2140,7 +2140,8 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
   resident::Args a = resident_args(op, which, b, x, o);
   const int vs = which_valset(which);
   const bool cluster = op->n <= (prec == PM_PREC_IC0 ? RESIDENT_CLUSTER_IC0 : RESIDENT_CLUSTER_ROWS);
-  a.out->status = -1;
+  a.out->res.status = -1;
+  a.out->timeout = 0;
   if (mixed) {
     a.val = o->precision == PM_FP32_REFINE ? (const void*)op->d_val32[vs] : (const void*)op->d_val16[vs];
     a.r = c->r32;
@@ -2167,9 +2168,8 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
   }
   if (st) return st;
   if ((st = cuda_check(cudaStreamSynchronize(s), "resident pcg"))) return st;
-  const resident::Out h = *a.out;
-  if (h.status == PM_TIMEOUT) return set_error(PM_TIMEOUT, "resident PCG: a grid barrier wait ran out");
-  if (h.status < 0) return set_error(PM_ECUDA, "resident PCG: the kernel reported nothing");
+  if ((st = resident::outcome(*a.out))) return st;
+  const resident::Result h = a.out->res;
   if (stats) {
     stats->iters = h.iters;
     stats->outer_iters = h.restarts;
