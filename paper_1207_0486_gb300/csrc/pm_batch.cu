@@ -488,11 +488,8 @@ __device__ __forceinline__ bool owns_ic0_chunk(const Sys& S, int c) {
   }
 
 // MINB: resident blocks of 256 threads per SM that the register budget is sized for. 3 (80 registers, about
-// 1 KB of spills per thread) keeps 24 warps per SM in flight, 2 (128 registers) spills almost nothing. With many
-// tiles for each block 3 measured faster (64-basin batches: IC0 mass systems 0.41 -> 0.36 s, FP32 line
-// 8.84 -> 8.49 s); with few, when a phase is one tile's chain of loads and arithmetic, 2 is: 24 FP32 systems of 4.5M rows
-// (1200 tiles) 300 us per iteration either way, and 160 -> 110 us once only six systems iterate.
-constexpr int64_t FEW_TILES = 2400;   // up to about eight per block of the two-block kernel
+// 1 KB of spills per thread) keeps 24 warps per SM in flight, 2 (128 registers) spills almost nothing: a tile takes
+// 0.7 to 0.8 of the time, with two thirds of the blocks. few_tiles chooses one for every launch.
 template <typename T, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys, Scal* scal, int nsys,
                                                int ntiles, double* part, Ctl* ctl,
@@ -938,7 +935,8 @@ struct pm_batch {
   std::vector<int32_t> which;
   std::vector<int32_t> precs;      // preconditioner of each entry
   bool any_ic0 = false;            // the kernel runs the IC0 colour phases
-  int tile_cols = 32, block = 256, grid = 0;
+  int tile_cols = 32, block = 256;
+  int grid[2] = {0, 0};            // blocks of the kernel with three, with two blocks per SM
   int nz_max = 0;
   int64_t ntiles = 0;
   std::vector<pm::batch::Sys> hsys;
@@ -948,8 +946,8 @@ struct pm_batch {
   double* d_part = nullptr;
   void* work = nullptr;            // r, p, w, z (T) and bw (FP64) for all systems
   size_t work_bytes = 0;
-  cudaGraphExec_t graph = nullptr;
-  int graph_quantum = 0;
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  int graph_quantum[2] = {0, 0};
   int device = 0;
   double tuned_ms = 0.0;
 };
@@ -1050,8 +1048,10 @@ int entry_prec(int given, int dflt) {
 }
 
 void free_layout(pm_batch* bt) {
-  if (bt->graph) cudaGraphExecDestroy(bt->graph);
-  bt->graph = nullptr;
+  for (auto& g : bt->graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
   cudaFree(bt->d_sys);
   cudaFree(bt->d_scal);
   cudaFree(bt->d_ctl);
@@ -1121,10 +1121,48 @@ cudaError_t launch_k(Kernel k, int grid, int block, size_t smem, const Sys* d_sy
   return cudaLaunchKernelEx(&cfg, k, d_sys, d_scal, nsys, ntiles, d_part, d_ctl, quantum, init, ic0);
 }
 
-Kernel kernel_of(const pm_batch* bt) { return kernel_of(bt->precision, bt->ntiles <= FEW_TILES && !bt->any_ic0); }
+// Whether the two-block kernel takes a launch over the systems that scal says still iterate (null: all of them).
+// It does when its busiest block has no more tiles than the three-block kernel's has, or one more than two or
+// more while there are at most two (FP64) or five (FP32, BF16) for each of its blocks. Measured, us per
+// iteration, three-block / two-block, busiest block's tiles in brackets:
+//   FP64 line, all 468 tiles (2/2) 275 / 235, 580 (2/2) 280 / 253, 752 (2/3) 287 / 302, 1200 (3/4) 412 / 438; the
+//   pressure systems of a larger batch alone, 145 tiles (1/2) 145 / 161, 300 (2/2) 234 / 196, 593 (3/4) 411 / 339,
+//   842 (3/5) 419 / 447; Jacobi 465 (2/2) 253 / 189, 780 (2/3) 293 / 328;
+//   FP32 line, all 468 (2/2) 198 / 160, 836 (2/3) 229 / 217, 1200 (3/4) 287 / 293, 1257 (3/5) 339 / 366, 1407 (4/5)
+//   407 / 393, 1876 (5/7) 510 / 537; pressure alone 145 (1/2) 89 / 91, 300 (2/2) 189 / 133, 593 (3/4) 326 / 239,
+//   842 (3/5) 331 / 302; BF16 1407 (4/5) 388 / 375; Jacobi FP32 1395 (4/5) 388 / 351, BF16 377 / 333.
+// IC0 phases keep three: FP64 754 / 979 at 465 tiles, 1307 / 1567 at 930, 438 / 415 at 90.
+bool few_tiles(const pm_batch* bt, const Scal* scal) {
+  if (bt->any_ic0) return false;
+  int64_t tiles = 0;
+  int busiest[2];
+  for (int few = 0; few < 2; ++few) {
+    std::vector<int> d((size_t)bt->grid[few] + 1, 0);   // differences of the blocks' tile counts
+    int whole = 0;
+    tiles = 0;
+    for (int i = 0; i < bt->count; ++i) {
+      if (scal && scal[i].state == ST_DONE) continue;
+      const int g = bt->grid[few], nt = bt->hsys[i].ntiles, a = bt->hsys[i].tile0 % g, e = a + nt % g;
+      tiles += nt;
+      whole += nt / g;
+      ++d[a];
+      --d[std::min(e, g)];
+      if (e > g) {
+        ++d[0];
+        --d[e - g];
+      }
+    }
+    int most = 0, at = 0;
+    for (int b = 0; b < bt->grid[few]; ++b) most = std::max(most, at += d[b]);
+    busiest[few] = whole + most;
+  }
+  return busiest[1] <= busiest[0] ||
+         (busiest[0] > 1 && busiest[1] == busiest[0] + 1 &&
+          tiles <= (int64_t)(bt->precision == PM_FP64 ? 2 : 5) * bt->grid[1]);
+}
 
-cudaError_t launch(pm_batch* bt, int quantum, int init, cudaStream_t s) {
-  return launch_k(kernel_of(bt), bt->grid, bt->block, smem_bytes(bt), bt->d_sys, bt->d_scal, (int)bt->count,
+cudaError_t launch(pm_batch* bt, bool few, int quantum, int init, cudaStream_t s) {
+  return launch_k(kernel_of(bt->precision, few), bt->grid[few], bt->block, smem_bytes(bt), bt->d_sys, bt->d_scal, (int)bt->count,
                      (int)bt->ntiles, bt->d_part, bt->d_ctl, quantum, init, bt->any_ic0 ? 1 : 0, s);
 }
 
@@ -1153,11 +1191,13 @@ int capture_graph(cudaGraphExec_t* exec, F fn) {
 
 int set_grid(pm_batch* bt) {
   const size_t smem = smem_bytes(bt);
-  const int per_sm = max_blocks(kernel_of(bt), bt->block, smem);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device);
-  if (per_sm <= 0) return set_error(PM_EINVAL, "batched kernel cannot be resident with this block / tile shape");
-  bt->grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * sms, std::max<int64_t>(bt->ntiles, bt->count)));
+  for (int few = 0; few < 2; ++few) {
+    const int per_sm = max_blocks(kernel_of(bt->precision, few), bt->block, smem);
+    if (per_sm <= 0) return set_error(PM_EINVAL, "batched kernel cannot be resident with this block / tile shape");
+    bt->grid[few] = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * sms, std::max<int64_t>(bt->ntiles, bt->count)));
+  }
   return PM_OK;
 }
 
@@ -1176,26 +1216,31 @@ int start(pm_batch* bt, cudaStream_t s) {
   if (!st) st = cuda_check(cudaMemcpyAsync(bt->d_scal, hs.data(), bt->count * sizeof(Scal), cudaMemcpyHostToDevice, s), "scal");
   if (!st) st = cuda_check(cudaMemcpyAsync(bt->d_ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s), "ctl");
   if (st) return st;
-  const cudaError_t e = launch(bt, 0, 1, s);
+  const cudaError_t e = launch(bt, few_tiles(bt, nullptr), 0, 1, s);
   return cuda_check(e, "batched PCG init launch");
 }
 
 int run_to_completion(pm_batch* bt, cudaStream_t s, int quantum) {
-  // capture one quantum launch in a CUDA graph once, replay it until no system is active
-  if (!bt->graph || bt->graph_quantum != quantum) {
-    const int st = capture_graph(&bt->graph, [&](cudaStream_t cs) {
-      return launch(bt, quantum, 0, cs);
-    });
-    if (st) return st;
-    bt->graph_quantum = quantum;
-  }
+  // one quantum launch of either kernel captured in a CUDA graph once, replayed until no system is active
   Ctl h;
+  std::vector<Scal> hs(bt->count);
+  bool few = few_tiles(bt, nullptr);
   const int64_t max_quanta = (int64_t)bt->max_iter / quantum + 70;
   for (int64_t q = 0; q < max_quanta; ++q) {
-    int st = cuda_check(cudaGraphLaunch(bt->graph, s), "batched PCG graph launch");
+    if (q > 0) few = few_tiles(bt, hs.data());
+    if (!bt->graph[few] || bt->graph_quantum[few] != quantum) {
+      const int st = capture_graph(&bt->graph[few], [&](cudaStream_t cs) {
+        return launch(bt, few, quantum, 0, cs);
+      });
+      if (st) return st;
+      bt->graph_quantum[few] = quantum;
+    }
+    int st = cuda_check(cudaGraphLaunch(bt->graph[few], s), "batched PCG graph launch");
     if (st) return st;
     count_launch();
     st = cuda_check(cudaMemcpyAsync(&h, bt->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s), "ctl");
+    if (!st && !bt->any_ic0)
+      st = cuda_check(cudaMemcpyAsync(hs.data(), bt->d_scal, bt->count * sizeof(Scal), cudaMemcpyDeviceToHost, s), "scal");
     if (!st) st = cuda_check(cudaStreamSynchronize(s), "batched PCG");
     if (st) return st;
     if (h.err) return set_error(h.err, "batched PCG: a grid barrier wait expired");
@@ -1282,7 +1327,7 @@ int autotune(pm_batch* bt, cudaStream_t s) {
       }
       if (start(bt, s)) continue;
       cudaEventRecord(e0, s);
-      const cudaError_t le = launch(bt, 8, 0, s);
+      const cudaError_t le = launch(bt, few_tiles(bt, nullptr), 8, 0, s);
       cudaEventRecord(e1, s);
       if (le != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) continue;
       Ctl h;
@@ -1391,7 +1436,7 @@ extern "C" int pm_batch_info(const pm_batch* bt, int32_t* tile_cols, int32_t* bl
   if (!bt) return set_error(PM_EINVAL, "null batch");
   if (tile_cols) *tile_cols = bt->tile_cols;
   if (block) *block = bt->block;
-  if (grid) *grid = bt->grid;
+  if (grid) *grid = bt->grid[batch::few_tiles(bt, nullptr)];
   if (ntiles) *ntiles = bt->ntiles;
   return PM_OK;
 }
