@@ -14,8 +14,9 @@
 //     with global stores to publish), block sums exchanged through distributed shared memory: for systems so
 //     small that the grid barrier would cost more than the work the other SMs take over.
 //
-// Rows: SpMV, update and preconditioners by column work on whole columns, dealt evenly and
-// contiguously to the blocks; an IC0 colour phase deals the colour's rows (in class order, as the
+// Rows: the line preconditioner works on whole columns, dealt evenly and contiguously to the blocks; without it
+// a block takes an even share of the rows, however few columns they make up (16 columns of 20,000 levels, Jacobi:
+// 32 us per iteration, 172 by whole columns, 71 as a stream); an IC0 colour phase deals the colour's rows (in class order, as the
 // factor is stored) evenly to the blocks. Vectors that other blocks read (p, x, the IC0 work vector)
 // go through L2: a barrier's release / acquire pair orders them, and the acquire drops stale L1 lines,
 // so plain loads may use L1 within a phase.
@@ -217,6 +218,27 @@ struct Team {
     return true;
   }
 };
+
+// A block's rows [r0, r1); with the line preconditioner they are its whole columns [c0, c1).
+struct Share {
+  int r0, r1, c0, c1;
+};
+template <int PREC>
+__device__ __forceinline__ Share share_of(const Geom& g, int rank, int G) {
+  Share s;
+  if (PREC == PM_PREC_LINE) {
+    s.c0 = (int)((int64_t)g.ncols * rank / G);
+    s.c1 = (int)((int64_t)g.ncols * (rank + 1) / G);
+    s.r0 = s.c0 * g.nz;
+    s.r1 = s.c1 * g.nz;
+  } else {   // in runs of 32 rows, so that a warp's accesses are aligned
+    const int64_t runs = (g.n + 31) / 32;
+    s.c0 = s.c1 = 0;
+    s.r0 = (int)min(g.n, 32 * (runs * rank / G));
+    s.r1 = (int)min(g.n, 32 * (runs * (rank + 1) / G));
+  }
+  return s;
+}
 
 // Neighbour q, by its index within its class, of the column at place i in class order (-1: none).
 __device__ __forceinline__ int ccls_of(const Args& a, int i, int q) {
@@ -467,17 +489,17 @@ __device__ __forceinline__ bool ic0_backward(const Args& a, Team<CL>& team, T al
 
 // ---- the update and the column-local preconditioners ------------------------------------------
 
-// r -= alpha w (UPDATE), then z by the preconditioner, on this block's columns [c0, c1). LINE: zt is the
+// r -= alpha w (UPDATE), then z by the preconditioner, on this block's rows. LINE: zt is the
 // block's tile of columns, ld apart (shared memory, or its part of the z vector).
 template <typename T, int PREC, bool UPDATE>
-__device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alpha, T* zt, int ld, Dots<T>& dots) {
+__device__ __forceinline__ void update_rows(const Args& a, const Share& sh, T alpha, T* zt, int ld, Dots<T>& dots) {
   const Geom& g = a.g;
-  const int nz = g.nz, row0 = c0 * nz, row1 = c1 * nz;
+  const int nz = g.nz, row1 = sh.r1;
   T* r = static_cast<T*>(a.r);
   const T* w = static_cast<const T*>(a.w);
   const T* dinv = static_cast<const T*>(a.dinv);
   constexpr int U = 4;   // rows whose loads are in flight together
-  for (int i0 = row0 + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
+  for (int i0 = sh.r0 + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
     T rv[U], wv[U], dv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -503,7 +525,7 @@ __device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alp
         if (a.proj) add_m(dots.mz, a, row, zi);
       } else {
         const int col = fdiv(g.nzd, row), k = row - col * nz;
-        if (PREC == PM_PREC_LINE) zt[(col - c0) * ld + k] = ri;
+        if (PREC == PM_PREC_LINE) zt[(col - sh.c0) * ld + k] = ri;
         else colour0_y(a, col, k, ri, dots.rz);
       }
     }
@@ -513,8 +535,8 @@ __device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alp
   // Thomas solve of each column, one thread per column; (r, z) = sum_k t_k y_k (symmetric blocks)
   const T* F = static_cast<const T*>(a.line);
   const int nc = g.ncols, n = (int)g.n;
-  for (int col = c0 + (int)threadIdx.x; col < c1; col += NT) {
-    T* cs = zt + (col - c0) * ld;
+  for (int col = sh.c0 + (int)threadIdx.x; col < sh.c1; col += NT) {
+    T* cs = zt + (col - sh.c0) * ld;
     T y = 0;
 #pragma unroll 8
     for (int k = 0; k < nz; ++k) {
@@ -533,9 +555,9 @@ __device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alp
   }
   __syncthreads();
   if (!a.proj) return;
-  for (int row = row0 + (int)threadIdx.x; row < row1; row += NT) {
+  for (int row = sh.r0 + (int)threadIdx.x; row < row1; row += NT) {
     const int col = fdiv(g.nzd, row);
-    add_m(dots.mz, a, row, zt[(col - c0) * ld + row - col * nz]);
+    add_m(dots.mz, a, row, zt[(col - sh.c0) * ld + row - col * nz]);
   }
 }
 
@@ -543,16 +565,16 @@ __device__ __forceinline__ void update_rows(const Args& a, int c0, int c1, T alp
 // here anyway. FIRST: p = z - c.
 // LAST: x alone, when no further direction is needed.
 template <typename T, int PREC, bool FIRST, bool LAST>
-__device__ __forceinline__ void direction(const Args& a, int c0, int c1, T alpha, T beta, T c, const T* zt, int ld) {
+__device__ __forceinline__ void direction(const Args& a, const Share& sh, T alpha, T beta, T c, const T* zt, int ld) {
   const Geom& g = a.g;
-  const int nz = g.nz, row1 = c1 * nz;
+  const int nz = g.nz, row1 = sh.r1;
   T* p = static_cast<T*>(a.p);
   T* x = iterate<T>(a);
   const T* r = static_cast<const T*>(a.r);
   const T* zv = static_cast<const T*>(a.z);
   const T* dinv = static_cast<const T*>(a.dinv);
   constexpr int U = 4;
-  for (int i0 = c0 * nz + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
+  for (int i0 = sh.r0 + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
     T z[U], pv[U], xv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -562,7 +584,7 @@ __device__ __forceinline__ void direction(const Args& a, int c0, int c1, T alpha
           z[u] = (dinv ? __ldg(dinv + row) : (T)1) * r[row];
         } else if (PREC == PM_PREC_LINE) {
           const int col = fdiv(g.nzd, row);
-          z[u] = zt[(col - c0) * ld + row - col * nz];
+          z[u] = zt[(col - sh.c0) * ld + row - col * nz];
         } else {
           const int col = fdiv(g.nzd, row);
           z[u] = zv[colour_pos(a, col, row - col * nz)];
@@ -594,10 +616,10 @@ struct Cg {
 // known: true ends the step with x moved (the recursion has met its target). cg.status is PM_BREAKDOWN
 // when rho is not positive. Returns false when a wait ran out.
 template <typename T, int PREC, bool FIRST, bool CL, typename Stop>
-__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, int c0, int c1, T* zt, int ld, double alpha, Cg& cg,
+__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Share& sh, T* zt, int ld, double alpha, Cg& cg,
                                         bool& stopped, Stop stop) {
   Dots<T> dots;
-  update_rows<T, PREC, !FIRST>(a, c0, c1, (T)alpha, zt, ld, dots);
+  update_rows<T, PREC, !FIRST>(a, sh, (T)alpha, zt, ld, dots);
   double c = 0.0, rho = 0.0;
   if (PREC == PM_PREC_IC0) {
     double v[1] = {dots.rr.value()};
@@ -610,7 +632,7 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, int c0, i
       const T* r = static_cast<const T*>(a.r);
       const T* z = static_cast<const T*>(a.z);
       AccFor<T> rz;
-      for (int row = c0 * a.g.nz + (int)threadIdx.x; row < c1 * a.g.nz; row += NT) {
+      for (int row = sh.r0 + (int)threadIdx.x; row < sh.r1; row += NT) {
         const int col = fdiv(a.g.nzd, row);
         const T zi = z[colour_pos(a, col, row - col * a.g.nz)];
         rz.add_prod(r[row], zi);
@@ -638,7 +660,7 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, int c0, i
   const bool broken = !stopped && (!(rho > 0.0) || !isfinite(rho));
   if (broken) cg.status = PM_BREAKDOWN;
   if (stopped || broken) {
-    direction<T, PREC, FIRST, true>(a, c0, c1, (T)alpha, (T)0, (T)0, zt, ld);
+    direction<T, PREC, FIRST, true>(a, sh, (T)alpha, (T)0, (T)0, zt, ld);
     return team.barrier();
   }
   const T beta = FIRST ? (T)0 : (T)(rho / cg.rho);
@@ -648,19 +670,19 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, int c0, i
     // p may hold anything yet (not a number included): set afterwards, not scaled by 0
     if (!ic0_backward<T, false>(a, team, (T)0, (T)0)) return false;
   }
-  direction<T, PREC, FIRST, false>(a, c0, c1, (T)alpha, beta, (T)c, zt, ld);
+  direction<T, PREC, FIRST, false>(a, sh, (T)alpha, beta, (T)c, zt, ld);
   return team.barrier();
 }
 
 // w = A p on the block's rows; v = (p, w) over the team.
 template <typename T, typename TV, bool CL>
-__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, int c0, int c1, double& pw) {
+__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const Share& sh, double& pw) {
   const Geom& g = a.g;
   const TV* val = static_cast<const TV*>(a.val);
   const T* p = static_cast<const T*>(a.p);
   T* w = static_cast<T*>(a.w);
   AccFor<T> acc;
-  for (int row = c0 * g.nz + (int)threadIdx.x; row < c1 * g.nz; row += NT) {
+  for (int row = sh.r0 + (int)threadIdx.x; row < sh.r1; row += NT) {
     const int col = fdiv(g.nzd, row);
     const T wi = row_apply<T, TV>(g, val, p, a.mask, row, col, row - col * g.nz);
     w[row] = wi;
@@ -674,12 +696,12 @@ __device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, int c0,
 
 // r = b - A x (compensated), (r, r) and the floor's (|A||x| + |b|)^2 over the team.
 template <typename T, bool CL>
-__device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, int c0, int c1, const double* b, double& rr,
+__device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, const Share& sh, const double* b, double& rr,
                                               double& ff) {
   const Geom& g = a.g;
   T* r = static_cast<T*>(a.r);
   double v[2] = {0.0, 0.0};
-  for (int row = c0 * g.nz + (int)threadIdx.x; row < c1 * g.nz; row += NT) {
+  for (int row = sh.r0 + (int)threadIdx.x; row < sh.r1; row += NT) {
     const int col = fdiv(g.nzd, row);
     double asum;
     const double bi = b[row];
@@ -697,14 +719,13 @@ __device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, int
 
 // Right-hand side, initial guess and first residual: (b', b') and (r, r). From x = 0 the residual is b' itself.
 template <typename T, bool CL>
-__device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, int c0, int c1, const double*& b, double& bb,
+__device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, const Share& sh, const double*& b, double& bb,
                                             double& rr) {
-  const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
   double lam = 0.0, xs = 0.0;
   b = a.b;
   if (a.proj) {
     double v[2] = {0.0, 0.0};
-    for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) {
+    for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) {
       v[0] += b[i];
       if (a.x0_is_guess) v[1] = fma(a.m[i], a.x[i], v[1]);
     }
@@ -714,7 +735,7 @@ __device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, int c
   }
   T* r = static_cast<T*>(a.r);
   double v[2] = {0.0, 0.0};
-  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) {
+  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) {
     double bi = b[i];
     if (a.proj) {
       bi = bi - lam * a.m[i];
@@ -734,28 +755,27 @@ __device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, int c
   bb = v[0];
   rr = bb;
   double ff;
-  if (a.x0_is_guess && !true_residual<T>(a, team, c0, c1, b, rr, ff)) return false;
+  if (a.x0_is_guess && !true_residual<T>(a, team, sh, b, rr, ff)) return false;
   return true;
 }
 
 // The returned pressure has m'x = 0.
 template <bool CL>
-__device__ __forceinline__ bool zero_mean(const Args& a, Team<CL>& team, int c0, int c1) {
-  const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
+__device__ __forceinline__ bool zero_mean(const Args& a, Team<CL>& team, const Share& sh) {
   double v[1] = {0.0};
-  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) v[0] = fma(a.m[i], a.x[i], v[0]);
+  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) v[0] = fma(a.m[i], a.x[i], v[0]);
   if (!team.template sum<1>(v)) return false;
-  const double sh = v[0] / a.one_m;
-  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.x[i] -= sh;
+  const double shift = v[0] / a.one_m;
+  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.x[i] -= shift;
   return true;
 }
 
 // The FP64 solve: PCG on the recursive residual, then the true residual, restarts while they help.
 template <int PREC, bool CL>
-__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, int c1, double* zt, int ld, Result& o) {
+__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, const Share& sh, double* zt, int ld, Result& o) {
   const double* b;
   double bb, rr;
-  if (!start_solve<double>(a, team, c0, c1, b, bb, rr)) return false;
+  if (!start_solve<double>(a, team, sh, b, bb, rr)) return false;
   const double tol2 = a.rtol * a.rtol * bb;
   Cg cg;
   int restarts = 0, first_pass = -1;
@@ -765,19 +785,19 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, i
   if (!skip && a.max_iter == 0 && bb != 0.0) cg.status = PM_NOT_CONVERGED;
   cg.rr = rr;
   if (bb == 0.0)
-    for (int i = c0 * a.g.nz + (int)threadIdx.x; i < c1 * a.g.nz; i += NT) a.x[i] = 0.0;
+    for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.x[i] = 0.0;
   while (bb != 0.0) {
     if (cg.status == PM_OK && !skip) {
       bool converged = false, stopped;
-      if (!advance<double, PREC, true>(a, team, c0, c1, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
+      if (!advance<double, PREC, true>(a, team, sh, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
       while (cg.status == PM_OK && cg.iter < a.max_iter) {
         double pw;
-        if (!apply_dot<double, double>(a, team, c0, c1, pw)) return false;
+        if (!apply_dot<double, double>(a, team, sh, pw)) return false;
         if (!(pw > 0.0) || !isfinite(pw)) {
           cg.status = PM_BREAKDOWN;
           break;
         }
-        const bool fine = advance<double, PREC, false>(a, team, c0, c1, zt, ld, cg.rho / pw, cg, stopped, [&] {
+        const bool fine = advance<double, PREC, false>(a, team, sh, zt, ld, cg.rho / pw, cg, stopped, [&] {
           ++cg.iter;
           converged = cg.rr <= tol2;
           return converged || cg.iter >= a.max_iter;
@@ -790,7 +810,7 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, i
     skip = false;
     if (first_pass < 0) first_pass = cg.iter;
     double tr, ff;
-    if (!true_residual<double>(a, team, c0, c1, b, tr, ff)) return false;
+    if (!true_residual<double>(a, team, sh, b, tr, ff)) return false;
     rel_true = sqrt(tr / bb);
     floor = ldexp(1.0, -53) * sqrt(ff / bb);
     const bool stalled = prev_true >= 0.0 && rel_true > 0.5 * prev_true;
@@ -802,7 +822,7 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, i
     ++restarts;
   }
   if (bb != 0.0 && cg.status == PM_OK && !accepted) cg.status = PM_NOT_CONVERGED;
-  if (a.proj && !zero_mean(a, team, c0, c1)) return false;
+  if (a.proj && !zero_mean(a, team, sh)) return false;
   o.iters = cg.iter;
   o.restarts = restarts;
   o.first_pass = first_pass < 0 ? cg.iter : first_pass;
@@ -818,18 +838,17 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, int c0, i
 // recursive residual has dropped by inner_rtol, or claims convergence, the FP32 correction is folded into the
 // FP64 iterate, the true residual b - A x is formed (compensated) and a new inner solve starts from it.
 template <typename TV, int PREC, bool CL>
-__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c0, int c1, float* zt, int ld, Result& o) {
-  const int row0 = c0 * a.g.nz, row1 = c1 * a.g.nz;
+__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, const Share& sh, float* zt, int ld, Result& o) {
   const double* b;
   double bb, rr;
-  for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.d[i] = 0.f;
-  if (!start_solve<float>(a, team, c0, c1, b, bb, rr)) return false;
+  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.d[i] = 0.f;
+  if (!start_solve<float>(a, team, sh, b, bb, rr)) return false;
   const double tol2 = a.rtol * a.rtol * bb, drop = a.inner_rtol * a.inner_rtol;
   Cg cg;
   int outer = 0, stalled = 0;
   double rel_true = 0.0, floor = 0.0, prev_true = 1e300;
   if (bb == 0.0) {
-    for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) a.x[i] = 0.0;
+    for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.x[i] = 0.0;
   } else if (rr <= tol2 || a.max_iter == 0) {   // x0 already meets rtol, or no iteration is allowed
     if (!(rr <= tol2)) cg.status = PM_NOT_CONVERGED;   // not a number included
     rel_true = sqrt(rr / bb);
@@ -837,28 +856,28 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c
     for (;;) {
       const double target = fmax(tol2, drop * rr);
       bool stopped;
-      if (!advance<float, PREC, true>(a, team, c0, c1, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
+      if (!advance<float, PREC, true>(a, team, sh, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
       while (cg.status == PM_OK) {
         double pw;
-        if (!apply_dot<float, TV>(a, team, c0, c1, pw)) return false;
+        if (!apply_dot<float, TV>(a, team, sh, pw)) return false;
         if (!(pw > 0.0) || !isfinite(pw)) {
           cg.status = PM_BREAKDOWN;
           break;
         }
-        const bool fine = advance<float, PREC, false>(a, team, c0, c1, zt, ld, cg.rho / pw, cg, stopped, [&] {
+        const bool fine = advance<float, PREC, false>(a, team, sh, zt, ld, cg.rho / pw, cg, stopped, [&] {
           ++cg.iter;
           return cg.rr <= target || cg.iter >= a.max_iter;
         });
         if (!fine) return false;
         if (stopped) break;
       }
-      for (int i = row0 + (int)threadIdx.x; i < row1; i += NT) {
+      for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) {
         a.x[i] += (double)a.d[i];
         a.d[i] = 0.f;
       }
       if (!team.barrier()) return false;
       double ff;
-      if (!true_residual<float>(a, team, c0, c1, b, rr, ff)) return false;
+      if (!true_residual<float>(a, team, sh, b, rr, ff)) return false;
       ++outer;
       rel_true = sqrt(rr / bb);
       floor = ldexp(1.0, -53) * sqrt(ff / bb);
@@ -882,7 +901,7 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, int c
       }
     }
   }
-  if (a.proj && !zero_mean(a, team, c0, c1)) return false;
+  if (a.proj && !zero_mean(a, team, sh)) return false;
   o.iters = o.first_pass = cg.iter;
   o.restarts = outer;
   o.status = cg.status;
@@ -918,20 +937,19 @@ __global__ void __launch_bounds__(NT, 1) k_resident(Args a) {
   __syncthreads();
   Team<CL> team(a, &scratch);
   if (CL) team.barrier();   // every block of the cluster runs before one writes to another's shared memory
-  // whole columns, dealt evenly
-  const int c0 = (int)((int64_t)a.g.ncols * team.rank / team.G), c1 = (int)((int64_t)a.g.ncols * (team.rank + 1) / team.G);
+  const Share sh = share_of<PREC>(a.g, team.rank, team.G);
   T* zt;
   int ld = a.g.nz | 1;   // odd: a warp's columns fall into different banks
   if (a.z_in_smem) {
     zt = reinterpret_cast<T*>(smem_raw);
   } else {
-    zt = static_cast<T*>(a.z) + (int64_t)c0 * a.g.nz;
+    zt = static_cast<T*>(a.z) + (PREC == PM_PREC_LINE ? sh.r0 : 0);
     ld = a.g.nz;
   }
   Result o;
   bool fine;
-  if constexpr (std::is_same<T, double>::value) fine = solve64<PREC>(a, team, c0, c1, zt, ld, o);
-  else fine = solve_mixed<TV, PREC>(a, team, c0, c1, zt, ld, o);
+  if constexpr (std::is_same<T, double>::value) fine = solve64<PREC>(a, team, sh, zt, ld, o);
+  else fine = solve_mixed<TV, PREC>(a, team, sh, zt, ld, o);
   report(a.out, team.rank, fine, o);
   if (!fine) return;
   if (CL) team.barrier();   // no block of a cluster leaves while another may still write to its shared memory
