@@ -33,7 +33,9 @@ namespace pm {
 
 struct SolveCtx {
   int64_t n = 0;
-  int line_slots = 0, line_slots_nz = -1;  // resident blocks of the fused line kernel (per nz)
+  // Resident blocks of the fused line kernels on the operator's device (0: not looked up yet): any nz; 32 levels with
+  // tasks of 16 and of 32 columns; FP32 without and with the projection.
+  int line_slots = 0, line_w_slots[2] = {0, 0}, line32_slots[2] = {0, 0};
   double *r = nullptr, *p = nullptr, *w = nullptr, *z = nullptr, *bw = nullptr;
   double* partials = nullptr;
   PcgScalars* sc = nullptr;
@@ -952,15 +954,41 @@ __global__ void __launch_bounds__(LINE_WTPB, TCOLS == 32 ? 3 : 4) k_update_line_
 // Columns per task: 32, so that every lane of a warp sweeps a column (an FP64 instruction costs the
 // FP64 pipe the same with idle lanes, and the sweep is a third of the kernel's FP64 work), unless
 // that leaves fewer tasks than resident warps (basins under about 600 x 600 columns of 32 levels):
-// then 16, twice the warps and half the lanes sweeping. line_w_slots gives the resident tasks of
+// then 16, twice the warps and half the lanes sweeping. line_w_setup gives the resident blocks of
 // one choice.
+//
+// Function attributes are per device, so they are set for every operator, not once in the process.
+constexpr int LINE_SMEM = 200 * 1024;
+int smem_limit(const void* kernel, size_t bytes) {
+  return cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), "line shared memory");
+}
+
 template <int TC>
-int line_w_slots(const void* kernel, int num_sms) {
+int line_w_setup(pm_operator* op, int* slots) {
   const size_t smem = (size_t)(LINE_WTPB / 32) * TC * (LINE_WNZ + 1) * sizeof(double);
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, LINE_WTPB, smem);
-  return std::max(1, per_sm) * num_sms;
+  int st, per_sm = 0;
+  if ((st = smem_limit((const void*)k_update_line_w<0, TC>, smem))) return st;
+  if ((st = smem_limit((const void*)k_update_line_w<1, TC>, smem))) return st;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update_line_w<1, TC>, LINE_WTPB, smem);
+  *slots = std::max(1, per_sm) * op->num_sms;
+  return PM_OK;
+}
+
+// What the FP64 line kernels need before their first launch for this operator.
+int line_setup(pm_operator* op) {
+  SolveCtx* c = op->ctx;
+  if (c->line_slots) return PM_OK;
+  int st, per_sm = 0;
+  if ((st = smem_limit((const void*)k_line_rho<0>, LINE_SMEM))) return st;
+  if ((st = smem_limit((const void*)k_line_rho<1>, LINE_SMEM))) return st;
+  if ((st = smem_limit((const void*)k_update_line<0, 0>, LINE_SMEM))) return st;
+  if ((st = smem_limit((const void*)k_update_line<1, 0>, LINE_SMEM))) return st;
+  if ((st = line_w_setup<16>(op, &c->line_w_slots[0]))) return st;
+  if ((st = line_w_setup<32>(op, &c->line_w_slots[1]))) return st;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update_line<1, 0>, LINE_FTPB,
+                                                (size_t)LINE_FCOLS * (op->nz + 1) * sizeof(double));
+  c->line_slots = std::max(1, per_sm) * op->num_sms;
+  return PM_OK;
 }
 
 template <int TC>
@@ -982,13 +1010,7 @@ void launch_line_w(pm_operator* op, int which, bool proj, double* x, int slots, 
 // Launch of k_update_line_w: exactly the resident blocks (capped by the partials buffer, 4 lanes
 // per block, and by one task per warp).
 void update_line_w(pm_operator* op, int which, bool proj, double* x, cudaStream_t s) {
-  static int slots32 = 0, slots16 = 0;
-  if (!slots32) {
-    slots32 = line_w_slots<32>((const void*)k_update_line_w<1, 32>, op->num_sms);
-    line_w_slots<32>((const void*)k_update_line_w<0, 32>, op->num_sms);
-    slots16 = line_w_slots<16>((const void*)k_update_line_w<1, 16>, op->num_sms);
-    line_w_slots<16>((const void*)k_update_line_w<0, 16>, op->num_sms);
-  }
+  const int slots16 = op->ctx->line_w_slots[0], slots32 = op->ctx->line_w_slots[1];
   const int64_t tasks32 = (op->ncols + 31) / 32;
   if (tasks32 >= (int64_t)slots32 * (LINE_WTPB / 32)) launch_line_w<32>(op, which, proj, x, slots32, s);
   else launch_line_w<16>(op, which, proj, x, slots16, s);
@@ -1003,19 +1025,7 @@ void update_line(pm_operator* op, int which, bool proj, double* x, cudaStream_t 
   SolveCtx* c = op->ctx;
   Geom g = geom_of(op);
   const size_t smem = (size_t)LINE_FCOLS * (op->nz + 1) * sizeof(double);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_update_line<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_update_line<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set = true;
-  }
-  // resident blocks of this shape: the full-width tiles fill exactly one wave of them
-  if (c->line_slots_nz != op->nz) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update_line<1, 0>, LINE_FTPB, smem);
-    c->line_slots = std::max(1, per_sm) * op->num_sms;
-    c->line_slots_nz = op->nz;
-  }
+  // The full-width tiles fill exactly one wave of the resident blocks;
   // four partial lanes per block must fit the partials buffer (NPART x MAX_GRID doubles)
   const int nfull_max = (int)std::min<int64_t>(c->line_slots, (int64_t)NPART * MAX_GRID / 4);
   const int64_t nt_full = (op->ncols + LINE_FCOLS - 1) / LINE_FCOLS;
@@ -1046,12 +1056,6 @@ void line_apply_rho(pm_operator* op, int which, bool proj, int is_first, cudaStr
   int grid = (int)std::min<int64_t>(ntiles, std::min<int64_t>((int64_t)op->num_sms * 8, MAX_GRID));
   if (grid < 1) grid = 1;
   const size_t smem = 2 * (size_t)LINE_COLS * (op->nz + 1) * sizeof(double);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_line_rho<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_line_rho<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set = true;
-  }
   if (proj)
     k_line_rho<1><<<grid, LINE_TPB, smem, s>>>(g, op->d_line[which], c->r, c->z, op->d_m, c->partials, c->sc, is_first);
   else
@@ -1371,7 +1375,7 @@ int pcg_run(pm_operator* op, int which, const double* b, double* x, const pm_sol
       if (bd) return set_error(PM_BREAKDOWN, "IC0 pivot failure after the shift limit");
     }
   }
-  if (prec == PM_PREC_LINE && (st = line_factor(op, which, s))) return st;
+  if (prec == PM_PREC_LINE && ((st = line_setup(op)) || (st = line_factor(op, which, s)))) return st;
   // Right-hand side and initial guess.
   const int G = grid_for(op->n, TPB, op->num_sms);
   PcgScalars init;
@@ -2010,19 +2014,30 @@ constexpr size_t LINE32_TILE = 200 * 1024;   // shared memory of a block's warp 
 size_t line32_tile(int nz) { return (size_t)(LINE_WTPB / 32) * LINE32_TC * (nz | 1) * sizeof(float); }
 
 template <int PROJ, int NZ>
+int line32_setup(pm_operator* op) {
+  int& slots = op->ctx->line32_slots[PROJ];
+  if (slots) return PM_OK;
+  const void* kern = (const void*)k32_update_line_w<PROJ, LINE32_TC, NZ>;
+  int st, per_sm = 0;
+  if ((st = smem_limit(kern, LINE32_TILE))) return st;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, LINE_WTPB, line32_tile(op->nz));
+  slots = std::max(1, per_sm) * op->num_sms;
+  return PM_OK;
+}
+// What the FP32 line kernel needs before its first launch for this operator.
+int line32_setup(pm_operator* op, bool proj) {
+  if (op->nz == LINE_WNZ) return proj ? line32_setup<1, LINE_WNZ>(op) : line32_setup<0, LINE_WNZ>(op);
+  return proj ? line32_setup<1, 0>(op) : line32_setup<0, 0>(op);
+}
+
+template <int PROJ, int NZ>
 void launch_line32_w(pm_operator* op, int which, int mode, cudaStream_t s) {
   SolveCtx* c = op->ctx;
-  const void* kern = (const void*)k32_update_line_w<PROJ, LINE32_TC, NZ>;
-  const size_t smem = line32_tile(op->nz);
-  static const bool attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LINE32_TILE) == cudaSuccess;
-  (void)attr;
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, LINE_WTPB, smem);
   // the resident blocks, capped by the partials buffer (4 lanes per block) and by one task per warp
   const int64_t ntask = (op->ncols + LINE32_TC - 1) / LINE32_TC;
-  int64_t blocks = std::min<int64_t>((int64_t)std::max(1, per_sm) * op->num_sms, (int64_t)NPART * MAX_GRID / 4);
+  int64_t blocks = std::min<int64_t>(c->line32_slots[PROJ], (int64_t)NPART * MAX_GRID / 4);
   blocks = std::min<int64_t>(blocks, (ntask + LINE_WTPB / 32 - 1) / (LINE_WTPB / 32));
-  k32_update_line_w<PROJ, LINE32_TC, NZ><<<(int)std::max<int64_t>(1, blocks), LINE_WTPB, smem, s>>>(
+  k32_update_line_w<PROJ, LINE32_TC, NZ><<<(int)std::max<int64_t>(1, blocks), LINE_WTPB, line32_tile(op->nz), s>>>(
       geom_of(op), op->d_line32[which], c->d32, c->r32, c->p32, c->w32, c->z32, op->d_m2f, c->partials, c->sc_in, mode);
 }
 
@@ -2270,6 +2285,7 @@ int mixed_run(pm_operator* op, int which, const double* b, double* x, const pm_s
   int st;
   if (prec == PM_PREC_LINE && line32_tile(op->nz) > LINE32_TILE)
     return set_error(PM_ECUDA, "line preconditioner: columns too tall for shared memory");
+  if (prec == PM_PREC_LINE && (st = line32_setup(op, proj))) return st;
   if ((st = ensure_prec(op, which, prec, s))) return st;
   if ((st = ensure_mixed(op, which, o->precision, prec, s))) return st;
   const int vs = which_valset(which);

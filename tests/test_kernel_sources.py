@@ -23,6 +23,18 @@ def _early_kernels():
     return out
 
 
+def test_nothing_of_a_device_is_kept_for_the_process():
+    """A kernel's shared-memory limit and occupancy belong to the device that was current. Kept in a function's static, they
+    would hold for the first device alone: an operator on a second one could not launch tiles above 48 KB."""
+    kept = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        src = open(path).read()
+        kept += [(os.path.basename(path), m.group(0).strip())
+                 for m in re.finditer(r"^[ \t]+static (?:const )?(?:bool|int|size_t) \w+[^;(]*[;=].*$", src, re.M)
+                 if "constexpr" not in m.group(0)]
+    assert not kept, kept
+
+
 def test_kernels_launched_early_read_nothing_as_constant_after_their_wait():
     """A kernel launched ahead of its predecessor's end is resident while that one still writes. A const
     __restrict__ parameter or __ldg may be a read-only load, which is defined only for data that nobody writes
