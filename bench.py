@@ -202,6 +202,7 @@ def run_cpu_oracle_all_cores(max_workers: int = 16):
 
 # live timing classes of the library (index = KT_* value) and the kernels they stand for
 KT_NAMES = ("k_cg_spmv", "k_cg_update", "k_cg_rho+k_cg_pupd", "k_ic0_sweep", "k_update_line")
+KT_RESIDENT = 5     # one launch that runs a whole solve (basins below about 3M rows), all phases in it
 SMS, FP64_FMA_PER_CLK_SM = 152, 2
 
 
@@ -211,11 +212,13 @@ def fp64_peak_tflops(sm_mhz):
     return SMS * FP64_FMA_PER_CLK_SM * 2 * float(sm_mhz) * 1e6 / 1e12
 
 
-def roofline_of(kt, n, steps, ms_total, peak, peak_kind, sm_mhz=None):
+def roofline_of(kt, n, steps, ms_total, peak, peak_kind, sm_mhz=None, solve_bytes=0.0):
     """Roofline of the dominant kernel class. kt: {class: (total ms, launches)} over `steps`
-    steps of an n-row basin. Algorithmic bytes per launch per class (each array once); the FP64
-    SpMV is bound by the FP64 pipe (ncu: 83 % busy, DRAM 44 %), so when it dominates it is
-    reported as "alu" against the FP64 peak, with its HBM-equivalent rate beside it."""
+    steps of an n-row basin, whose solves move solve_bytes in all. Algorithmic bytes per launch
+    per class (each array once); the FP64 SpMV is bound by the FP64 pipe (ncu: 83 % busy, DRAM
+    44 %), so when it dominates it is reported as "alu" against the FP64 peak, with its
+    HBM-equivalent rate beside it. Resident launches (whole solves) share the bytes that the other
+    classes' launches do not account for."""
     per_launch_bytes = {
         0: n * (15 * 8 + 8 + 8),            # SpMV: values, p (gathers cached), w
         1: n * (4 * 8 + 2 * 8),             # IC0 path update: x, r, p, w read; x, r written
@@ -226,11 +229,18 @@ def roofline_of(kt, n, steps, ms_total, peak, peak_kind, sm_mhz=None):
     }
     spmv_flops = 2 * 16 * n                 # 15 slot FMAs and the (p, Ap) FMA per row
     live = {k: v for k, v in kt.items() if v[1] > 0}
+    names = dict(enumerate(KT_NAMES))
+    if KT_RESIDENT in live:
+        names[KT_RESIDENT] = "k_resident"
+        streamed = sum(per_launch_bytes[k] * v[1] for k, v in live.items() if k != KT_RESIDENT)
+        per_launch_bytes[KT_RESIDENT] = max(solve_bytes - streamed, 0.0) / live[KT_RESIDENT][1]
+    if not live:     # no system had work to do
+        return {"kernel": None, "kernel_share_of_step": 0.0, "classes": {}}
     dom = max(live, key=lambda k: live[k][0])
     dom_ms, dom_launches = live[dom]
     avg_s = dom_ms * 1e-3 / dom_launches
     gbs = per_launch_bytes[dom] / avg_s / 1e9
-    out = {"kernel": KT_NAMES[dom], "traffic": dram_traffic(KT_NAMES[dom]),
+    out = {"kernel": names[dom], "traffic": dram_traffic(names[dom]),
            "kernel_share_of_step": round(dom_ms / max(ms_total, 1e-9), 4)}
     if dom == 0:
         pk = fp64_peak_tflops(sm_mhz or 2070.0)
@@ -244,11 +254,11 @@ def roofline_of(kt, n, steps, ms_total, peak, peak_kind, sm_mhz=None):
     else:
         out.update({"bound": "hbm", "achieved": round(gbs, 1), "peak": peak, "unit": "GB/s",
                     "frac": round(gbs / peak, 4), "peak_source": peak_kind})
-    out["classes_ms_per_step"] = {KT_NAMES[k]: round(v[0] / steps, 3) for k, v in kt.items()}
-    out["classes"] = {KT_NAMES[k]: {"launches_per_step": v[1] // max(steps, 1),
-                                    "us_per_launch": round(v[0] * 1e3 / v[1], 1),
-                                    "gbs": round(per_launch_bytes[k] / (v[0] * 1e-3 / v[1]) / 1e9, 1),
-                                    "frac": round(per_launch_bytes[k] / (v[0] * 1e-3 / v[1]) / 1e9 / peak, 4)}
+    out["classes_ms_per_step"] = {names[k]: round(v[0] / steps, 3) for k, v in kt.items() if k in names}
+    out["classes"] = {names[k]: {"launches_per_step": v[1] // max(steps, 1),
+                                 "us_per_launch": round(v[0] * 1e3 / v[1], 1),
+                                 "gbs": round(per_launch_bytes[k] / (v[0] * 1e-3 / v[1]) / 1e9, 1),
+                                 "frac": round(per_launch_bytes[k] / (v[0] * 1e-3 / v[1]) / 1e9 / peak, 4)}
                       for k, v in live.items()}
     return out
 
@@ -674,8 +684,9 @@ def run_ours(args):
     st = pm.State(op)
     t1 = torch.from_numpy(op.column_field(basin.theta[0])).cuda()
     t2 = torch.from_numpy(op.column_field(basin.theta[1])).cuda()
-    vel = pm.Options(rtol=1e-8, prec=pm.PREC_IC0, max_iter=500000)
-    pres = pm.Options(rtol=1e-8, prec=pm.PREC_LINE, max_iter=500000)
+    kernel = pm.KERNEL_STREAM if args.kernel == "stream" else pm.KERNEL_AUTO
+    vel = pm.Options(rtol=1e-8, prec=pm.PREC_IC0, max_iter=500000, kernel=kernel)
+    pres = pm.Options(rtol=1e-8, prec=pm.PREC_LINE, max_iter=500000, kernel=kernel)
 
     def one_step(v=vel, p=pres, allow=False):
         return pm.project_step(op, st, t1, t2, v, p, allow_not_converged=allow)
@@ -710,7 +721,7 @@ def run_ours(args):
     ms_total = ev[0].elapsed_time(ev[-1])
     ms_steps = [ev[k].elapsed_time(ev[k + 1]) for k in range(args.steps)]
     kt = {k: api.kernel_timing_get(k) for k in (api.KT_SPMV, api.KT_UPDATE, api.KT_PUPDATE, api.KT_IC0,
-                                                 api.KT_LINE)}
+                                                 api.KT_LINE, api.KT_RESIDENT)}
     api.kernel_timing(False)
     clk = clocks.stop()
 
@@ -727,7 +738,8 @@ def run_ours(args):
     # roofline of the dominant kernel class, timed live with events on the solve stream
     n = op.n
     peak, peak_kind = measured_peaks()
-    roofline = roofline_of(kt, n, args.steps, ms_total, peak, peak_kind, (clk or {}).get("sm_mhz"))
+    roofline = roofline_of(kt, n, args.steps, ms_total, peak, peak_kind, (clk or {}).get("sm_mhz"),
+                           bytes_step * args.steps)
 
     # end to end through the C ABI with host buffers: the same timed steps replayed from the
     # snapshot, theta in and (u1, u2, u3, p) out every step; diagnostics read after each step
@@ -801,8 +813,8 @@ def run_ours(args):
         ref = fp64_fields_at[k_m]
         ms_fp64 = sum(ms_steps[:k_m]) / k_m
         for label, prc in (("fp32", pm.FP32_REFINE), ("bf16", pm.BF16_REFINE)):
-            vm = pm.Options(rtol=1e-8, prec=pm.PREC_IC0, precision=prc, max_iter=60000)
-            pmo = pm.Options(rtol=1e-8, prec=pm.PREC_LINE, precision=prc, max_iter=60000)
+            vm = pm.Options(rtol=1e-8, prec=pm.PREC_IC0, precision=prc, max_iter=60000, kernel=kernel)
+            pmo = pm.Options(rtol=1e-8, prec=pm.PREC_LINE, precision=prc, max_iter=60000, kernel=kernel)
             try:
                 st.restore(snap)      # untimed first pass: operator copies, factors, workspace
                 one_step(vm, pmo, True)
@@ -955,6 +967,9 @@ def main():
     ap.add_argument("--prec", default="ic0", choices=["ic0", "jacobi", "line"])
     ap.add_argument("--nx", type=int, default=512,
                     help="basin columns per side (512 = the benchmark workload; smaller for profiling)")
+    ap.add_argument("--kernel", default="auto", choices=["auto", "stream"],
+                    help="stream: the step's solves by one kernel per phase whatever their size, as a basin below "
+                         "about 3M rows needs for a profile of the kernels that the benchmark workload runs")
     args = ap.parse_args()
     if args.cpu_worker:
         cpu_worker(args.steps, args.warmup)

@@ -381,7 +381,7 @@ int pm_last_error(char* buf, int32_t len);
 int64_t pm_kernel_launch_count(void);
 
 /* Live kernel timing. When enabled, the PCG driver brackets every launch of the kernel classes
- * below (stream solves; a resident solve is one launch of none of these classes) with CUDA events
+ * below (a stream solve's kernels, or the one launch of a resident solve) with CUDA events
  * on the solve's stream and accumulates their elapsed times at its own
  * synchronisation points. pm_kernel_timing(enable) switches it and resets the totals;
  * pm_kernel_timing_get returns the total milliseconds and launch count of one class. Process-
@@ -391,7 +391,8 @@ enum { PM_KT_SPMV = 0,    /* SpMV + (p, Ap) reduction, one launch per PCG iterat
        PM_KT_PUPDATE = 2, /* search-direction update (with the (r, z) reduction for IC0) */
        PM_KT_IC0 = 3,     /* the IC0 colour sweeps of one preconditioner apply (16 kernels) */
        PM_KT_LINE = 4,    /* the vertical-line solve fused with the (r, z) reduction     */
-       PM_KT_COUNT = 5 };
+       PM_KT_RESIDENT = 5, /* a whole resident solve, one launch                         */
+       PM_KT_COUNT = 6 };
 int pm_kernel_timing(int32_t enable);
 int pm_kernel_timing_get(int32_t kind, double* total_ms, int64_t* launches);
 

@@ -125,7 +125,7 @@ SIGNATURES = {
     "pm_build_flags": (ctypes.c_int32, []),
 }
 
-KT_SPMV, KT_UPDATE, KT_PUPDATE, KT_IC0, KT_LINE = 0, 1, 2, 3, 4
+KT_SPMV, KT_UPDATE, KT_PUPDATE, KT_IC0, KT_LINE, KT_RESIDENT = 0, 1, 2, 3, 4, 5
 
 
 def kernel_timing(enable: bool):

@@ -2168,6 +2168,7 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
     a.dinv = prec == PM_PREC_NONE ? nullptr : op->d_dinv32[which];
     a.ic0 = op->d_ic0_32[which];
     a.line = op->d_line32[which];
+    KtScope t(PM_KT_RESIDENT, 1, s);
     st = o->precision == PM_FP32_REFINE ? resident::launch_fp32(a, prec, cluster, op->num_sms, s)
                                         : resident::launch_bf16(a, prec, cluster, op->num_sms, s);
   } else {
@@ -2179,10 +2180,12 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
     a.dinv = prec == PM_PREC_NONE ? nullptr : op->d_dinv[which];
     a.ic0 = op->ic0[which].F;
     a.line = op->d_line[which];
+    KtScope t(PM_KT_RESIDENT, 1, s);
     st = resident::launch_fp64(a, prec, cluster, op->num_sms, s);
   }
   if (st) return st;
   if ((st = cuda_check(cudaStreamSynchronize(s), "resident pcg"))) return st;
+  if (!g_kt.pending.empty()) kt_collect();
   if ((st = resident::outcome(*a.out))) return st;
   const resident::Result h = a.out->res;
   if (stats) {
