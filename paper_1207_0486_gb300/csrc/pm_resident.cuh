@@ -219,26 +219,26 @@ struct Team {
   }
 };
 
-// A block's rows [r0, r1); with the line preconditioner they are its whole columns [c0, c1).
-struct Share {
-  int r0, r1, c0, c1;
-};
+// A block's share: whole columns [c0, c1) with the line preconditioner, else rows. Only one of the pairs is kept
+// in registers (with both, line solves of 1M to 3M rows were 3 to 7 % slower).
 template <int PREC>
-__device__ __forceinline__ Share share_of(const Geom& g, int rank, int G) {
-  Share s;
-  if (PREC == PM_PREC_LINE) {
-    s.c0 = (int)((int64_t)g.ncols * rank / G);
-    s.c1 = (int)((int64_t)g.ncols * (rank + 1) / G);
-    s.r0 = s.c0 * g.nz;
-    s.r1 = s.c1 * g.nz;
-  } else {   // in runs of 32 rows, so that a warp's accesses are aligned
-    const int64_t runs = (g.n + 31) / 32;
-    s.c0 = s.c1 = 0;
-    s.r0 = (int)min(g.n, 32 * (runs * rank / G));
-    s.r1 = (int)min(g.n, 32 * (runs * (rank + 1) / G));
+struct Share {
+  int first, past;
+  __device__ __forceinline__ Share(const Geom& g, int rank, int G) {
+    if (PREC == PM_PREC_LINE) {
+      first = (int)((int64_t)g.ncols * rank / G);
+      past = (int)((int64_t)g.ncols * (rank + 1) / G);
+    } else {   // in runs of 32 rows, so that a warp's accesses are aligned
+      const int64_t runs = (g.n + 31) / 32;
+      first = (int)min(g.n, 32 * (runs * rank / G));
+      past = (int)min(g.n, 32 * (runs * (rank + 1) / G));
+    }
   }
-  return s;
-}
+  __device__ __forceinline__ int row0(const Geom& g) const { return PREC == PM_PREC_LINE ? first * g.nz : first; }
+  __device__ __forceinline__ int row1(const Geom& g) const { return PREC == PM_PREC_LINE ? past * g.nz : past; }
+  __device__ __forceinline__ int col0() const { return first; }   // line preconditioner
+  __device__ __forceinline__ int col1() const { return past; }
+};
 
 // Neighbour q, by its index within its class, of the column at place i in class order (-1: none).
 __device__ __forceinline__ int ccls_of(const Args& a, int i, int q) {
@@ -492,14 +492,14 @@ __device__ __forceinline__ bool ic0_backward(const Args& a, Team<CL>& team, T al
 // r -= alpha w (UPDATE), then z by the preconditioner, on this block's rows. LINE: zt is the
 // block's tile of columns, ld apart (shared memory, or its part of the z vector).
 template <typename T, int PREC, bool UPDATE>
-__device__ __forceinline__ void update_rows(const Args& a, const Share& sh, T alpha, T* zt, int ld, Dots<T>& dots) {
+__device__ __forceinline__ void update_rows(const Args& a, const Share<PREC>& sh, T alpha, T* zt, int ld, Dots<T>& dots) {
   const Geom& g = a.g;
-  const int nz = g.nz, row1 = sh.r1;
+  const int nz = g.nz, row1 = sh.row1(a.g);
   T* r = static_cast<T*>(a.r);
   const T* w = static_cast<const T*>(a.w);
   const T* dinv = static_cast<const T*>(a.dinv);
   constexpr int U = 4;   // rows whose loads are in flight together
-  for (int i0 = sh.r0 + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
+  for (int i0 = sh.row0(a.g) + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
     T rv[U], wv[U], dv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -525,7 +525,7 @@ __device__ __forceinline__ void update_rows(const Args& a, const Share& sh, T al
         if (a.proj) add_m(dots.mz, a, row, zi);
       } else {
         const int col = fdiv(g.nzd, row), k = row - col * nz;
-        if (PREC == PM_PREC_LINE) zt[(col - sh.c0) * ld + k] = ri;
+        if (PREC == PM_PREC_LINE) zt[(col - sh.col0()) * ld + k] = ri;
         else colour0_y(a, col, k, ri, dots.rz);
       }
     }
@@ -535,8 +535,8 @@ __device__ __forceinline__ void update_rows(const Args& a, const Share& sh, T al
   // Thomas solve of each column, one thread per column; (r, z) = sum_k t_k y_k (symmetric blocks)
   const T* F = static_cast<const T*>(a.line);
   const int nc = g.ncols, n = (int)g.n;
-  for (int col = sh.c0 + (int)threadIdx.x; col < sh.c1; col += NT) {
-    T* cs = zt + (col - sh.c0) * ld;
+  for (int col = sh.col0() + (int)threadIdx.x; col < sh.col1(); col += NT) {
+    T* cs = zt + (col - sh.col0()) * ld;
     T y = 0;
 #pragma unroll 8
     for (int k = 0; k < nz; ++k) {
@@ -555,9 +555,9 @@ __device__ __forceinline__ void update_rows(const Args& a, const Share& sh, T al
   }
   __syncthreads();
   if (!a.proj) return;
-  for (int row = sh.r0 + (int)threadIdx.x; row < row1; row += NT) {
+  for (int row = sh.row0(a.g) + (int)threadIdx.x; row < row1; row += NT) {
     const int col = fdiv(g.nzd, row);
-    add_m(dots.mz, a, row, zt[(col - sh.c0) * ld + row - col * nz]);
+    add_m(dots.mz, a, row, zt[(col - sh.col0()) * ld + row - col * nz]);
   }
 }
 
@@ -565,16 +565,16 @@ __device__ __forceinline__ void update_rows(const Args& a, const Share& sh, T al
 // here anyway. FIRST: p = z - c.
 // LAST: x alone, when no further direction is needed.
 template <typename T, int PREC, bool FIRST, bool LAST>
-__device__ __forceinline__ void direction(const Args& a, const Share& sh, T alpha, T beta, T c, const T* zt, int ld) {
+__device__ __forceinline__ void direction(const Args& a, const Share<PREC>& sh, T alpha, T beta, T c, const T* zt, int ld) {
   const Geom& g = a.g;
-  const int nz = g.nz, row1 = sh.r1;
+  const int nz = g.nz, row1 = sh.row1(a.g);
   T* p = static_cast<T*>(a.p);
   T* x = iterate<T>(a);
   const T* r = static_cast<const T*>(a.r);
   const T* zv = static_cast<const T*>(a.z);
   const T* dinv = static_cast<const T*>(a.dinv);
   constexpr int U = 4;
-  for (int i0 = sh.r0 + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
+  for (int i0 = sh.row0(a.g) + (int)threadIdx.x; i0 < row1; i0 += U * NT) {
     T z[U], pv[U], xv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -584,7 +584,7 @@ __device__ __forceinline__ void direction(const Args& a, const Share& sh, T alph
           z[u] = (dinv ? __ldg(dinv + row) : (T)1) * r[row];
         } else if (PREC == PM_PREC_LINE) {
           const int col = fdiv(g.nzd, row);
-          z[u] = zt[(col - sh.c0) * ld + row - col * nz];
+          z[u] = zt[(col - sh.col0()) * ld + row - col * nz];
         } else {
           const int col = fdiv(g.nzd, row);
           z[u] = zv[colour_pos(a, col, row - col * nz)];
@@ -616,7 +616,7 @@ struct Cg {
 // known: true ends the step with x moved (the recursion has met its target). cg.status is PM_BREAKDOWN
 // when rho is not positive. Returns false when a wait ran out.
 template <typename T, int PREC, bool FIRST, bool CL, typename Stop>
-__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Share& sh, T* zt, int ld, double alpha, Cg& cg,
+__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Share<PREC>& sh, T* zt, int ld, double alpha, Cg& cg,
                                         bool& stopped, Stop stop) {
   Dots<T> dots;
   update_rows<T, PREC, !FIRST>(a, sh, (T)alpha, zt, ld, dots);
@@ -632,7 +632,7 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Sha
       const T* r = static_cast<const T*>(a.r);
       const T* z = static_cast<const T*>(a.z);
       AccFor<T> rz;
-      for (int row = sh.r0 + (int)threadIdx.x; row < sh.r1; row += NT) {
+      for (int row = sh.row0(a.g) + (int)threadIdx.x; row < sh.row1(a.g); row += NT) {
         const int col = fdiv(a.g.nzd, row);
         const T zi = z[colour_pos(a, col, row - col * a.g.nz)];
         rz.add_prod(r[row], zi);
@@ -675,14 +675,14 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Sha
 }
 
 // w = A p on the block's rows; v = (p, w) over the team.
-template <typename T, typename TV, bool CL>
-__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const Share& sh, double& pw) {
+template <typename T, typename TV, bool CL, int PREC>
+__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const Share<PREC>& sh, double& pw) {
   const Geom& g = a.g;
   const TV* val = static_cast<const TV*>(a.val);
   const T* p = static_cast<const T*>(a.p);
   T* w = static_cast<T*>(a.w);
   AccFor<T> acc;
-  for (int row = sh.r0 + (int)threadIdx.x; row < sh.r1; row += NT) {
+  for (int row = sh.row0(a.g) + (int)threadIdx.x; row < sh.row1(a.g); row += NT) {
     const int col = fdiv(g.nzd, row);
     const T wi = row_apply<T, TV>(g, val, p, a.mask, row, col, row - col * g.nz);
     w[row] = wi;
@@ -695,13 +695,13 @@ __device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const S
 }
 
 // r = b - A x (compensated), (r, r) and the floor's (|A||x| + |b|)^2 over the team.
-template <typename T, bool CL>
-__device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, const Share& sh, const double* b, double& rr,
+template <typename T, bool CL, int PREC>
+__device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, const Share<PREC>& sh, const double* b, double& rr,
                                               double& ff) {
   const Geom& g = a.g;
   T* r = static_cast<T*>(a.r);
   double v[2] = {0.0, 0.0};
-  for (int row = sh.r0 + (int)threadIdx.x; row < sh.r1; row += NT) {
+  for (int row = sh.row0(a.g) + (int)threadIdx.x; row < sh.row1(a.g); row += NT) {
     const int col = fdiv(g.nzd, row);
     double asum;
     const double bi = b[row];
@@ -718,14 +718,14 @@ __device__ __forceinline__ bool true_residual(const Args& a, Team<CL>& team, con
 }
 
 // Right-hand side, initial guess and first residual: (b', b') and (r, r). From x = 0 the residual is b' itself.
-template <typename T, bool CL>
-__device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, const Share& sh, const double*& b, double& bb,
+template <typename T, bool CL, int PREC>
+__device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, const Share<PREC>& sh, const double*& b, double& bb,
                                             double& rr) {
   double lam = 0.0, xs = 0.0;
   b = a.b;
   if (a.proj) {
     double v[2] = {0.0, 0.0};
-    for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) {
+    for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) {
       v[0] += b[i];
       if (a.x0_is_guess) v[1] = fma(a.m[i], a.x[i], v[1]);
     }
@@ -735,7 +735,7 @@ __device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, const
   }
   T* r = static_cast<T*>(a.r);
   double v[2] = {0.0, 0.0};
-  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) {
+  for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) {
     double bi = b[i];
     if (a.proj) {
       bi = bi - lam * a.m[i];
@@ -760,19 +760,19 @@ __device__ __forceinline__ bool start_solve(const Args& a, Team<CL>& team, const
 }
 
 // The returned pressure has m'x = 0.
-template <bool CL>
-__device__ __forceinline__ bool zero_mean(const Args& a, Team<CL>& team, const Share& sh) {
+template <bool CL, int PREC>
+__device__ __forceinline__ bool zero_mean(const Args& a, Team<CL>& team, const Share<PREC>& sh) {
   double v[1] = {0.0};
-  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) v[0] = fma(a.m[i], a.x[i], v[0]);
+  for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) v[0] = fma(a.m[i], a.x[i], v[0]);
   if (!team.template sum<1>(v)) return false;
   const double shift = v[0] / a.one_m;
-  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.x[i] -= shift;
+  for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) a.x[i] -= shift;
   return true;
 }
 
 // The FP64 solve: PCG on the recursive residual, then the true residual, restarts while they help.
 template <int PREC, bool CL>
-__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, const Share& sh, double* zt, int ld, Result& o) {
+__device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, const Share<PREC>& sh, double* zt, int ld, Result& o) {
   const double* b;
   double bb, rr;
   if (!start_solve<double>(a, team, sh, b, bb, rr)) return false;
@@ -785,7 +785,7 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, const Sha
   if (!skip && a.max_iter == 0 && bb != 0.0) cg.status = PM_NOT_CONVERGED;
   cg.rr = rr;
   if (bb == 0.0)
-    for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.x[i] = 0.0;
+    for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) a.x[i] = 0.0;
   while (bb != 0.0) {
     if (cg.status == PM_OK && !skip) {
       bool converged = false, stopped;
@@ -838,17 +838,17 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, const Sha
 // recursive residual has dropped by inner_rtol, or claims convergence, the FP32 correction is folded into the
 // FP64 iterate, the true residual b - A x is formed (compensated) and a new inner solve starts from it.
 template <typename TV, int PREC, bool CL>
-__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, const Share& sh, float* zt, int ld, Result& o) {
+__device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, const Share<PREC>& sh, float* zt, int ld, Result& o) {
   const double* b;
   double bb, rr;
-  for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.d[i] = 0.f;
+  for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) a.d[i] = 0.f;
   if (!start_solve<float>(a, team, sh, b, bb, rr)) return false;
   const double tol2 = a.rtol * a.rtol * bb, drop = a.inner_rtol * a.inner_rtol;
   Cg cg;
   int outer = 0, stalled = 0;
   double rel_true = 0.0, floor = 0.0, prev_true = 1e300;
   if (bb == 0.0) {
-    for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) a.x[i] = 0.0;
+    for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) a.x[i] = 0.0;
   } else if (rr <= tol2 || a.max_iter == 0) {   // x0 already meets rtol, or no iteration is allowed
     if (!(rr <= tol2)) cg.status = PM_NOT_CONVERGED;   // not a number included
     rel_true = sqrt(rr / bb);
@@ -871,7 +871,7 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, const
         if (!fine) return false;
         if (stopped) break;
       }
-      for (int i = sh.r0 + (int)threadIdx.x; i < sh.r1; i += NT) {
+      for (int i = sh.row0(a.g) + (int)threadIdx.x; i < sh.row1(a.g); i += NT) {
         a.x[i] += (double)a.d[i];
         a.d[i] = 0.f;
       }
@@ -937,13 +937,13 @@ __global__ void __launch_bounds__(NT, 1) k_resident(Args a) {
   __syncthreads();
   Team<CL> team(a, &scratch);
   if (CL) team.barrier();   // every block of the cluster runs before one writes to another's shared memory
-  const Share sh = share_of<PREC>(a.g, team.rank, team.G);
+  const Share<PREC> sh(a.g, team.rank, team.G);
   T* zt;
   int ld = a.g.nz | 1;   // odd: a warp's columns fall into different banks
   if (a.z_in_smem) {
     zt = reinterpret_cast<T*>(smem_raw);
   } else {
-    zt = static_cast<T*>(a.z) + (PREC == PM_PREC_LINE ? sh.r0 : 0);
+    zt = static_cast<T*>(a.z) + (PREC == PM_PREC_LINE ? sh.row0(a.g) : 0);
     ld = a.g.nz;
   }
   Result o;
