@@ -39,7 +39,6 @@ namespace na {
 
 constexpr int64_t MAXR = PM_NOALLOC_MAX_ROWS;
 constexpr int TPB = 256;
-constexpr int64_t CLUSTER_ROWS = 8192;   // one cluster of blocks up to here, as pm_pcg_solve's Jacobi solves
 constexpr int64_t OFF_R = 0;
 constexpr int64_t OFF_P = 1 * MAXR;
 constexpr int64_t OFF_W = 2 * MAXR;
@@ -131,7 +130,7 @@ int run(pm_operator* op, int which, const double* b, double* x, const pm_solve_o
   }
   int st = cuda_check(cudaMemsetAsync(a.out, 0xff, sizeof(resident::Out), s), "noalloc results");
   if (st) return st;
-  if ((st = resident::launch_fp64(a, PM_PREC_JACOBI, n <= CLUSTER_ROWS, op->num_sms, s))) return st;
+  if ((st = resident::launch_fp64(a, PM_PREC_JACOBI, op->num_sms, s))) return st;
   resident::Out got;
   if ((st = cuda_check(cudaMemcpyAsync(&got, a.out, sizeof(got), cudaMemcpyDeviceToHost, s), "noalloc results"))) return st;
   if ((st = cuda_check(cudaStreamSynchronize(s), "noalloc pcg"))) return st;

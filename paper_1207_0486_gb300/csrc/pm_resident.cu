@@ -4,8 +4,8 @@
 namespace pm {
 namespace resident {
 
-int launch_fp64(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s) {
-  return launch<double, double>(a, prec, cluster, num_sms, s);
+int launch_fp64(Args& a, int prec, int num_sms, cudaStream_t s) {
+  return launch<double, double>(a, prec, num_sms, s);
 }
 
 // One block takes the parts of both: as rank 1 of two it waits for an arrival that never comes, then it

@@ -12,7 +12,8 @@
 //     cycles, 3000 with stores to publish;
 //   - cluster: 16 blocks of one thread-block cluster, the hardware cluster barrier (550 to 980 cycles, 2000
 //     with global stores to publish), block sums exchanged through distributed shared memory: for systems so
-//     small that the grid barrier would cost more than the work the other SMs take over.
+//     small that the grid barrier would cost more than the work the other SMs take over. The smallest have a
+//     team of one block, whose barrier is the block's own: no fence, and L1 keeps what it holds between phases.
 //
 // Rows: the line preconditioner works on whole columns, dealt evenly and contiguously to the blocks; without it
 // a block takes an even share of the rows, however few columns they make up (16 columns of 20,000 levels, Jacobi:
@@ -117,6 +118,7 @@ struct Scratch {
   double v[4][NT];
   double q[4][128];
   double res[4];
+  double sc[3];                // block_scalars
   double xch[2][4][CLUSTER];   // cluster team: the blocks' sums
   int ok;
   int first[8], past[8];       // this block's share of each colour's rows
@@ -137,7 +139,7 @@ struct Team {
   // This block's stores so far are published; wait() returns when every block has arrived.
   __device__ __forceinline__ void arrive() {
     if (CL) {
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      if (G > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     } else {
       __syncthreads();
       if (threadIdx.x == 0) red_release(&ctl->arrive);
@@ -146,7 +148,8 @@ struct Team {
   }
   __device__ __forceinline__ bool wait() {
     if (CL) {
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      if (G > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      else __syncthreads();
       return true;
     }
     if (threadIdx.x == 0) {
@@ -174,6 +177,7 @@ struct Team {
   template <int NV>
   __device__ __forceinline__ bool sum(double (&v)[NV]) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const bool alone = CL && G == 1;
     static_assert(NT == 512 && NV <= 4, "four warps per value");
 #pragma unroll
     for (int i = 0; i < NV; ++i) s->v[i][tid] = v[i];
@@ -186,7 +190,9 @@ struct Team {
     if (wid < NV) {
       const double* c = s->q[wid] + lane;
       double t = warp_sum((c[0] + c[32]) + (c[64] + c[96]));
-      if (CL) {
+      if (alone) {
+        if (lane == 0) s->res[wid] = t;
+      } else if (CL) {
         t = __shfl_sync(0xffffffffu, t, 0);
         if (lane < G) {
           const uint32_t local = (uint32_t)__cvta_generic_to_shared(&s->xch[buf][wid][rank]);
@@ -201,7 +207,7 @@ struct Team {
     }
     arrive();
     if (!wait()) return false;
-    if (wid < NV) {
+    if (wid < NV && !alone) {
       double t = 0.0;
       if (CL) {
         t = lane < G ? s->xch[buf][wid][lane] : 0.0;
@@ -211,13 +217,26 @@ struct Team {
       t = warp_sum(t);
       if (lane == 0) s->res[wid] = t;
     }
-    __syncthreads();
+    if (!alone) __syncthreads();
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = s->res[i];
     buf ^= 1;
     return true;
   }
 };
+
+// Scalars formed from a sum, by one thread for its block. A division takes some ten instructions of the FP64 pipe, 64
+// cycles each per warp and sub-core: repeated by 16 warps, the three of an iteration held the pipe for about 7,500
+// cycles. By one thread: 512 rows, Jacobi pressure, 3.06 -> 2.38 ms (one block of 8 warps had taken 2.82); 0.06M 9 to 14 %
+// less by the diagonal, 6 to 10 % by columns, 4 % IC0; nothing from 2M rows on.
+template <int NV, typename F>
+__device__ __forceinline__ void block_scalars(Scratch* s, double (&out)[NV], F f) {
+  static_assert(NV <= 3, "Scratch::sc");
+  if (threadIdx.x == 0) f(s->sc);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) out[i] = s->sc[i];
+}
 
 // A block's share: whole columns [c0, c1) with the line preconditioner, else rows. Only one of the pairs is kept
 // in registers (with both, line solves of 1M to 3M rows were 3 to 7 % slower).
@@ -616,17 +635,29 @@ struct Cg {
 // known: true ends the step with x moved (the recursion has met its target). cg.status is PM_BREAKDOWN
 // when rho is not positive. Returns false when a wait ran out.
 template <typename T, int PREC, bool FIRST, bool CL, typename Stop>
-__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Share<PREC>& sh, T* zt, int ld, double alpha, Cg& cg,
-                                        bool& stopped, Stop stop) {
+__device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Share<PREC>& sh, T* zt, int ld,
+                                        double alpha, Cg& cg, bool& stopped, Stop stop) {
   Dots<T> dots;
   update_rows<T, PREC, !FIRST>(a, sh, (T)alpha, zt, ld, dots);
-  double c = 0.0, rho = 0.0;
+  double c = 0.0, rho = 0.0, beta64 = 0.0;
+  const auto scalars = [&](double rz, double mz, double sr) {
+    double u[3];
+    block_scalars(team.s, u, [&](double* o) {
+      o[0] = a.proj ? mz / a.one_m : 0.0;
+      o[1] = a.proj ? rz - o[0] * sr : rz;
+      o[2] = FIRST ? 0.0 : o[1] / cg.rho;
+    });
+    c = u[0];
+    rho = u[1];
+    beta64 = u[2];
+  };
   if (PREC == PM_PREC_IC0) {
     double v[1] = {dots.rr.value()};
     if (!team.template sum<1>(v)) return false;
     cg.rr = v[0];
     stopped = stop();
     if (!stopped && !ic0_forward<T>(a, team, dots.rz, rho)) return false;
+    if (!stopped && !a.proj) scalars(rho, 0.0, 0.0);
     if (!stopped && a.proj) {   // the projection needs the whole z before p
       if (!ic0_backward<T, false>(a, team, (T)0, (T)0)) return false;
       const T* r = static_cast<const T*>(a.r);
@@ -640,21 +671,19 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Sha
       }
       double u[3] = {rz.value(), dots.mz.value(), dots.sr.value()};
       if (!team.template sum<3>(u)) return false;
-      c = u[1] / a.one_m;
-      rho = u[0] - c * u[2];
+      scalars(u[0], u[1], u[2]);
     }
   } else if (a.proj) {
     double v[4] = {dots.rr.value(), dots.rz.value(), dots.mz.value(), dots.sr.value()};
     if (!team.template sum<4>(v)) return false;
     cg.rr = v[0];
-    c = v[2] / a.one_m;
-    rho = v[1] - c * v[3];
+    scalars(v[1], v[2], v[3]);
     stopped = stop();
   } else {
     double v[2] = {dots.rr.value(), dots.rz.value()};
     if (!team.template sum<2>(v)) return false;
     cg.rr = v[0];
-    rho = v[1];
+    scalars(v[1], 0.0, 0.0);
     stopped = stop();
   }
   const bool broken = !stopped && (!(rho > 0.0) || !isfinite(rho));
@@ -663,7 +692,7 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Sha
     direction<T, PREC, FIRST, true>(a, sh, (T)alpha, (T)0, (T)0, zt, ld);
     return team.barrier();
   }
-  const T beta = FIRST ? (T)0 : (T)(rho / cg.rho);
+  const T beta = (T)beta64;
   cg.rho = rho;
   if (PREC == PM_PREC_IC0 && !a.proj) {
     if (!FIRST) return ic0_backward<T, true>(a, team, (T)alpha, beta);
@@ -674,9 +703,10 @@ __device__ __forceinline__ bool advance(const Args& a, Team<CL>& team, const Sha
   return team.barrier();
 }
 
-// w = A p on the block's rows; v = (p, w) over the team.
+// w = A p on the block's rows; pw = (p, w) over the team and alpha = rho / pw.
 template <typename T, typename TV, bool CL, int PREC>
-__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const Share<PREC>& sh, double& pw) {
+__device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const Share<PREC>& sh, double rho, double& pw,
+                                          double& alpha) {
   const Geom& g = a.g;
   const TV* val = static_cast<const TV*>(a.val);
   const T* p = static_cast<const T*>(a.p);
@@ -691,6 +721,9 @@ __device__ __forceinline__ bool apply_dot(const Args& a, Team<CL>& team, const S
   double v[1] = {acc.value()};
   if (!team.template sum<1>(v)) return false;
   pw = v[0];
+  double u[1];
+  block_scalars(team.s, u, [&](double* o) { o[0] = rho / pw; });
+  alpha = u[0];
   return true;
 }
 
@@ -791,13 +824,13 @@ __device__ __forceinline__ bool solve64(const Args& a, Team<CL>& team, const Sha
       bool converged = false, stopped;
       if (!advance<double, PREC, true>(a, team, sh, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
       while (cg.status == PM_OK && cg.iter < a.max_iter) {
-        double pw;
-        if (!apply_dot<double, double>(a, team, sh, pw)) return false;
+        double pw, alpha;
+        if (!apply_dot<double, double>(a, team, sh, cg.rho, pw, alpha)) return false;
         if (!(pw > 0.0) || !isfinite(pw)) {
           cg.status = PM_BREAKDOWN;
           break;
         }
-        const bool fine = advance<double, PREC, false>(a, team, sh, zt, ld, cg.rho / pw, cg, stopped, [&] {
+        const bool fine = advance<double, PREC, false>(a, team, sh, zt, ld, alpha, cg, stopped, [&] {
           ++cg.iter;
           converged = cg.rr <= tol2;
           return converged || cg.iter >= a.max_iter;
@@ -858,13 +891,13 @@ __device__ __forceinline__ bool solve_mixed(const Args& a, Team<CL>& team, const
       bool stopped;
       if (!advance<float, PREC, true>(a, team, sh, zt, ld, 0.0, cg, stopped, [] { return false; })) return false;
       while (cg.status == PM_OK) {
-        double pw;
-        if (!apply_dot<float, TV>(a, team, sh, pw)) return false;
+        double pw, alpha;
+        if (!apply_dot<float, TV>(a, team, sh, cg.rho, pw, alpha)) return false;
         if (!(pw > 0.0) || !isfinite(pw)) {
           cg.status = PM_BREAKDOWN;
           break;
         }
-        const bool fine = advance<float, PREC, false>(a, team, sh, zt, ld, cg.rho / pw, cg, stopped, [&] {
+        const bool fine = advance<float, PREC, false>(a, team, sh, zt, ld, alpha, cg, stopped, [&] {
           ++cg.iter;
           return cg.rr <= target || cg.iter >= a.max_iter;
         });
@@ -968,7 +1001,9 @@ inline int launch_one(Args& a, int grid, size_t smem, cudaStream_t s) {
   if (smem && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_LIMIT),
                                "resident shared memory")))
     return st;
-  if (CL && (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster size")))
+  const bool team = !CL || grid > 1;   // more than one block
+  if (CL && team &&
+      (st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster size")))
     return st;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -985,8 +1020,8 @@ inline int launch_one(Args& a, int grid, size_t smem, cudaStream_t s) {
     at[0].val.cooperative = 1;
   }
   cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if ((st = cuda_check(cudaMemsetAsync(a.ctl, 0, sizeof(Ctl), s), "resident barrier"))) return st;
+  cfg.numAttrs = team ? 1 : 0;
+  if (!CL && (st = cuda_check(cudaMemsetAsync(a.ctl, 0, sizeof(Ctl), s), "resident barrier"))) return st;
   st = cuda_check(cudaLaunchKernelEx(&cfg, k_resident<T, TV, PREC, CL>, a), "k_resident");
   count_launch();
   return st;
@@ -1010,15 +1045,32 @@ int launch_prec(Args& a, int prec, int grid, cudaStream_t s) {
   }
 }
 
+// Blocks of a solve's team: one, one cluster's, or (0) the grid's. Measured, us per iteration or, marked ms, whole
+// solves:
+//   cluster / grid: IC0 n = 2,048 40 / 49, 18,000 50 / 49; line 11,803 18.3 / 18.1, 18,000 24 / 21; Jacobi 2,048
+//   10 / 14, 11,803 15.5 / 14.2;
+//   one block / cluster, FP64 velocity and pressure in ms: IC0 n = 512 0.22 / 0.29 and 3.40 / 4.84, 1,024 0.42 / 0.47 and
+//   7.57 / 9.09, 1,600 0.55 / 0.48 and 13.4 / 12.1; line 288 0.14 / 0.17 and 0.20 / 0.24, 512 0.20 / 0.21 and 0.33 / 0.35,
+//   648 0.25 / 0.24 and 0.46 / 0.44; Jacobi 288 0.15 / 0.17 and 1.41 / 1.66, 400 0.26 / 0.27 and 2.26 / 2.33, 512 0.22 / 0.20
+//   and 2.48 / 2.38. FP32 alike (IC0 1,024 0.40 / 0.38 and 7.2 / 11.0, Jacobi 400 0.28 / 0.30 and 3.4 / 3.9).
+constexpr int64_t ONE_BLOCK_ROWS = 400, ONE_BLOCK_IC0 = 1024;
+constexpr int64_t CLUSTER_ROWS = 8192, CLUSTER_IC0 = 16384;
+inline int team_blocks(int64_t n, int prec) {
+  const bool ic0 = prec == PM_PREC_IC0;
+  if (n <= (ic0 ? ONE_BLOCK_IC0 : ONE_BLOCK_ROWS)) return 1;
+  return n <= (ic0 ? CLUSTER_IC0 : CLUSTER_ROWS) ? CLUSTER : 0;
+}
+
 template <typename T, typename TV>
-int launch(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s) {
-  return cluster ? launch_prec<T, TV, true>(a, prec, CLUSTER, s) : launch_prec<T, TV, false>(a, prec, num_sms, s);
+int launch(Args& a, int prec, int num_sms, cudaStream_t s) {
+  const int blocks = team_blocks(a.g.n, prec);
+  return blocks ? launch_prec<T, TV, true>(a, prec, blocks, s) : launch_prec<T, TV, false>(a, prec, num_sms, s);
 }
 
 // One file each (pm_resident.cu, pm_resident_fp32.cu, pm_resident_bf16.cu), so that they compile side by side.
-int launch_fp64(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s);
-int launch_fp32(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s);
-int launch_bf16(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s);
+int launch_fp64(Args& a, int prec, int num_sms, cudaStream_t s);
+int launch_fp32(Args& a, int prec, int num_sms, cudaStream_t s);
+int launch_bf16(Args& a, int prec, int num_sms, cudaStream_t s);
 
 }  // namespace resident
 }  // namespace pm

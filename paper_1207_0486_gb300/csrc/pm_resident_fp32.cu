@@ -4,8 +4,8 @@
 namespace pm {
 namespace resident {
 
-int launch_fp32(Args& a, int prec, bool cluster, int num_sms, cudaStream_t s) {
-  return launch<float, float>(a, prec, cluster, num_sms, s);
+int launch_fp32(Args& a, int prec, int num_sms, cudaStream_t s) {
+  return launch<float, float>(a, prec, num_sms, s);
 }
 
 }  // namespace resident

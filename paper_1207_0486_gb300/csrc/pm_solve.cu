@@ -1466,9 +1466,6 @@ int pcg_run(pm_operator* op, int which, const double* b, double* x, const pm_sol
 constexpr int64_t RESIDENT_MAX_ROWS = 1 << 20;    // accepted when requested explicitly
 // Automatic choice of the resident solve (measured lines: resident_auto).
 constexpr int64_t RESIDENT_AUTO_ROWS = 3 << 20, RESIDENT_AUTO_IC0 = 2 << 20, RESIDENT_AUTO_MIXED_LINE = 5 << 18;
-// Up to here by one cluster of blocks. Measured, us per iteration, cluster / grid: IC0 n = 2,048 40 / 49, 18,000
-// 50 / 49; line 11,803 18.3 / 18.1, 18,000 24 / 21; Jacobi 2,048 10 / 14, 11,803 15.5 / 14.2.
-constexpr int64_t RESIDENT_CLUSTER_ROWS = 8192, RESIDENT_CLUSTER_IC0 = 16384;
 
 static_assert(sizeof(resident::Out) <= 64 && sizeof(resident::Ctl) <= 64, "resident buffers");
 
@@ -2154,7 +2151,6 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
   if (mixed && (st = ensure_mixed(op, which, o->precision, prec, s))) return st;
   resident::Args a = resident_args(op, which, b, x, o);
   const int vs = which_valset(which);
-  const bool cluster = op->n <= (prec == PM_PREC_IC0 ? RESIDENT_CLUSTER_IC0 : RESIDENT_CLUSTER_ROWS);
   a.out->res.status = -1;
   a.out->timeout = 0;
   if (mixed) {
@@ -2169,8 +2165,8 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
     a.ic0 = op->d_ic0_32[which];
     a.line = op->d_line32[which];
     KtScope t(PM_KT_RESIDENT, 1, s);
-    st = o->precision == PM_FP32_REFINE ? resident::launch_fp32(a, prec, cluster, op->num_sms, s)
-                                        : resident::launch_bf16(a, prec, cluster, op->num_sms, s);
+    st = o->precision == PM_FP32_REFINE ? resident::launch_fp32(a, prec, op->num_sms, s)
+                                        : resident::launch_bf16(a, prec, op->num_sms, s);
   } else {
     a.val = a.val64;
     a.r = c->r;
@@ -2181,7 +2177,7 @@ int resident_run(pm_operator* op, int which, const double* b, double* x, const p
     a.ic0 = op->ic0[which].F;
     a.line = op->d_line[which];
     KtScope t(PM_KT_RESIDENT, 1, s);
-    st = resident::launch_fp64(a, prec, cluster, op->num_sms, s);
+    st = resident::launch_fp64(a, prec, op->num_sms, s);
   }
   if (st) return st;
   if ((st = cuda_check(cudaStreamSynchronize(s), "resident pcg"))) return st;
