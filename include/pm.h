@@ -130,8 +130,13 @@ typedef struct pm_solve_opts {
 /* How a solve runs on the GPU (no paper counterpart; the iterates are those of the Section 5 PCG
  * either way). STREAM issues one kernel per phase of every PCG iteration over the whole GPU;
  * RESIDENT runs the whole solve in one cooperative launch of one block per SM (one cluster of 16 blocks for the
- * smallest systems), with a bounded grid barrier between phases (an expired wait returns PM_TIMEOUT) and one
- * wait on the host: for systems whose stream iterations are bound by launches. */
+ * smaller systems, one block for the smallest), with a bounded grid barrier between phases (an expired wait returns
+ * PM_TIMEOUT) and one wait on the host: for systems whose stream iterations are bound by launches. A resident solve
+ * above 8,192 rows (IC0 16,384) holds every SM until it ends, so that solves and other kernels on other streams wait for
+ * it, where STREAM's kernels interleave with them. One solve at a time is faster resident up to the AUTO
+ * limits, and so are two of less than a million rows; a program that solves from four or more threads at once, or that needs the GPU for other work meanwhile, gets
+ * more from STREAM (eight threads, FP64 line, 0.12M rows each: 13 us per system and iteration against 25; measured figures
+ * in csrc/pm_resident.cuh). */
 enum { PM_KERNEL_AUTO = 0, PM_KERNEL_STREAM = 1, PM_KERNEL_RESIDENT = 2 };
 
 typedef struct pm_solve_stats {

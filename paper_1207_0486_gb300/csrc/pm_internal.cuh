@@ -141,7 +141,7 @@ __host__ __device__ inline bool is_dirichlet(uint8_t flag, int k, int nz, int c)
 }
 
 // Division of a non-negative 32-bit integer by a divisor known on the host (a basin's levels per
-// column): q = (umulhi(t, mul) + t) >> shift, exact for 0 <= t < 2^31 and 1 <= d < 2^31. Four integer instructions where
+// column), by Granlund and Montgomery, "Division by invariant integers using multiplication" (1994): q = (umulhi(t, mul) + t) >> shift, exact for 0 <= t < 2^31 and 1 <= d < 2^31. Four integer instructions where
 // a division by a run-time value takes about twenty (32 bits) or a hundred (64 bits).
 struct FastDiv {
   uint32_t mul, shift;

@@ -31,8 +31,15 @@
 // sweep can form p at once. The pressure's projection needs m'z first: its IC0 sums and p follow the
 // sweeps as passes of their own.
 //
-// What bounds it: barriers and load latency below about 0.3M rows (IC0 51 us per iteration at 0.12M rows, where a
-// stream of kernels took 218), the FP64 pipe (64 cycles per warp instruction and sub-core) above.
+// What bounds it: barriers and load latency below about 0.3M rows (IC0 49 us per iteration at 0.12M rows; the stream of
+// kernels takes 132 now, and took 218 before its sweeps were in colour order), the FP64 pipe (64 cycles per warp
+// instruction and sub-core) above.
+//
+// A grid team holds every SM to the end of its solve (512 threads of 128 registers fill the register file): solves on
+// other streams queue behind it, where the stream's kernels interleave. Several solves at once, one operator
+// and host thread each, us per system and iteration, 1 / 2 / 4 / 8 threads: FP64 line, 0.12M rows, resident 25 / 25 / 25 /
+// 25, stream 51 / 30 / 20 / 13; FP64 IC0 41 / 41 / 41 / 41 and 77 / 43 / 29 / 21; FP64 IC0 2.0M 272 whatever the number and 285 /
+// 213 / 188 / 194. One cluster's or one block's solves do run side by side (2,048 rows, IC0: 7.3 / 3.8 / 1.9 / 1.2).
 #pragma once
 
 #include <cuda_bf16.h>

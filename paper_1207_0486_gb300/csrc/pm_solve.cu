@@ -1654,7 +1654,7 @@ __device__ __forceinline__ void ld4(const __nv_bfloat16* p, float (&v)[4]) {
 
 // k32_spmv for level counts that are multiples of 4: four consecutive rows of a column per thread, so that a
 // slot's values and a neighbour column's entries are one 16-byte load each (the entry above or below the four is a
-// load of its own): 45 loads for four rows instead of 148. The FP32 SpMV is bound by load instructions,
+// load of its own): 37 loads for four rows instead of 148. The FP32 SpMV is bound by load instructions,
 // not by its 68 bytes a row. Slots by the mask (structural slots, or a component's kept ones): a clear
 // bit's value is 0 or, eliminated, goes to the drop term.
 template <typename TV>

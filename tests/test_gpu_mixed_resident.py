@@ -1,4 +1,4 @@
-"""Mixed-precision solves in one launch: what is not a number never passes for a solution."""
+"""Mixed-precision solves in one launch: what is not a number never passes for a solution, and guesses are used."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -40,4 +40,29 @@ def test_last_iteration_that_overflows(precision, kernel):
                   allow_not_converged=True)
     assert st.iters == 1 and not bool(torch.isfinite(x).all())
     assert st.status == pm.PM_NOT_CONVERGED
+    op.close()
+
+
+@pytest.mark.parametrize("shape", [(40, 40, 12), (14, 15, 16)])   # 19,200 rows: the grid; 3,360: one cluster
+@pytest.mark.parametrize("precision", [pm.FP64, *MIXED])
+@pytest.mark.parametrize("which,prec", [(pm.OP_PRESSURE, pm.PREC_IC0), (pm.OP_PRESSURE, pm.PREC_LINE),
+                                        (pm.OP_PRESSURE, pm.PREC_JACOBI), (pm.OP_VEL_U3, pm.PREC_LINE)])
+def test_from_a_guess_that_has_not_converged(shape, precision, which, prec):
+    """Against the stream of kernels, from zero and from a random guess. Both solutions have a true residual of rtol, so
+    their difference has one of at most the two; an outer step or a restart ends where a residual passes its target,
+    which rounding can move by one step."""
+    op = pm.assemble_operator(box_basin(nh=shape[0], nhy=shape[1], nz=shape[2]))
+    b, guess = (torch.from_numpy(random_vector(op.n, seed)).cuda() for seed in (51, 52))
+    rtol = 1e-8
+    for from_guess in (False, True):
+        xs, outer = [], []
+        for kernel in KERNELS:
+            xs.append(guess.clone() if from_guess else torch.zeros_like(b))
+            st = op.solve(which, b, xs[-1], pm.Options(rtol=rtol, prec=prec, precision=precision, x0_is_guess=from_guess,
+                                                       inner_rtol=1e-2, kernel=kernel))
+            assert st.status == pm.PM_OK and st.rel_residual_true <= rtol and st.iters > 0
+            outer.append(st.outer_iters)
+        assert abs(outer[0] - outer[1]) <= 1
+        rr, _, _ = op.residual(which, torch.zeros_like(b), xs[0] - xs[1], torch.empty_like(b))
+        assert rr ** 0.5 <= 2 * 1.05 * rtol * float(b.norm())
     op.close()
