@@ -135,7 +135,7 @@ typedef struct pm_solve_opts {
  * above 8,192 rows (IC0 16,384) holds every SM until it ends, so that solves and other kernels on other streams wait for
  * it, where STREAM's kernels interleave with them. One solve at a time is faster resident up to the AUTO
  * limits, and so are two of less than a million rows; a program that solves from four or more threads at once, or that needs the GPU for other work meanwhile, gets
- * more from STREAM (eight threads, FP64 line, 0.12M rows each: 13 us per system and iteration against 25; measured figures
+ * more from STREAM (eight threads, FP64 line, 0.12M rows each: 13 us per system and iteration against 24; measured figures
  * in csrc/pm_resident.cuh). */
 enum { PM_KERNEL_AUTO = 0, PM_KERNEL_STREAM = 1, PM_KERNEL_RESIDENT = 2 };
 

@@ -37,9 +37,9 @@
 //
 // A grid team holds every SM to the end of its solve (512 threads of 128 registers fill the register file): solves on
 // other streams queue behind it, where the stream's kernels interleave. Several solves at once, one operator
-// and host thread each, us per system and iteration, 1 / 2 / 4 / 8 threads: FP64 line, 0.12M rows, resident 25 / 25 / 25 /
-// 25, stream 51 / 30 / 20 / 13; FP64 IC0 41 / 41 / 41 / 41 and 77 / 43 / 29 / 21; FP64 IC0 2.0M 272 whatever the number and 285 /
-// 213 / 188 / 194. One cluster's or one block's solves do run side by side (2,048 rows, IC0: 7.3 / 3.8 / 1.9 / 1.2).
+// and host thread each, us per system and iteration, 1 / 2 / 4 / 8 threads: FP64 line, 0.12M rows, resident 24 whatever
+// the number, stream 53 / 30 / 19 / 13; FP32 line 19 and 37 / 19 / 11 / 7; FP64 IC0 40 and 76 / 43 / 29 / 21, 2.0M rows 272 and
+// 284 / 212 / 188 / 194. Solves by one cluster or one block run side by side (2,048 rows, IC0: 7.0 / 3.6 / 1.8 / 1.2).
 #pragma once
 
 #include <cuda_bf16.h>
