@@ -122,7 +122,13 @@ constexpr uint32_t SPIN_LIMIT = 1u << 22;  // polls of about half a microsecond:
 // acquire covers the block's later loads, so no other thread fences; the waiting thread polls without a sleep.
 // (With a fence in every thread, a 100 ns sleep between polls and a last look at the error word, a
 // 24-system batch of 4.5M rows took 188.6 ms, 185.2 without.)
-__device__ bool grid_barrier(Ctl* ctl) {
+//
+// quiet (IC0, more than one block per SM): relaxed polls with a short sleep, and one fence after the last. Every acquiring
+// poll drops the SM's L1, under the feet of the other blocks of the SM that may still work: IC0 phases read their factor rows and neighbour
+// tables through L1 (ld.global.nc). 48 velocity and pressure systems, IC0, 70 iterations: 62.8 ms FP64, 53.9 FP32 with acquiring
+// polls, 53.1 and 43.0 quiet; a server with one mass system of 2,048 rows 4.9 -> 3.6 ms. Where the phases reuse
+// little (no IC0) or the block has its SM to itself, the fence costs more than the polls (1 to 4 % of an iteration).
+__device__ bool grid_barrier(Ctl* ctl, bool quiet) {
   __shared__ int ok_s;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -136,15 +142,18 @@ __device__ bool grid_barrier(Ctl* ctl) {
     } else {
       uint32_t spins = 0;
       for (;;) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&ctl->bar_gen) : "memory");
+        if (quiet) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&ctl->bar_gen) : "memory");
+        else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&ctl->bar_gen) : "memory");
         if (g != g0) break;
         ++spins;
+        if (quiet) __nanosleep(32);
         if (spins > SPIN_LIMIT || ((spins & 1023u) == 0 && *((volatile int32_t*)&ctl->err) != 0)) {
           atomicExch(&ctl->err, PM_TIMEOUT);
           ok = 0;
           break;
         }
       }
+      if (quiet) asm volatile("fence.acq_rel.gpu;" ::: "memory");
     }
     ok_s = ok;
   }
@@ -484,7 +493,7 @@ __device__ __forceinline__ bool owns_ic0_chunk(const Sys& S, int c) {
         },                                                                                          \
         slist, wsum);                                                                               \
     for (int a_ = 0; a_ < na_; ++a_) ic0_phase<T>(sys[slist[a_]], ph_);                             \
-    if (!grid_barrier(ctl)) return;                                                                 \
+    if (!grid_barrier(ctl, quiet)) return;                                                          \
   }
 
 // MINB: resident blocks of 256 threads per SM that the register budget is sized for. 3 (80 registers, about
@@ -495,6 +504,8 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
                                                int ntiles, double* part, Ctl* ctl,
                                                int quantum, int init, int ic0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  // a constant for MINB = 2, which no IC0 launch takes: tested at run time, it cost FP32 batches 3 to 7 %
+  const bool quiet = MINB > 2 && ic0 > 1;
   int* slist = reinterpret_cast<int*>(smem_raw);                             // nsys entries
   T* smt = reinterpret_cast<T*>(smem_raw + ((size_t)nsys * 4 + 15) / 16 * 16);  // tile of columns
   __shared__ double red[NP * 32];
@@ -515,14 +526,14 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
       block_sum<1>(v, red);
       if (tid == 0) part[t] = v[0];
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     for (int s = blockIdx.x; s < nsys; s += gridDim.x) {
       const Sys& S = sys[s];
       if (scal[s].state != ST_NEW) continue;
       const double sb = sys_reduce(part, ntiles, 0, S.tile0, S.ntiles, red);
       if (tid == 0) scal[s].proj_c = S.proj ? sb / S.one_m : 0.0;  // lambda, reused below
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     // I2: b' = b - lambda m; x = 0; r = b'; z = P^{-1} r (Jacobi / line) and partials
     FOR_OWNED_TILES(3, t, tl) {
       const Sys& S = sys[tl.sys];
@@ -564,7 +575,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
         for (int l = 0; l < NP; ++l) part[(int64_t)l * ntiles + t] = v[l];
       __syncthreads();
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     if (ic0) {
       IC0_PHASES(3)
       FOR_OWNED_TILES(3, t, tl) {   // partials of the IC0 systems: (b', b'), (r, z), m'z, 1'r
@@ -588,7 +599,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
           for (int l = 0; l < NP; ++l) part[(int64_t)l * ntiles + t] = v[l];
         __syncthreads();
       }
-      if (!grid_barrier(ctl)) return;
+      if (!grid_barrier(ctl, quiet)) return;
     }
     for (int s = blockIdx.x; s < nsys; s += gridDim.x) {
       const Sys& S = sys[s];
@@ -613,7 +624,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
         c.prev_true = -1.0;
       }
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     // p = z - c
     FOR_OWNED_TILES(4, t, tl) {
       const Sys& S = sys[tl.sys];
@@ -621,11 +632,11 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
       const T c = (T)scal[tl.sys].proj_c;
       for (int i = tid; i < rows; i += blockDim.x) ((T*)S.p)[row0 + i] = ldcg(((const T*)S.z) + row0 + i) - c;
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     for (int s = blockIdx.x; s < nsys; s += gridDim.x)
       if (tid == 0 && scal[s].state == ST_PINIT) scal[s].state = ST_ITER;
     if (blockIdx.x == 0 && tid == 0) ctl->pending = 0;
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
   }
 
   for (int it = 0; it < quantum; ++it) {
@@ -666,7 +677,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
         part[(int64_t)ntiles + t] = v[1];
       }
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     // ---- Ar ------------------------------------------------------------------------------------------
     for (int s = blockIdx.x; s < nsys; s += gridDim.x) {
       const Sys& S = sys[s];
@@ -704,7 +715,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
         }
       }
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     // ---- B: update + preconditioner + dots | RESTART: preconditioner + dots ---------------------------
     FOR_OWNED_TILES(1, t, tl) {
       const Sys& S = sys[tl.sys];
@@ -803,7 +814,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
         for (int l = 0; l < NP; ++l) part[(int64_t)l * ntiles + t] = v[l];
       __syncthreads();
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     if (ic0) {
       IC0_PHASES(1)
       FOR_OWNED_TILES(1, t, tl) {   // (r, z), m'z, 1'r of IC0 systems' ITER / RESTART tiles into lanes 1..3
@@ -832,7 +843,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
           for (int l = 1; l < NP; ++l) part[(int64_t)l * ntiles + t] = v[l];
         __syncthreads();
       }
-      if (!grid_barrier(ctl)) return;
+      if (!grid_barrier(ctl, quiet)) return;
     }
     // ---- Br ------------------------------------------------------------------------------------------
     for (int s = blockIdx.x; s < nsys; s += gridDim.x) {
@@ -877,7 +888,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
         }
       }
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     // ---- C: p = (z - c) + beta p | SHIFT2: x -= shift; count systems still active -----------------------
     if (blockIdx.x == 0) {
       int act = 0;
@@ -913,7 +924,7 @@ __global__ void __launch_bounds__(256, MINB) k_batch(const Sys* __restrict__ sys
           if (i0 + u * bd < rows) p[row0 + i0 + u * bd] = (zv[u] - c) + beta * pv[u];
       }
     }
-    if (!grid_barrier(ctl)) return;
+    if (!grid_barrier(ctl, quiet)) return;
     // SHIFT2 -> DONE; no phase before the next C reads SHIFT2 or DONE as active, so no barrier
     for (int s = blockIdx.x; s < nsys; s += gridDim.x)
       if (tid == 0 && scal[s].state == ST_SHIFT2) scal[s].state = ST_DONE;
@@ -937,6 +948,7 @@ struct pm_batch {
   bool any_ic0 = false;            // the kernel runs the IC0 colour phases
   int tile_cols = 32, block = 256;
   int grid[2] = {0, 0};            // blocks of the kernel with three, with two blocks per SM
+  int sms = 0;
   int nz_max = 0;
   int64_t ntiles = 0;
   std::vector<pm::batch::Sys> hsys;
@@ -1163,7 +1175,7 @@ bool few_tiles(const pm_batch* bt, const Scal* scal) {
 
 cudaError_t launch(pm_batch* bt, bool few, int quantum, int init, cudaStream_t s) {
   return launch_k(kernel_of(bt->precision, few), bt->grid[few], bt->block, smem_bytes(bt), bt->d_sys, bt->d_scal, (int)bt->count,
-                     (int)bt->ntiles, bt->d_part, bt->d_ctl, quantum, init, bt->any_ic0 ? 1 : 0, s);
+                     (int)bt->ntiles, bt->d_part, bt->d_ctl, quantum, init, bt->any_ic0 ? (bt->grid[few] > bt->sms ? 2 : 1) : 0, s);
 }
 
 // Capture one launch (made by `fn` on the capture stream) into an executable graph.
@@ -1193,6 +1205,7 @@ int set_grid(pm_batch* bt) {
   const size_t smem = smem_bytes(bt);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device);
+  bt->sms = sms;
   for (int few = 0; few < 2; ++few) {
     const int per_sm = max_blocks(kernel_of(bt->precision, few), bt->block, smem);
     if (per_sm <= 0) return set_error(PM_EINVAL, "batched kernel cannot be resident with this block / tile shape");
@@ -1711,7 +1724,7 @@ extern "C" int pm_server_run(pm_server* sv, int32_t quantum, int32_t* active, pm
                                     cudaMemcpyHostToDevice, s), "ctl");
     if (st) return st;
   }
-  const int ic0 = sv->n_ic0 > 0 ? 1 : 0;
+  const int ic0 = sv->n_ic0 > 0 ? 2 : 0;   // several blocks per SM
   if (!sv->graph || sv->graph_quantum != quantum || sv->graph_tcap != sv->tcap || sv->graph_ic0 != ic0) {
     const size_t smem = server_smem(sv);
     st = capture_graph(&sv->graph, [&](cudaStream_t cs) {
@@ -1795,7 +1808,7 @@ extern "C" void pm_server_destroy(pm_server* sv) {
 // Test aid: block 1 leaves without arriving at the barrier, so block 0's bounded wait expires.
 __global__ void k_barrier_probe(pm::batch::Ctl* ctl) {
   if (blockIdx.x != 0) return;
-  pm::batch::grid_barrier(ctl);
+  pm::batch::grid_barrier(ctl, false);
 }
 
 extern "C" int pm_debug_barrier_timeout(pm_stream stream) {
