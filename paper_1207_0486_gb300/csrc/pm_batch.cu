@@ -1143,10 +1143,19 @@ cudaError_t launch_k(Kernel k, int grid, int block, size_t smem, const Sys* d_sy
 //   FP32 line, all 468 (2/2) 198 / 160, 836 (2/3) 229 / 217, 1200 (3/4) 287 / 293, 1257 (3/5) 339 / 366, 1407 (4/5)
 //   407 / 393, 1876 (5/7) 510 / 537; pressure alone 145 (1/2) 89 / 91, 300 (2/2) 189 / 133, 593 (3/4) 326 / 239,
 //   842 (3/5) 331 / 302; BF16 1407 (4/5) 388 / 375; Jacobi FP32 1395 (4/5) 388 / 351, BF16 377 / 333.
+// Velocity and pressure systems of boxes, ms for 100 iterations: FP32 line 1252 (3/5) 29.4 / 36.2, 1440 (4/5) 30.3 / 29.0,
+// 1663 (4/6) 40.9 / 44.7, 2070 (5/7) 38.8 / 39.6, 2340 (6/8) 44.0 / 44.3; FP64 line 1440 49.1 / 46.5, 1404 (4/5) 55.6 / 57.2.
+// Mass systems alone, whose tiles gain most from the wider budget (0.69 of three blocks' time with two in FP64, 0.6 in FP32
+// and BF16), go by the busiest block's time: ms for 70 iterations,
+//   FP64 Jacobi 939 tiles (3/4) 25.7 / 23.4, 1252 (3/5) 26.8 / 28.9, 2072 (5/7) 44.3 / 41.5, 5000 (11/17) 93.4 / 93.4; line 2072
+//   47.8 / 45.2, 3600 (8/12) 65.2 / 69.8;
+//   FP32 Jacobi 432 (1/2) 7.4 / 8.4, 939 22.8 / 17.9, 1878 (5/7) 37.3 / 30.9, 5000 87.5 / 75.2, 8595 (19/29) 137.6 / 119.5; line
+//   2072 42.3 / 35.0, 8595 149.6 / 134.6; BF16 Jacobi 1252 21.5 / 21.0, 5000 86.1 / 74.1.
 // IC0 phases keep three: FP64 754 / 979 at 465 tiles, 1307 / 1567 at 930, 438 / 415 at 90.
 bool few_tiles(const pm_batch* bt, const Scal* scal) {
   if (bt->any_ic0) return false;
   int64_t tiles = 0;
+  bool mass = true;
   int busiest[2];
   for (int few = 0; few < 2; ++few) {
     std::vector<int> d((size_t)bt->grid[few] + 1, 0);   // differences of the blocks' tile counts
@@ -1156,6 +1165,7 @@ bool few_tiles(const pm_batch* bt, const Scal* scal) {
       if (scal && scal[i].state == ST_DONE) continue;
       const int g = bt->grid[few], nt = bt->hsys[i].ntiles, a = bt->hsys[i].tile0 % g, e = a + nt % g;
       tiles += nt;
+      mass = mass && bt->which[i] == PM_OP_MASS;
       whole += nt / g;
       ++d[a];
       --d[std::min(e, g)];
@@ -1167,6 +1177,10 @@ bool few_tiles(const pm_batch* bt, const Scal* scal) {
     int most = 0, at = 0;
     for (int b = 0; b < bt->grid[few]; ++b) most = std::max(most, at += d[b]);
     busiest[few] = whole + most;
+  }
+  if (mass) {
+    const double tile = bt->precision == PM_FP64 ? 0.69 : 0.6;   // a tile's time with two blocks over that with three
+    return tile * busiest[1] <= busiest[0];
   }
   return busiest[1] <= busiest[0] ||
          (busiest[0] > 1 && busiest[1] == busiest[0] + 1 &&
@@ -1238,9 +1252,10 @@ int run_to_completion(pm_batch* bt, cudaStream_t s, int quantum) {
   Ctl h;
   std::vector<Scal> hs(bt->count);
   bool few = few_tiles(bt, nullptr);
+  const bool settled = bt->any_ic0 || bt->ntiles <= bt->grid[1];   // three blocks; two, with a tile at most for each
   const int64_t max_quanta = (int64_t)bt->max_iter / quantum + 70;
   for (int64_t q = 0; q < max_quanta; ++q) {
-    if (q > 0) few = few_tiles(bt, hs.data());
+    if (q > 0 && !settled) few = few_tiles(bt, hs.data());
     if (!bt->graph[few] || bt->graph_quantum[few] != quantum) {
       const int st = capture_graph(&bt->graph[few], [&](cudaStream_t cs) {
         return launch(bt, few, quantum, 0, cs);
@@ -1252,7 +1267,7 @@ int run_to_completion(pm_batch* bt, cudaStream_t s, int quantum) {
     if (st) return st;
     count_launch();
     st = cuda_check(cudaMemcpyAsync(&h, bt->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s), "ctl");
-    if (!st && !bt->any_ic0)
+    if (!st && !settled)
       st = cuda_check(cudaMemcpyAsync(hs.data(), bt->d_scal, bt->count * sizeof(Scal), cudaMemcpyDeviceToHost, s), "scal");
     if (!st) st = cuda_check(cudaStreamSynchronize(s), "batched PCG");
     if (st) return st;

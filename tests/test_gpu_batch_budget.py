@@ -39,6 +39,20 @@ def test_budget_follows_the_tiles(ops, precision, systems, per_sm):
         assert i["grid"] == per_sm * sms, i
 
 
+@pytest.mark.parametrize("precision,systems,per_sm", [
+    (pm.FP64, 5, 3), (pm.FP64, 12, 2), (pm.FP64, 24, 2),                          # 319, 938, 1,876 tiles
+    (pm.FP32_REFINE, 5, 3), (pm.FP32_REFINE, 24, 2), (pm.BF16_REFINE, 60, 2)])    # 319, 1,876, 4,690 tiles
+def test_budget_of_mass_systems(ops, precision, systems, per_sm):
+    """Mass systems alone gain more from two blocks per SM: a batch takes them wherever the busiest block ends sooner."""
+    bt = pm.Batch([ops[i % 6] for i in range(systems)], [pm.OP_MASS] * systems,
+                  pm.Options(rtol=1e-8, prec=pm.PREC_LINE, precision=precision, inner_rtol=1e-4))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    i = bt.info()
+    bt.close()
+    if sms == 152:
+        assert i["grid"] == (per_sm * sms if per_sm == 2 else min(per_sm * sms, i["tiles"])), i
+
+
 @pytest.mark.parametrize("precision", [pm.FP64, pm.FP32_REFINE, pm.BF16_REFINE])
 def test_solutions_do_not_depend_on_the_budget(ops, precision):
     """Twenty-four systems that end at very different iterations, so that the launches pass from three blocks per SM to
